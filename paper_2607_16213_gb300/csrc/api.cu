@@ -3,13 +3,11 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
-#include <mutex>
 
 #include "selkv_internal.cuh"
 
 namespace selkv {
 cudaError_t launch_setup(const CompressArgs& a, const SeqTable& tab, const SelectWs& w, cudaStream_t s);
-cudaError_t launch_vnorm(const CompressArgs& a, cudaStream_t s);
 cudaError_t launch_merge(const CompressArgs& a, cudaStream_t s);
 
 namespace {
@@ -32,35 +30,6 @@ bool shape_ok(const selkv_shape* s) {
 }
 
 size_t round256(size_t x) { return (x + 255) & ~size_t(255); }
-
-// A side stream per device: the value-norm pass (HBM-bound) runs on it next to the scoring
-// passes (bound by the exponentials), forked from and joined back to the caller's stream with
-// events, a pattern that also records into a CUDA graph.  Created on first use outside a
-// capture; if it cannot be had, the pass runs on the caller's stream.
-struct SideStream {
-  cudaStream_t s = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr;
-  bool ready = false, failed = false;
-};
-constexpr int kMaxDevices = 64;
-std::mutex g_side_mu;
-SideStream g_side[kMaxDevices];
-
-// Requires g_side_mu.
-SideStream* side_stream(cudaStream_t caller) {
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
-  SideStream& x = g_side[dev];
-  if (!x.ready && !x.failed) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(caller, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return nullptr;
-    x.ready = cudaStreamCreateWithFlags(&x.s, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreateWithFlags(&x.fork, cudaEventDisableTiming) == cudaSuccess &&
-              cudaEventCreateWithFlags(&x.join, cudaEventDisableTiming) == cudaSuccess;
-    x.failed = !x.ready;
-  }
-  return x.ready ? &x : nullptr;
-}
 
 // Key slices of the scoring's first pass (one row-statistics partial per slice and row).
 int score_chunks(const selkv_shape& s, int R) {
@@ -172,15 +141,15 @@ T* at(void* ws, size_t off) {
 
 void note_launches(int kernels) { g_launches += (uint64_t)kernels; }
 
-// Kernels one selkv_compress call enqueues, mirroring the launch code: set-up and value norms;
-// the scoring's two passes and the fold of the row statistics between them; the selection
+// Kernels one selkv_compress call enqueues, mirroring the launch code: set-up; the scoring's two
+// passes and the fold of the row statistics between them; the selection
 // (pooling with digit pass 0 and digit passes 1-2 of each KV head's top-k, then, in the
 // shared mode only, the union with the trim's pass 0 and its passes 1-2; finally the
 // compaction's count and write); the RoPE tables when repositioning;
 // the routing and merge (bucket: route and merge, plus the kept-row copy unless the merge
 // does it; cosine: the copy and the cosine kernels); the bias.
 int compress_kernel_count(const CompressArgs& a) {
-  int k = 2 + 3;
+  int k = 1 + 3;
   k += a.per_head ? 5 : 8;
   if (a.rope != SELKV_ROPE_OFF) k += 1;
   if (a.routing == SELKV_ROUTE_COSINE)
@@ -367,19 +336,8 @@ selkv_status selkv_compress(const selkv_shape* shape, const int32_t* n_len, doub
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const SelectWs sw = carve_select_ws(at<char>(workspace, plan.select), s.batch, s.num_kv_heads, s.n_cap);
   cudaError_t e = launch_setup(a, tab, sw, st);
-  {
-    // value norms on the side stream (they need seq_n from the set-up; selection needs them)
-    std::lock_guard<std::mutex> lock(g_side_mu);
-    SideStream* side = e == cudaSuccess ? side_stream(st) : nullptr;
-    if (side != nullptr) {
-      e = cudaEventRecord(side->fork, st);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(side->s, side->fork, 0);
-      if (e == cudaSuccess) e = launch_vnorm(a, side->s);
-      if (e == cudaSuccess) e = cudaEventRecord(side->join, side->s);
-    }
-    if (e == cudaSuccess) e = score_uses_tc(a.dtype, a.D, a.R) ? launch_score_tc(a, st) : launch_score_simt(a, st);
-    if (e == cudaSuccess) e = side != nullptr ? cudaStreamWaitEvent(st, side->join, 0) : launch_vnorm(a, st);
-  }
+  // the scoring also takes the value norms
+  if (e == cudaSuccess) e = score_uses_tc(a.dtype, a.D, a.R) ? launch_score_tc(a, st) : launch_score_simt(a, st);
   if (e == cudaSuccess)
     e = launch_select_grid(a, sw, st);
   if (e == cudaSuccess) e = launch_merge(a, st);

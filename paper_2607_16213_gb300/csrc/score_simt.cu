@@ -9,6 +9,8 @@
 // twice: pass 1 gathers per-row (max, sum) over column chunks, a small kernel folds the
 // chunks, and pass 2 recomputes the same tiles and sums columns.  Both passes use the same
 // tile code, so pass 2 sees bit-identical scores.
+#include <algorithm>
+
 #include "selkv_internal.cuh"
 
 namespace selkv {
@@ -132,9 +134,8 @@ __global__ __launch_bounds__(256) void rowstats_kernel(CompressArgs a) {
   }
 }
 
-// Fold the column chunks: (M, 1 / (G * Z)) per row.
-__global__ void rowstat_reduce_kernel(CompressArgs a) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+// Fold of the column chunks of row idx: (M, 1 / (G * Z)).
+__device__ __forceinline__ void fold_row(const CompressArgs& a, int idx) {
   if (idx >= a.B * a.Hkv * a.R) return;
   const int r = idx % a.R, bk = idx / a.R;
   const int nch = a.nchunks;  // chunks without visible columns hold (-inf, 0)
@@ -147,6 +148,49 @@ __global__ void rowstat_reduce_kernel(CompressArgs a) {
     if (p.x != -INFINITY) Z += p.y * exp2f(p.x - M);
   }
   a.rowstat[idx] = make_float2(M, 1.f / ((float)a.G * Z));
+}
+
+__global__ void rowstat_reduce_kernel(CompressArgs a) { fold_row(a, blockIdx.x * blockDim.x + threadIdx.x); }
+
+// The fold in the first `fold_blocks` CTAs and ||v_j|| of Eq. 1 in the others: two kernels' work
+// that does not depend on one another in one launch.  D / 8 lanes per row (at most 16), each
+// loading 8 elements at a time.
+template <typename T, int D>
+__global__ __launch_bounds__(256) void fold_norm_kernel(CompressArgs a, int fold_blocks) {
+  if ((int)blockIdx.x < fold_blocks) {
+    fold_row(a, blockIdx.x * blockDim.x + threadIdx.x);
+    return;
+  }
+  constexpr int EPL = 8;                            // elements per load8
+  constexpr int LPR = D / EPL < 16 ? D / EPL : 16;  // lanes per row
+  constexpr int RPW = 32 / LPR;                     // rows per warp step
+  const int lane = threadIdx.x & 31, sub = lane / LPR, sl = lane % LPR;
+  const size_t total = (size_t)a.B * a.Hkv * a.n_cap;
+  const size_t nwarps = (size_t)(gridDim.x - fold_blocks) * (blockDim.x / 32);
+  const size_t warp = ((blockIdx.x - fold_blocks) * (size_t)blockDim.x + threadIdx.x) / 32;
+  for (size_t row0 = warp * RPW; row0 < total; row0 += nwarps * RPW) {
+    const size_t row = row0 + sub;
+    float s = 0.f;
+    bool ok = false;
+    if (row < total) {
+      const int j = (int)(row % a.n_cap);
+      const int b = (int)(row / a.n_cap) / a.Hkv;
+      ok = j < a.seq_n[b];
+      if (ok) {
+        const T* p = static_cast<const T*>(a.V) + row * D;
+#pragma unroll
+        for (int d = sl * EPL; d < D; d += LPR * EPL) {
+          float x[8];
+          load8(p + d, x);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) s = fmaf(x[e], x[e], s);
+        }
+      }
+    }
+#pragma unroll
+    for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (ok && sl == 0) a.vnorm[row] = sqrtf(s);
+  }
 }
 
 // Pass 2: grid (column tile, b * Hkv); a_j = sum_r 2^(s'_rj - M_r) / (G Z_r).
@@ -194,7 +238,13 @@ cudaError_t launch_score_t(const CompressArgs& a, cudaStream_t s, int passes) {
   const int row_tiles = (a.R + kTile - 1) / kTile;
   if (passes & kScoreRowstats) {
     rowstats_kernel<T, D><<<dim3(a.nchunks, row_tiles, a.B * a.Hkv), 256, 0, s>>>(a);
-    launch_rowstat_reduce(a, s);
+    if (a.V == nullptr) {
+      launch_rowstat_reduce(a, s);
+    } else {
+      const size_t rows = (size_t)a.B * a.Hkv * a.n_cap;
+      const int fold = (a.B * a.Hkv * a.R + 255) / 256, norm = (int)std::min<size_t>((rows + 15) / 16, 152 * 8);
+      fold_norm_kernel<T, D><<<fold + norm, 256, 0, s>>>(a, fold);
+    }
   }
   if (passes & kScoreColsums)
     colsum_kernel<T, D><<<dim3((a.n_cap + kTile - 1) / kTile, a.B * a.Hkv), 256, 0, s>>>(a);

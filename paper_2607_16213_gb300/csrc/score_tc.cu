@@ -42,9 +42,99 @@ constexpr uint32_t kTmemCols = 512;  // two accumulators of up to 256 fp32 colum
 // A TMA producer warp and an MMA warp follow them.
 constexpr int kP1Parts = SELKV_P1_KEYS / (32 * SELKV_P1_CPW);
 static_assert(kP1Parts * 32 * SELKV_P1_CPW == SELKV_P1_KEYS && kP1Parts >= 1, "pass-1 tile split");
-static_assert(4 * kP1Parts + 2 <= 32 && SELKV_P1_KEYS <= 256, "pass-1 warps per CTA");
+// Both passes also carry the value norms of Eq. 1 (selkv_compress only) in a few more warps, half
+// of the rows each.  A kernel of its own for them, whether before the passes or beside them on
+// another stream, took all SMs first and cost its whole time (58 us for one layer of 8 x 100k
+// rows); the passes, bound by their epilogues at 60% of HBM, have room for its bytes: with them
+// 50 + 51 us become 62 + 56 us.  All rows in pass 1 make it wait for HBM (73 + 51 us).  Pass 2
+// has shared memory for three warps of two copies in flight, which bounds its share (three
+// quarters of the rows there: 57 + 72 us with two warps).
+__host__ __device__ constexpr int norm_warps(int pass) { return pass == 1 ? 4 : 3; }
+__host__ __device__ constexpr int norm_stages(int pass) { return pass == 1 ? 3 : 2; }
+static_assert(4 * kP1Parts + 2 + norm_warps(1) <= 32 && SELKV_P1_KEYS <= 256, "pass-1 warps per CTA");
 __host__ __device__ constexpr int epi_warps(int pass) { return pass == 1 ? 4 * kP1Parts : 16; }
-__host__ __device__ constexpr int cta_threads(int pass) { return (epi_warps(pass) + 2) * 32; }
+__host__ __device__ constexpr int cta_threads(int pass, bool norms) {
+  return (epi_warps(pass) + 2 + (norms ? norm_warps(pass) : 0)) * 32;
+}
+
+// Value norms of rows [row_lo, row_hi) by warp `w` of norm_warps(PASS).  The rows of a (sequence,
+// KV head) are contiguous, so lane 0 streams them as 4 KB bulk copies into the warp's own ring
+// (bytes in flight cost no registers; with 4 KB in registers per warp the round trips of eight
+// warps made pass 1 277 us for 64 x 8k where this takes 235).  D / 8 lanes take a row, 16 bytes a
+// lane: a lane squares its 8 elements in order and the lanes of a row meet in a butterfly; the
+// sums of a chunk's 8 row groups share it (each level keeps half of the values), pairing the
+// lanes as a butterfly per value does.  The copies are marked for early eviction from L2.
+constexpr int kNormChunk = 4096;  // bytes per copy
+__host__ __device__ constexpr int norm_ring(int pass) { return norm_warps(pass) * norm_stages(pass) * kNormChunk; }
+template <int D, int PASS>
+__device__ __forceinline__ void norm_rows(const __nv_bfloat16* V, float* norm, int row_lo, int row_hi, int w,
+                                          unsigned char* ring, uint64_t* bars, uint32_t* flags) {
+  constexpr int LPR = D / 8, RPL = 32 / LPR, kGroups = kNormChunk / 512;  // lanes per row, rows per group of lanes
+  constexpr int kNormStages = norm_stages(PASS), nw = norm_warps(PASS);
+  constexpr int kRows = RPL * kGroups;                     // rows per chunk
+  static_assert(kRows * D * 2 == kNormChunk, "a chunk is whole rows");
+  const int lane = threadIdx.x & 31, sub = lane / LPR;
+  ring += w * kNormStages * kNormChunk;
+  bars += w * kNormStages;
+  const int first = row_lo + w * kRows, stride = nw * kRows;
+  const int chunks = first < row_hi ? (row_hi - first + stride - 1) / stride : 0;
+  const uint64_t pol = l2_evict_first_policy();
+  auto load = [&](int c) {
+    const int r0 = first + c * stride, st = c % kNormStages;
+    const uint32_t bytes = (uint32_t)min(kRows, row_hi - r0) * D * 2;
+    mbar_arrive_expect_tx(&bars[st], bytes);
+    bulk_load_hint(ring + st * kNormChunk, V + (size_t)r0 * D, bytes, &bars[st], pol);
+  };
+  if (lane == 0)
+    for (int c = 0; c < min(chunks, kNormStages); ++c) load(c);
+  for (int c = 0; c < chunks; ++c) {
+    const int st = c % kNormStages, r0 = first + c * stride;
+    if (!__all_sync(0xffffffffu, mbar_wait(&bars[st], (c / kNormStages) & 1))) {
+      if (lane == 0) {
+        raise_flag(flags, SELKV_DEVERR_TIMEOUT);
+        for (int k = c; k < min(chunks, c + kNormStages); ++k)  // (bounded) let the copies in flight land
+          mbar_wait(&bars[k % kNormStages], (k / kNormStages) & 1);
+      }
+      return;
+    }
+    const uint4* src = reinterpret_cast<const uint4*>(ring + st * kNormChunk) + lane;
+    float q[kGroups];
+#pragma unroll
+    for (int k = 0; k < kGroups; ++k) {
+      const uint4 u = src[k * 32];
+      const uint32_t x[4] = {u.x, u.y, u.z, u.w};
+      float s = 0.f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float lo = bf16_lo(x[e]), hi = bf16_hi(x[e]);
+        s = fmaf(lo, lo, s);
+        s = fmaf(hi, hi, s);
+      }
+      q[k] = s;
+    }
+    __syncwarp();
+    if (lane == 0 && c + kNormStages < chunks) load(c + kNormStages);
+    int k0 = 0;  // first group whose sum this lane still holds; `keep` of them follow
+#pragma unroll
+    for (int o = LPR / 2, keep = kGroups; o > 0; o >>= 1) {
+      const bool up = lane & o;
+      if (keep > 1) {
+        keep >>= 1;
+#pragma unroll
+        for (int i = 0; i < keep; ++i) {
+          const float mine = up ? q[keep + i] : q[i], other = up ? q[i] : q[keep + i];
+          q[i] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+        }
+        k0 += up ? keep : 0;
+      } else {
+        q[0] += __shfl_xor_sync(0xffffffffu, q[0], o);
+      }
+    }
+    // LPR lanes hold kGroups sums: the lowest of the lanes that share one writes it
+    const int row = r0 + k0 * RPL + sub;
+    if ((lane % (LPR / kGroups)) == 0 && row < row_hi) norm[row] = sqrtf(q[0]);
+  }
+}
 
 #ifndef SELKV_P2_PIPE
 #define SELKV_P2_PIPE 1   // pass 2: pipelined 16-column TMEM loads on full, unmasked tiles
@@ -101,12 +191,14 @@ struct SCfg {
   static constexpr int kQBytes = kRows * D * 2;
   static constexpr int kRing = kStages * kKTile;
   // barriers | -(M + log2(G Z)) of up to 512 rows | pass 1: [parts][128] float2, pass 2: [2][4][128] float
-  static constexpr int kMisc = 256 + 256 * 8 + (kP1Parts * 128 * 8 > 4096 ? kP1Parts * 128 * 8 : 4096);
-  static constexpr int kSmem = 1024 + kQBytes + kRing + kMisc;
+  static constexpr int kHead = 384;  // barriers and flags
+  static constexpr int kMisc = kHead + 256 * 8 + (kP1Parts * 128 * 8 > 4096 ? kP1Parts * 128 * 8 : 4096);
+  static constexpr int kSmem = 1024 + kQBytes + kRing + kMisc + norm_ring(PASS);
+  static_assert(kSmem <= 232448, "227 KB of shared memory");
 };
 
 template <int D, int PASS, int HALVES>
-__global__ __launch_bounds__(cta_threads(PASS), 1) void score_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
+__global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
                                                                         const __grid_constant__ CUtensorMap tmK,
                                                                         CompressArgs a) {
   using C = SCfg<D, PASS, HALVES>;
@@ -131,8 +223,13 @@ __global__ __launch_bounds__(cta_threads(PASS), 1) void score_tc_kernel(const __
   // "part 0 has read them"
   uint64_t* cs_full = reinterpret_cast<uint64_t*>(misc + 128);  // [4][2]
   uint64_t* cs_empty = cs_full + 8;                              // [4][2]
-  float* rneg = reinterpret_cast<float*>(misc + 256);               // pass 2: -(M + log2(G Z)) per row
-  float* colpart = reinterpret_cast<float*>(misc + 256 + 256 * 8);  // pass 1: [parts][128] float2; pass 2: [2][4][128]
+  // the norm warps' copies, and their ring
+  constexpr int kNormBars = norm_warps(PASS) * norm_stages(PASS);
+  static_assert(kNormBars <= 16, "norm barriers fit");
+  uint64_t* nbar = reinterpret_cast<uint64_t*>(misc + 256);
+  unsigned char* nring = misc + C::kMisc;
+  float* rneg = reinterpret_cast<float*>(misc + C::kHead);               // pass 2: -(M + log2(G Z)) per row
+  float* colpart = reinterpret_cast<float*>(misc + C::kHead + 256 * 8);  // pass 1: [parts][128] float2; pass 2: [2][4][128]
 
   const int kv = blockIdx.y, b = blockIdx.z;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -163,9 +260,12 @@ __global__ __launch_bounds__(cta_threads(PASS), 1) void score_tc_kernel(const __
     }
     mbar_init(qbar, 1);
     mbar_init(done, 1);
-    for (int i = 0; i < 8; ++i) {
-      mbar_init(&cs_full[i], 3 * 32);
-      mbar_init(&cs_empty[i], 32);
+    for (int i = 0; i < kNormBars; ++i) mbar_init(&nbar[i], 1);
+    if (PASS == 2) {
+      for (int i = 0; i < 8; ++i) {
+        mbar_init(&cs_full[i], 3 * 32);
+        mbar_init(&cs_empty[i], 32);
+      }
     }
     *abort_flag = 0;
     fence_mbar_init();
@@ -247,6 +347,14 @@ __global__ __launch_bounds__(cta_threads(PASS), 1) void score_tc_kernel(const __
       umma_commit(done);  // every MMA issued above has completed once this arrives
       mbar_wait(done, 0);
     }
+  } else if (warp > kMmaWarp) {
+    // ---------------- value norms: this CTA's share of the pass's rows ----------------
+    const int n1 = n / 2;
+    const int lo = PASS == 1 ? 0 : n1, hi = PASS == 1 ? n1 : n;
+    const int share = ((hi - lo + (int)gridDim.x - 1) / (int)gridDim.x + 15) & ~15;
+    const int r_lo = lo + (int)blockIdx.x * share;
+    norm_rows<D, PASS>(static_cast<const __nv_bfloat16*>(a.V) + bk * a.n_cap * D, a.vnorm + bk * a.n_cap, r_lo,
+                 min(hi, r_lo + share), warp - kMmaWarp - 1, nring, nbar, a.flags);
   } else {
     // ---------------- epilogue: warps 0-15 ----------------
     const int q = warp & 3, part = warp >> 2;  // lane quarter of TMEM, and which part of the work
@@ -344,10 +452,11 @@ __global__ __launch_bounds__(cta_threads(PASS), 1) void score_tc_kernel(const __
       const int klane = q * 32 + lane;   // key owned by this thread within the tile
       int u = 0;                         // accumulator use, as counted by the MMA thread
       for (int t = 0; t < nt; ++t) {
-        const int j = (t_begin + t) * kKeys + klane;
+        const int key0 = (t_begin + t) * kKeys;
+        const int j = key0 + klane;
         const int jrel = j - (n - a.W);  // > 0: only rows with (r mod W) >= jrel see key j
         // every key of this warp is seen by every row: the whole tile is unmasked
-        const bool unmasked = (t_begin + t) * kKeys + q * 32 + 31 <= n - a.W;
+        const bool unmasked = key0 + q * 32 + 31 <= n - a.W;
         float acc = 0.f;
         for (int ph = 0; ph < HALVES; ++ph, ++u) {
           const int buf = u & 1;
@@ -458,11 +567,11 @@ cudaError_t launch_tc_t(const CompressArgs& a, cudaStream_t st, int passes) {
   if (e == cudaSuccess) e = set_smem_once<score_tc_kernel<D, 2, HALVES>>(C2::kSmem);
   if (e != cudaSuccess) return e;
   if (passes & kScoreRowstats) {
-    k1<<<grid1, cta_threads(1), C1::kSmem, st>>>(tq, tk1, a);
+    k1<<<grid1, cta_threads(1, a.V != nullptr), C1::kSmem, st>>>(tq, tk1, a);
     e = launch_rowstat_reduce(a, st);
     if (e != cudaSuccess) return e;
   }
-  if (passes & kScoreColsums) k2<<<grid2, cta_threads(2), C2::kSmem, st>>>(tq, tk2, a);
+  if (passes & kScoreColsums) k2<<<grid2, cta_threads(2, a.V != nullptr), C2::kSmem, st>>>(tq, tk2, a);
   return cudaGetLastError();
 }
 

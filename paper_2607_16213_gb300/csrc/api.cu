@@ -7,7 +7,7 @@
 #include "selkv_internal.cuh"
 
 namespace selkv {
-cudaError_t launch_setup(const CompressArgs& a, const SeqTable& tab, const SelectWs& w, cudaStream_t s);
+cudaError_t launch_setup(const CompressArgs& a, const SeqTable& tab, cudaStream_t s);
 cudaError_t launch_merge(const CompressArgs& a, cudaStream_t s);
 
 namespace {
@@ -142,15 +142,14 @@ T* at(void* ws, size_t off) {
 void note_launches(int kernels) { g_launches += (uint64_t)kernels; }
 
 // Kernels one selkv_compress call enqueues, mirroring the launch code: set-up; the scoring's two
-// passes and the fold of the row statistics between them; the selection
-// (pooling with digit pass 0 and digit passes 1-2 of each KV head's top-k, then, in the
-// shared mode only, the union with the trim's pass 0 and its passes 1-2; finally the
-// compaction's count and write); the RoPE tables when repositioning;
+// passes and the fold of the row statistics between them; the selection (pooling with each KV
+// head's top-k, then, in the shared mode only, the union and its trim, with the compaction in
+// the last of them); the RoPE tables when repositioning;
 // the routing and merge (bucket: route and merge, plus the kept-row copy unless the merge
 // does it; cosine: the copy and the cosine kernels); the bias.
 int compress_kernel_count(const CompressArgs& a) {
   int k = 1 + 3;
-  k += a.per_head ? 5 : 8;
+  k += a.per_head ? 1 : 2;
   if (a.rope != SELKV_ROPE_OFF) k += 1;
   if (a.routing == SELKV_ROUTE_COSINE)
     k += 1 + (a.m_cap > 0 ? cosine_kernels(a.dtype, a.D) : 0);
@@ -335,7 +334,7 @@ selkv_status selkv_compress(const selkv_shape* shape, const int32_t* n_len, doub
   }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const SelectWs sw = carve_select_ws(at<char>(workspace, plan.select), s.batch, s.num_kv_heads, s.n_cap);
-  cudaError_t e = launch_setup(a, tab, sw, st);
+  cudaError_t e = launch_setup(a, tab, st);
   // the scoring also takes the value norms
   if (e == cudaSuccess) e = score_uses_tc(a.dtype, a.D, a.R) ? launch_score_tc(a, st) : launch_score_simt(a, st);
   if (e == cudaSuccess)

@@ -1,20 +1,15 @@
-// Per-call set-up: sequence table, output lengths, the selection's initial states.
+// Per-call set-up: sequence table, output lengths.
 #include "selkv_internal.cuh"
 
 namespace selkv {
 namespace {
 
-// Sequence table, output lengths and the selection's initial radix states.
-__global__ void setup_kernel(SeqTable tab, CompressArgs a, SelectWs w) {
+// Sequence table and output lengths.
+__global__ void setup_kernel(SeqTable tab, CompressArgs a) {
   for (int b = threadIdx.x; b < a.B; b += blockDim.x) {
     a.seq_n[b] = tab.n[b];
     a.seq_m[b] = tab.m[b];
     a.lengths[b] = tab.m[b];
-  }
-  const int units = a.B * a.Hkv;
-  for (int i = threadIdx.x; i < units + a.B; i += blockDim.x) {
-    const int b = i >= units ? i - units : i / a.Hkv;
-    select_init_state(a, w, i, tab.n[b], tab.m[b]);
   }
 }
 
@@ -28,8 +23,8 @@ __global__ void seq_setup_kernel(SeqTable tab, int32_t* seq_n, int32_t* seq_m, i
 
 }  // namespace
 
-cudaError_t launch_setup(const CompressArgs& a, const SeqTable& tab, const SelectWs& w, cudaStream_t s) {
-  setup_kernel<<<1, 256, 0, s>>>(tab, a, w);
+cudaError_t launch_setup(const CompressArgs& a, const SeqTable& tab, cudaStream_t s) {
+  setup_kernel<<<1, 256, 0, s>>>(tab, a);
   return cudaGetLastError();
 }
 

@@ -209,52 +209,15 @@ __host__ __device__ constexpr int rope_coarse(int n_cap) { return n_cap / 256 + 
 
 constexpr int kRowChunk = 512;  // columns per CTA in the row-statistics pass
 
-// Grid-wide exact radix selection (select_grid.cu).
-struct RadixState {
-  uint32_t prefix;    // threshold bits fixed so far (the threshold T after the last pass)
-  uint32_t krem;      // entries still to take among those matching `prefix`
-  uint32_t count_eq;  // after the last pass: entries equal to T
-  int32_t jcut;       // last position taken among the entries equal to T
-  uint32_t active;    // a selection is still being narrowed
-  uint32_t arrive;    // CTAs of the current pass that have finished (self-resetting)
-  uint32_t ucount;    // trim only: size of the union
-  uint32_t pad;
+// Exact radix selection (select_grid.cu).
+struct RadixCut {
+  uint32_t T;  // bits of the threshold
+  int32_t jcut;  // last position taken among the entries equal to T
 };
 struct SelectWs {
-  RadixState* topk;     // [B * Hkv]
-  RadixState* trim;     // [B]
-  uint32_t* topk_hist;  // [B * Hkv][3][2048]
-  uint32_t* trim_hist;  // [B][3][2048]
-  size_t hist_bytes;    // both histogram arrays (contiguous)
-  uint32_t* blkcnt;     // [B][position blocks]
-  float* tkey;          // [B][n_cap] score summed over KV heads
-  uint8_t* uflag;       // [B][n_cap] member of the union
+  RadixCut* topk;  // [B * Hkv] each KV head's top-m_s
+  uint32_t* tkey;  // [B][n_cap] trim keys, where a span of them does not fit shared memory
 };
-// Initial radix state i of units + B: top-m_s per (b, kv), then the trim per b.  Called by
-// the set-up kernel with seq_n and seq_m of this call.
-__device__ __forceinline__ void select_init_state(const CompressArgs& a, const SelectWs& w, int i, int n_b, int m_b) {
-  const int units = a.B * a.Hkv;
-  const bool trim = i >= units;
-  const int b = trim ? i - units : i / a.Hkv;
-  (void)b;
-  const int k = m_b - a.recent;
-  const int ncand = n_b - a.recent;
-  RadixState s{};
-  s.krem = (uint32_t)max(k, 0);
-  s.jcut = INT_MAX;
-  if (trim) {
-    s.active = k > 0 ? 1u : 0u;  // the union kernel switches it off when |U| <= m_s
-  } else if (k <= 0) {
-    s.prefix = 0xffffffffu;  // select nothing
-    s.jcut = -1;
-  } else if (k >= ncand) {
-    s.prefix = 0u;  // select every candidate
-  } else {
-    s.active = 1u;
-  }
-  if (trim) w.trim[i - units] = s; else w.topk[i] = s;
-}
-
 size_t select_ws_bytes(int B, int Hkv, int n_cap);
 SelectWs carve_select_ws(void* base, int B, int Hkv, int n_cap);
 cudaError_t launch_select_grid(const CompressArgs& a, const SelectWs& w, cudaStream_t s);
@@ -330,6 +293,20 @@ cudaError_t set_smem_once(int bytes) {
   const uint64_t bit = dev < 64 ? (uint64_t)1 << dev : 0;
   if (bit != 0 && (done.load(std::memory_order_acquire) & bit)) return cudaSuccess;
   e = cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && bit != 0) done.fetch_or(bit, std::memory_order_acq_rel);
+  return e;
+}
+
+// Once per kernel and device: clusters of more than eight CTAs.
+template <auto Kern>
+cudaError_t allow_any_cluster_once() {
+  static std::atomic<uint64_t> done{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = dev < 64 ? (uint64_t)1 << dev : 0;
+  if (bit != 0 && (done.load(std::memory_order_acquire) & bit)) return cudaSuccess;
+  e = cudaFuncSetAttribute(Kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess && bit != 0) done.fetch_or(bit, std::memory_order_acq_rel);
   return e;
 }

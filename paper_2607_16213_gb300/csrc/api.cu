@@ -38,7 +38,7 @@ int score_chunks(const selkv_shape& s, int R) {
 }
 
 struct CompressPlan {
-  size_t seq_n, seq_m, rowpart, rowstat, attn, vnorm, rope_tab, mcount, score, kflag, slot, kept_pos, tau, atau, ratio, select, total;
+  size_t seq_n, seq_m, rowpart, rowstat, attn, vnorm, rope_tab, mcount, score, kflag, slot, kmask, kept_pos, tau, atau, ratio, select, total;
   size_t ev_pos, cos_invn, cos_rank, cos_order, cos_cnt, cos_seg;
   int nchunks, R;
 };
@@ -64,6 +64,7 @@ CompressPlan plan_compress(const selkv_shape& s) {
   // kept flags, slot maps: per sequence, or per KV head in the per-head mode (sized for that)
   p.kflag = take(B * Hkv * n);
   p.slot = take(B * Hkv * n * 4);
+  p.kmask = take(B * Hkv * ((n + 31) / 32) * sizeof(uint2));
   p.kept_pos = take(B * Hkv * (size_t)s.m_cap * 4);
   // merge targets per bucket, sized for the smallest bucket (the size is a call parameter)
   p.tau = take(B * Hkv * n * 4);
@@ -145,12 +146,14 @@ void note_launches(int kernels) { g_launches += (uint64_t)kernels; }
 // passes and the fold of the row statistics between them; the selection (pooling with each KV
 // head's top-k, then, in the shared mode only, the union and its trim, with the compaction in
 // the last of them); the RoPE tables when repositioning;
-// the routing and merge (bucket: route and merge, plus the kept-row copy unless the merge
-// does it; cosine: the copy and the cosine kernels); the bias.
+// the routing and merge (bucket: one kernel for bf16 and buckets of 32, else route and merge, plus
+// the kept-row copy unless the merge does it; cosine: the copy and the cosine kernels); the bias,
+// which the one kernel writes itself in the per-head mode.
 int compress_kernel_count(const CompressArgs& a) {
   int k = 1 + 3;
   k += a.per_head ? 1 : 2;
   if (a.rope != SELKV_ROPE_OFF) k += 1;
+  if (a.use_kmask) return k + 1 + (a.rope != SELKV_ROPE_OFF ? 1 : 0) + (a.per_head ? 0 : 1);
   if (a.routing == SELKV_ROUTE_COSINE)
     k += 1 + (a.m_cap > 0 ? cosine_kernels(a.dtype, a.D) : 0);
   else
@@ -305,6 +308,9 @@ selkv_status selkv_compress(const selkv_shape* shape, const int32_t* n_len, doub
   a.score = (debug && debug->score) ? debug->score : at<float>(workspace, plan.score);
   a.kflag = at<uint8_t>(workspace, plan.kflag);
   a.slot_of = at<int32_t>(workspace, plan.slot);
+  a.kmask = at<uint2>(workspace, plan.kmask);
+  a.kmask_ld = (s.n_cap + 31) / 32;
+  a.use_kmask = merge_uses_mma(s.dtype, s.head_dim, p.bucket, p.routing) ? 1 : 0;
   a.kept_pos = at<int32_t>(workspace, plan.kept_pos);
   a.nbk = (s.n_cap + p.bucket - 1) / p.bucket;
   a.tau = at<int32_t>(workspace, plan.tau);

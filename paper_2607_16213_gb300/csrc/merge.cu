@@ -1,5 +1,6 @@
 // Bucket-attention routing, soft cosine gate, gated merge, attention ratio and the
-// compressed-cache write-out of SelKV (Eq. 3-6, Sec. 3.6 GQA bias).  With the full cosine
+// compressed-cache write-out of SelKV (Eq. 3-6, Sec. 3.6 GQA bias).  bf16 caches with buckets of 32
+// take one kernel of merge_mma.cu for the routing, the merge and the copy.  With the full cosine
 // routing the route and merge kernels give way to those of route_cosine.cu, launched after
 // the copy.
 //
@@ -561,12 +562,16 @@ __global__ __launch_bounds__(256) void bias_kernel(CompressArgs a) {
 }
 
 template <typename T, int D>
-void launch_merge_t(const CompressArgs& a, cudaStream_t s) {
+void launch_copy_t(const CompressArgs& a, cudaStream_t s) {
   constexpr int kPieces = D * (int)sizeof(T) / 16;
   const size_t copy_threads = (size_t)a.Hkv * a.m_cap * 2 * kPieces;
+  copy_kernel<T, D><<<dim3((unsigned)((copy_threads + 255) / 256), a.B), 256, 0, s>>>(a);
+}
+
+template <typename T, int D>
+void launch_merge_t(const CompressArgs& a, cudaStream_t s) {
   // with the bucket routing and no repositioning the merge warps copy the kept rows themselves
-  if (!merge_copies_kept_rows(a))
-    copy_kernel<T, D><<<dim3((unsigned)((copy_threads + 255) / 256), a.B), 256, 0, s>>>(a);
+  if (!merge_copies_kept_rows(a)) launch_copy_t<T, D>(a, s);
   if (a.routing == SELKV_ROUTE_BUCKET) merge_kernel<T, D><<<dim3(a.nbk, a.B * a.Hkv), 32, 0, s>>>(a);
 }
 
@@ -581,6 +586,17 @@ cudaError_t launch_merge(const CompressArgs& a, cudaStream_t s) {
     const int groups = (a.rope_hi + 256 + kRopeRowsPerThread - 1) / kRopeRowsPerThread;
     const int threads = a.D / 2 * groups;
     rope_table_kernel<<<(threads + 127) / 128, 128, 0, s>>>(a);
+  }
+  if (a.use_kmask) {
+    if (a.rope != SELKV_ROPE_OFF) {
+      if (a.D == 128) launch_copy_t<__nv_bfloat16, 128>(a, s);
+      else launch_copy_t<__nv_bfloat16, 64>(a, s);
+    }
+    if (a.m_cap < 1) return cudaErrorInvalidConfiguration;  // no slot to launch for
+    const cudaError_t e = launch_merge_mma(a, s);
+    if (e != cudaSuccess || a.per_head) return e;
+    bias_kernel<<<dim3((a.m_cap + 255) / 256, a.B), 256, 0, s>>>(a);
+    return cudaGetLastError();
   }
   if (a.routing == SELKV_ROUTE_BUCKET)
     route_kernel<<<dim3((a.nbk + kWarpsPerCta - 1) / kWarpsPerCta, a.B), kWarpsPerCta * 32, 0, s>>>(a);

@@ -298,7 +298,7 @@ __device__ __forceinline__ void radix_select(Shared<NT>& sh, const Span& s, int 
   }
 }
 
-// Kept flags, slots in position order and the kept positions of selection unit u: the selected
+// Kept flags and slots in position order (or their masks) and the kept positions of selection unit u: the selected
 // keys below ncand and every position of the recent window [ncand, n).
 template <int NT>
 __device__ __forceinline__ void compact(const CompressArgs& a, Shared<NT>& sh, const Span& s, size_t u, int n, int ncand,
@@ -318,10 +318,13 @@ __device__ __forceinline__ void compact(const CompressArgs& a, Shared<NT>& sh, c
     const bool kept = kept_at(i);
     const uint32_t bal = __ballot_sync(0xffffffffu, kept);
     const int j = s.base + i, slot = (int)(slot0 + __popc(bal & ((1u << lane) - 1u)));
+    if (a.use_kmask && lane == 0) a.kmask[u * a.kmask_ld + (j >> 5)] = make_uint2(bal, slot0);
     slot0 += __popc(bal);
     if (j >= n) continue;
-    a.kflag[u * a.n_cap + j] = kept ? 1 : 0;
-    a.slot_of[u * a.n_cap + j] = kept ? slot : -1;
+    if (!a.use_kmask) {
+      a.kflag[u * a.n_cap + j] = kept ? 1 : 0;
+      a.slot_of[u * a.n_cap + j] = kept ? slot : -1;
+    }
     // with the full cosine routing: the evicted positions in order (slot = kept ones before j)
     if (!kept && a.routing == SELKV_ROUTE_COSINE) a.ev_pos[u * a.n_cap + (j - slot)] = j;
     if (kept && slot < a.m_cap) {

@@ -174,6 +174,11 @@ struct CompressArgs {
   uint8_t* kflag;    // [units][n_cap] 1 = kept (units: B, or B * Hkv in per-head mode)
   int32_t* slot_of;  // [units][n_cap] slot of a kept position, -1 otherwise
   int32_t* kept_pos; // [units][m_cap] position of each slot
+  // Kept masks per 32 positions (bit i: position 32 w + i is kept) and the slot of the first kept
+  // one, in the place of kflag and slot_of where merge_uses_mma
+  uint2* kmask;      // [units][kmask_ld] (mask, slot)
+  int kmask_ld;      // ceil(n_cap / 32)
+  int use_kmask;
   int nbk;           // buckets per sequence at n_cap: ceil(n_cap / bucket)
   int32_t* tau;      // [B][Hkv][nbk] merge target of each bucket (-1: no kept token)
   float* atau;       // [B][Hkv][nbk] a of that target
@@ -231,6 +236,9 @@ cudaError_t launch_score_tc(const CompressArgs& a, cudaStream_t s, int passes = 
 cudaError_t launch_score_simt(const CompressArgs& a, cudaStream_t s, int passes = kScoreAll);
 cudaError_t launch_seq_setup(const CompressArgs& a, const SeqTable& tab, cudaStream_t s);
 cudaError_t launch_rowstat_reduce(const CompressArgs& a, cudaStream_t s);
+// Routing, merge and kept-row copy in one kernel (merge_mma.cu): bf16, buckets of 32, bucket routing.
+bool merge_uses_mma(int dtype, int D, int bucket, int routing);
+cudaError_t launch_merge_mma(const CompressArgs& a, cudaStream_t s);
 // Compensation averaged across layers (layer_average.cu).
 constexpr int kMaxLayers = 128;
 struct LayerPtrs {

@@ -1,0 +1,74 @@
+"""The one-kernel merge of bf16 caches with 32-token buckets, against the oracle: lengths around the
+edges of a bucket and of a warp's walk, buckets without a kept token (tight budgets), both head
+sizes, and rows that are not finite."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from oracle import selkv_oracle as O
+from paper_2607_16213_gb300 import api
+import paper_2607_16213_gb300 as S
+
+from parity import check_sequence, params_of, run_compress, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_2607_16213_gb300 import build as b
+    b.build()
+    S.library()
+
+
+def workload(n, d=128, heads=(8, 2), batch=2, rho=0.25):
+    return synth.WORKLOADS["llama_layer"].with_(name="merge_%d" % n, batch=batch, n=n, head_dim=d, num_q_heads=heads[0],
+                                                num_kv_heads=heads[1], obs_window=24, rho=rho, ragged=(0.6, 1.0), seed=n)
+
+
+@pytest.mark.parametrize("mode", ["shared", "per_head", "rope", "drop"])
+@pytest.mark.parametrize("n,d,rho", [(64, 128, 0.5), (65, 64, 0.3), (95, 128, 0.3), (257, 64, 0.1), (2049, 128, 0.02),
+                                     (4000, 128, 0.008), (4000, 64, 0.6)])
+def test_merge_matches_the_oracle(n, d, rho, mode):
+    wl = workload(n, d, rho=rho, batch=1 if n >= 4000 else 2)
+    p = O.Params(recent=min(16, int(0.5 * rho * wl.n * 0.6)),
+                 select_mode=O.SELECT_PER_HEAD if mode == "per_head" else O.SELECT_SHARED,
+                 rope=O.ROPE_HALF if mode == "rope" else O.ROPE_OFF,
+                 empty_bucket=O.EMPTY_DROP if mode == "drop" else O.EMPTY_EXPAND)
+    x = synth.gen_layer(wl, 0)
+    _, host, _ = run_compress(wl, x, p)
+    for b in range(wl.batch):
+        check_sequence(wl, x, host, b, p)
+
+
+def test_long_walks_match_the_oracle():
+    """Enough buckets that a warp walks its longest range."""
+    wl = workload(26000, 64, heads=(16, 16), batch=1, rho=0.05).with_(ragged=None)
+    p = O.Params()
+    x = synth.gen_layer(wl, 0)
+    _, host, _ = run_compress(wl, x, p)
+    check_sequence(wl, x, host, 0, p)
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_a_kept_row_that_is_not_finite_stays_where_it_is(bad):
+    """Such a row is copied; the rows merged in its bucket are as without it."""
+    wl = workload(1000, batch=1).with_(ragged=None)
+    p = O.Params()
+    x = synth.gen_layer(wl, 0)
+    _, host, (K, V, Q) = run_compress(wl, x, p)
+    targets = set(host["target"][0].ravel().tolist())
+    pos = next(j for j in range(wl.n - 1, wl.n - p.recent - 1, -1) if j not in targets)
+    m = int(host["lengths"][0])
+    slot = int(np.flatnonzero(host["kept_idx"][0, :m] == pos)[0])
+    V2 = V.clone()
+    V2[0, :, pos, 3] = bad
+    shape = api.make_shape("bf16", 1, wl.num_q_heads, wl.num_kv_heads, wl.head_dim, wl.obs_window, wl.n,
+                           host["V_c"].shape[2])
+    c = api.compress(shape, [wl.n], wl.rho, K, V2, Q, params=params_of(p))
+    torch.cuda.synchronize()
+    got = c.V_c[0, :, :m].float().cpu().numpy()
+    others = np.arange(m) != slot
+    np.testing.assert_array_equal(got[:, others], host["V_c"][0, :, :m][:, others])
+    np.testing.assert_array_equal(got[:, slot], V2[0, :, pos].float().cpu().numpy())

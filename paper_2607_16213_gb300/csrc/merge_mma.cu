@@ -13,11 +13,13 @@
 //     times d x 8, every column v_tau): bf16 products are exact and the sums fp32;
 //   * sum_j w_j v_j is another (d x tokens times tokens x 8): column 0 holds the weights' upper 8
 //     bits, columns 1 and 2 the next two 8, so together all 24 bits of the fp32 weights count;
-//   * kept key rows are copied by 16-byte loads, the kept value rows from the tile.
+//   * the kept value rows are copied from the tile; the kept key rows by other warps of the same launch,
+//     64 slots each, with bulk copies in and out of shared memory.
 // A bucket takes about 450 warp instructions where the CUDA-core kernel took 1900 (unpacking,
 // shuffles, one row at a time) and lane 0 keeps 16 KB per warp in flight without registers.
-// It is bound by HBM on long sequences: one layer of 8 x 100k rows at 25% (358 MB) took 83 us with
-// the route kernel's 9 us on top, 64 x 8k at 10% (1.04 GB) 275 + 15 us.
+// It is bound by HBM on long sequences: one layer of 8 x 100k rows at 25% (358 MB) takes 67 us, 64 x
+// 8k at 10% (1.04 GB) 182 us, 80% and 84% of the copy rate (83 and 275 us before, with 9 and 15 us of
+// route kernel on top); short ones by a walk's chain of dependent loads.
 #include <climits>
 
 #include "ptx.cuh"
@@ -28,6 +30,7 @@ namespace {
 
 constexpr int kStages = 2;       // value tiles in flight per warp
 constexpr int kCtasPerSm = 12;   // one-warp CTAs resident per SM (18 KB of shared memory each)
+constexpr int kKeySlots = 64;    // key rows a copying warp moves
 #ifndef SELKV_MERGE_SEG
 #define SELKV_MERGE_SEG 8  // most buckets a warp walks
 #endif
@@ -83,9 +86,52 @@ __device__ __forceinline__ int argmax_kept(uint32_t mask, float a, int lane, flo
   return __ffs(__ballot_sync(kFull, ((mask >> lane) & 1u) && key == mx)) - 1;
 }
 
+// Key rows of slots [s0, s0 + kKeySlots) of (sequence, KV head) bk, a warp's work: one bulk copy a row
+// into the idle ring, then all of them to the slots, which are consecutive, with one.
+template <int D>
+__device__ __forceinline__ void copy_keys(const CompressArgs& a, int bk, size_t unit, int s0, int m, unsigned char* ring,
+                                          uint64_t* bar) {
+  static_assert(kKeySlots * D * 2 <= MCfg<D>::kVt && kKeySlots % 32 == 0, "the ring holds the rows");
+  const int lane = threadIdx.x, rows = min(kKeySlots, m - s0);
+  if (rows <= 0) return;
+  const __nv_bfloat16* Kb = static_cast<const __nv_bfloat16*>(a.K) + (size_t)bk * a.n_cap * D;
+  int pos[kKeySlots / 32];
+  bool in = true;
+#pragma unroll
+  for (int i = 0; i < kKeySlots / 32; ++i) {
+    const int r = i * 32 + lane;
+    pos[i] = r < rows ? a.kept_pos[unit * a.m_cap + s0 + r] : 0;
+    in = in && pos[i] >= 0 && pos[i] < a.n_cap;
+  }
+  if (!__all_sync(kFull, in)) {  // (cannot happen: the selection writes them)
+    if (lane == 0) raise_flag(a.flags, SELKV_DEVERR_COUNT);
+    return;
+  }
+  if (lane == 0) {
+    mbar_init(bar, 1);
+    fence_mbar_init();
+    mbar_arrive_expect_tx(bar, (uint32_t)rows * D * 2);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < kKeySlots / 32; ++i) {
+    const int r = i * 32 + lane;
+    if (r < rows) bulk_load(ring + r * D * 2, Kb + (size_t)pos[i] * D, D * 2, bar);
+  }
+  if (!__all_sync(kFull, mbar_wait(bar, 0))) {
+    if (lane == 0) raise_flag(a.flags, SELKV_DEVERR_TIMEOUT);
+    mbar_wait(bar, 0);  // (bounded) the copies land before the CTA leaves
+    return;
+  }
+  if (lane == 0) {
+    bulk_store(static_cast<__nv_bfloat16*>(a.Kc) + ((size_t)bk * a.m_cap + s0) * D, ring, (uint32_t)rows * D * 2);
+    bulk_store_wait();
+  }
+}
+
 template <int D>
 __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_constant__ CUtensorMap tmV,
-                                                                  CompressArgs a, int seg) {
+                                                                  CompressArgs a, int seg, int walks) {
   using C = MCfg<D>;
   using bf16 = __nv_bfloat16;
   constexpr int PER = D / 32;        // elements of a row per lane
@@ -98,6 +144,10 @@ __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kBars);
   const int lane = threadIdx.x;
   const int bk = blockIdx.y, b = bk / a.Hkv, kv = bk % a.Hkv;
+  if ((int)blockIdx.x >= walks) {
+    copy_keys<D>(a, bk, sel_unit(a, b, kv), ((int)blockIdx.x - walks) * kKeySlots, a.seq_m[b], smem, bars);
+    return;
+  }
   const int n = a.seq_n[b], nb = (n + 31) / 32;
   const int x0 = blockIdx.x * seg, x1 = min(nb, x0 + seg);
   if (x0 >= nb) return;
@@ -160,9 +210,7 @@ __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_
 
   const bool own_copy = a.rope == SELKV_ROPE_OFF;
   const int mi = lane >> 3, ri = lane & 7, g8 = lane >> 2, c4 = lane & 3;
-  const bf16* Kb = static_cast<const bf16*>(a.K) + row_base * D;
   const bf16* Vb = static_cast<const bf16*>(a.V) + row_base * D;
-  bf16* Kc = static_cast<bf16*>(a.Kc) + (size_t)bk * a.m_cap * D;
   bf16* Vc = static_cast<bf16*>(a.Vc) + (size_t)bk * a.m_cap * D;
 
   uint32_t mask = win.mask(X);
@@ -191,25 +239,28 @@ __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_
   issue(lo);
   prefetch();
 
+  // What the next target needs is loaded a target ahead: its a and norms, and v_tau of it as soon as
+  // its a decide tau.
+  RowSlice<bf16, PER> vt;
+  vt.load(Vb + ((size_t)X * 32 + tl) * D + lane * PER);
+  uint32_t maskR = 0u;
+  int slotR = 0;
+  float AR = 0.f, NR = 0.f;
+  auto fetch = [&](int e) {
+    maskR = win.mask(e);
+    slotR = win.slot0(e);
+    const int j = e * 32 + lane;
+    AR = j < n ? A[j] : 0.f;
+    NR = j < n ? vn[j] : 0.f;
+  };
+  int R = win.next(X + 1);
+  if (R < nb) fetch(R);
+
   bool ok = true;
   while (true) {
     bf16* vts = reinterpret_cast<bf16*>(smem + C::kVt);
-    RowSlice<bf16, PER> vt;
-    vt.load(Vb + ((size_t)X * 32 + tl) * D + lane * PER);
     const float vn_tau = __shfl_sync(kFull, NX, tl);
-    // the next target and, with its a, the last bucket that routes to X
-    const int R = win.next(X + 1);
-    uint32_t maskR = 0u;
-    int slotR = 0, tR = 0, hi = X;
-    float AR = 0.f, NR = 0.f, aR = 0.f;
-    if (R < nb) {
-      maskR = win.mask(R);
-      slotR = win.slot0(R);
-      if (R * 32 + lane < n) {
-        AR = A[R * 32 + lane];
-        NR = vn[R * 32 + lane];
-      }
-    }
+    int hi = X;
     const uint32_t below = mask & ((1u << lane) - 1u);
     const bool keptX = (mask >> lane) & 1u;
     const int nk = __popc(mask);
@@ -219,17 +270,7 @@ __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_
       else *reinterpret_cast<uint32_t*>(vts + lane * PER) = vt.w;
     }
     __syncwarp();
-    // the kept key rows on their way
     const int sub = lane / LPR, sl = lane % LPR;
-    constexpr int kKeyLoads = 4;
-    uint4 kr[kKeyLoads];
-    if (own_copy) {
-#pragma unroll
-      for (int i = 0; i < kKeyLoads; ++i) {
-        const int r = i * RPI + sub;
-        if (r < nk) kr[i] = *reinterpret_cast<const uint4*>(Kb + ((size_t)X * 32 + list[r]) * D + sl * 8);
-      }
-    }
     uint32_t vb[2 * KS];  // B fragments of v_tau, every column the same
 #pragma unroll
     for (int i = 0; i < KS / 2; ++i) {
@@ -238,13 +279,29 @@ __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_
 #pragma unroll
       for (int t = 0; t < 4; ++t) vb[4 * i + t] = f[t];
     }
-    if (R < nb) tR = argmax_kept(maskR, AR, lane, aR);
+    // the next target's tau, and with its a the last bucket that routes to X
+    const int Y = R;  // the next target (nb: none)
+    const uint32_t maskY = maskR;
+    const int slotY = slotR;
+    const float AY = AR, NY = NR;
+    float aY = 0.f;
+    int tY = 0;
+    RowSlice<bf16, PER> vtY;
+    vtY.zero();
+    if (Y < nb) {
+      tY = argmax_kept(maskY, AY, lane, aY);
+      if (Y < x1) {
+        vtY.load(Vb + ((size_t)Y * 32 + tY) * D + lane * PER);
+        R = win.next(Y + 1);
+        if (R < nb) fetch(R);
+      }
+    }
     if (expand) {
-      if (R >= nb) {
+      if (Y >= nb) {
         hi = nb - 1;
-      } else if (R > X + 1) {
-        hi = (X + R - 1) / 2;
-        if (((X + R) & 1) == 0 && a_tau >= aR) hi = (X + R) / 2;
+      } else if (Y > X + 1) {
+        hi = (X + Y - 1) / 2;
+        if (((X + Y) & 1) == 0 && a_tau >= aY) hi = (X + Y) / 2;
       }
     }
     if (nk > 0 && (slot0 < 0 || slot0 + nk > a.m_cap)) {  // (cannot happen: the selection keeps m <= m_cap)
@@ -360,26 +417,6 @@ __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_
     }
     if (!ok) break;
 
-    // the first key rows have arrived by now; the others follow
-    if (own_copy) {
-#pragma unroll
-      for (int i = 0; i < kKeyLoads; ++i) {
-        const int r = i * RPI + sub;
-        if (r < nk) *reinterpret_cast<uint4*>(Kc + (size_t)(slot0 + r) * D + sl * 8) = kr[i];
-      }
-      for (int r0 = kKeyLoads * RPI; r0 < nk; r0 += kKeyLoads * RPI) {
-#pragma unroll
-        for (int i = 0; i < kKeyLoads; ++i) {
-          const int r = r0 + i * RPI + sub;
-          if (r < nk) kr[i] = *reinterpret_cast<const uint4*>(Kb + ((size_t)X * 32 + list[r]) * D + sl * 8);
-        }
-#pragma unroll
-        for (int i = 0; i < kKeyLoads; ++i) {
-          const int r = r0 + i * RPI + sub;
-          if (r < nk) *reinterpret_cast<uint4*>(Kc + (size_t)(slot0 + r) * D + sl * 8) = kr[i];
-        }
-      }
-    }
     // the target's value row: columns 0-2 of the product added up, a row's elements to its lane
 #pragma unroll
     for (int m = 0; m < MT; ++m) {
@@ -419,24 +456,25 @@ __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_
     __syncwarp();  // the lists and sums are read; the next target rewrites them
 
     if (!expand) {
-      dbg_untargeted(X + 1, min(R, x1));
-      if (R < x1) {  // step over the tiles of the empty buckets between
-        for (int e = X + 1; e < R && ok; ++e)
+      dbg_untargeted(X + 1, min(Y, x1));
+      if (Y < x1) {  // step over the tiles of the empty buckets between
+        for (int e = X + 1; e < Y && ok; ++e)
           if (e < next_e) {
             ok = wait_tile();
             ++consumed;
           }
-        next_e = max(next_e, R);
+        next_e = max(next_e, Y);
       }
     }
-    if (R >= x1 || !ok) break;
-    X = R;
-    mask = maskR;
-    slot0 = slotR;
-    AX = AR;
-    NX = NR;
-    tl = tR;
-    a_tau = aR;
+    if (Y >= x1 || !ok) break;
+    X = Y;
+    mask = maskY;
+    slot0 = slotY;
+    AX = AY;
+    NX = NY;
+    tl = tY;
+    a_tau = aY;
+    vt = vtY;
     lo = expand ? hi + 1 : X;
   }
   if (!ok && lane == 0) raise_flag(a.flags, SELKV_DEVERR_TIMEOUT);
@@ -454,7 +492,10 @@ cudaError_t launch_t(const CompressArgs& a, cudaStream_t s) {
   const int units = a.B * a.Hkv, nb = (a.n_cap + 31) / 32;
   const long long per = (long long)units * nb / (kPlanSMs * kCtasPerSm);
   const int seg = (int)(per < 1 ? 1 : per > SELKV_MERGE_SEG ? SELKV_MERGE_SEG : per);
-  merge_mma_kernel<D><<<dim3((nb + seg - 1) / seg, units), 32, MCfg<D>::kSmem, s>>>(tv, a, seg);
+  const int walks = (nb + seg - 1) / seg;
+  // with repositioning copy_kernel writes the keys
+  const int keys = a.rope == SELKV_ROPE_OFF ? (a.m_cap + kKeySlots - 1) / kKeySlots : 0;
+  merge_mma_kernel<D><<<dim3(walks + keys, units), 32, MCfg<D>::kSmem, s>>>(tv, a, seg, walks);
   return cudaGetLastError();
 }
 

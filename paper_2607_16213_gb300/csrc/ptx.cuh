@@ -197,6 +197,15 @@ __device__ __forceinline__ uint32_t swz128(int row, int chunk) {
 
 namespace selkv {
 
+// Bulk copy from this CTA's shared memory to global memory (16-byte aligned, whole 16 bytes); the
+// issuing thread waits for it with bulk_store_wait.
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n cp.async.bulk.commit_group;" ::"l"(dst),
+               "r"(smem_u32(src)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_store_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
 // ---- tcgen05 (5th-generation tensor cores, accumulators in tensor memory) ----------------
 // Instruction descriptor, kind::f16: bf16 A and B (both K-major), fp32 D, M x N tile.
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {

@@ -31,10 +31,12 @@ bool shape_ok(const selkv_shape* s) {
 
 size_t round256(size_t x) { return (x + 255) & ~size_t(255); }
 
+int simt_chunk(const selkv_shape& s, int R) { return score_simt_chunk(s.batch, s.num_kv_heads, s.n_cap, R); }
+
 // Key slices of the scoring's first pass (one row-statistics partial per slice and row).
 int score_chunks(const selkv_shape& s, int R) {
   return score_uses_tc(s.dtype, s.head_dim, R) ? score_tc_splits(s.batch, s.num_kv_heads, s.n_cap, R, kPlanSMs)
-                                               : (int)(((size_t)s.n_cap + kRowChunk - 1) / kRowChunk);
+                                               : (int)(((size_t)s.n_cap + simt_chunk(s, R) - 1) / simt_chunk(s, R));
 }
 
 struct CompressPlan {
@@ -279,6 +281,7 @@ selkv_status selkv_compress(const selkv_shape* shape, const int32_t* n_len, doub
   a.m_cap = s.m_cap;
   a.R = plan.R;
   a.nchunks = plan.nchunks;
+  a.row_chunk = simt_chunk(s, plan.R);
   a.alpha = p.alpha;
   a.pool_kernel = p.pool_kernel;
   a.bucket = p.bucket;
@@ -388,6 +391,7 @@ selkv_status selkv_score(const selkv_shape* shape, const int32_t* n_len, const v
   a.m_cap = s.m_cap;
   a.R = plan.R;
   a.nchunks = plan.nchunks;
+  a.row_chunk = simt_chunk(s, plan.R);
   a.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)s.head_dim));
   a.K = K;
   a.Q = Q_obs;

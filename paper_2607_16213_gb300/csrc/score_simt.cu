@@ -94,8 +94,8 @@ __global__ __launch_bounds__(256) void rowstats_kernel(CompressArgs a) {
   float m_run[4], l_run[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) { m_run[i] = -INFINITY; l_run[i] = 0.f; }
-  const int c_begin = chunk * kRowChunk;
-  const int c_end = min(n, c_begin + kRowChunk);
+  const int c_begin = chunk * a.row_chunk;
+  const int c_end = min(n, c_begin + a.row_chunk);
   for (int c0 = c_begin; c0 < c_end; c0 += kTile) {
     float acc[4][4];
     score_tile<T, D>(a, b, kv, n, r0, c0, Qs, Ks, acc);
@@ -141,8 +141,10 @@ __device__ __forceinline__ void fold_row(const CompressArgs& a, int idx) {
   const int nch = a.nchunks;  // chunks without visible columns hold (-inf, 0)
   const float2* part = a.rowpart + (size_t)bk * a.nchunks * a.R + r;
   float M = -INFINITY;
+#pragma unroll 8
   for (int c = 0; c < nch; ++c) M = fmaxf(M, part[(size_t)c * a.R].x);
   float Z = 0.f;
+#pragma unroll 8
   for (int c = 0; c < nch; ++c) {
     const float2 p = part[(size_t)c * a.R];
     if (p.x != -INFINITY) Z += p.y * exp2f(p.x - M);

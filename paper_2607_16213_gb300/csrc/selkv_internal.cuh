@@ -139,6 +139,7 @@ struct CompressArgs {
   int dtype, B, Hq, Hkv, G, D, W, n_cap, m_cap;
   int R;          // observation rows per KV head: G * W
   int nchunks;    // column chunks of the row-statistics pass
+  int row_chunk;  // columns of a chunk (CUDA-core scoring)
   float alpha;
   int pool_kernel, bucket, recent, gate_mode, empty_bucket;
   int per_head;   // SELKV_SELECT_PER_HEAD: selection units are (b, kv), not b
@@ -212,7 +213,14 @@ __host__ __device__ __forceinline__ size_t sel_unit(const CompressArgs& a, int b
 // e = 256 e_hi + e_lo.
 __host__ __device__ constexpr int rope_coarse(int n_cap) { return n_cap / 256 + 1; }
 
-constexpr int kRowChunk = 512;  // columns per CTA in the row-statistics pass
+// Columns per CTA in the CUDA-core row-statistics pass: 512 (few partials to fold), halved down to
+// a tile of 64 while the CTAs would leave SMs empty (one prompt of 1k with 2 KV heads: 4 CTAs of 512
+// columns took 40 us, 32 of 64 take 7).
+__host__ __device__ constexpr int score_simt_chunk(int B, int Hkv, int n_cap, int R) {
+  int chunk = 512;
+  while (chunk > 64 && (long long)B * Hkv * ((R + 63) / 64) * ((n_cap + chunk - 1) / chunk) < kPlanSMs) chunk /= 2;
+  return chunk;
+}
 
 // Exact radix selection (select_grid.cu).
 struct RadixCut {

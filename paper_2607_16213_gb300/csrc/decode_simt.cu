@@ -17,14 +17,49 @@
 namespace selkv {
 namespace {
 
-constexpr int kWarps = 4;
+// A warp takes kLoads loads of K and as many of V at a time, all in flight together: a lane holds
+// four elements of a row, so D / 4 lanes share a row and a step covers kLoads * 128 / D keys.
+// Small caches are bound by latency, a token of one sequence of 256 rows by its whole chain: with
+// a row per lane (its elements loaded eight at a time, values row by row) that launch took 27 us, now
+// 11 (both from a cold L2).
+constexpr int kLoads = 8;
+// Warps of a CTA (the fold's scratch stays within 48 KB of static shared memory).
+constexpr int warps_of(int GM) { return GM <= 8 ? 8 : 4; }
+
+// Sums of x[i] over the D / 4 lanes of a row, spread over them: every level keeps half of the
+// values and adds the partner's, so a lane ends with the sum of one i, given by its lane bits.
+template <int LPR>
+__device__ __forceinline__ float spread_sum(const float (&x)[kLoads], int lane) {
+  float q[kLoads];
+#pragma unroll
+  for (int i = 0; i < kLoads; ++i) q[i] = x[i];
+#pragma unroll
+  for (int o = LPR / 2, keep = kLoads; o > 0; o >>= 1) {
+    const bool up = lane & o;
+    if (keep > 1) {
+      keep >>= 1;
+#pragma unroll
+      for (int i = 0; i < keep; ++i) {
+        const float mine = up ? q[keep + i] : q[i], other = up ? q[i] : q[keep + i];
+        q[i] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+      }
+    } else {
+      q[0] += __shfl_xor_sync(0xffffffffu, q[0], o);
+    }
+  }
+  return q[0];
+}
 
 template <typename T, int D, int GM>
-__global__ __launch_bounds__(kWarps * 32) void decode_simt_kernel(DecodeArgs a) {
-  constexpr int PER = D / 32;
+__global__ __launch_bounds__(warps_of(GM) * 32) void decode_simt_kernel(DecodeArgs a) {
+  constexpr int kWarps = warps_of(GM);
+  constexpr int LPR = D / 4, RPI = 32 / LPR;  // lanes per row, rows per load
+  constexpr int kKeys = kLoads * RPI;         // keys of a warp's step
+  constexpr int kLow = LPR / kLoads;          // lanes that end with the same sum
+  static_assert(kLow >= 1, "a row's lanes hold every sum");
   __shared__ __align__(16) float qs[GM][D];
   __shared__ float wm[kWarps][GM], wl[kWarps][GM];
-  __shared__ float wo[kWarps][GM][D];
+  __shared__ __align__(16) float wo[kWarps][GM][D];
   __shared__ bool s_last;
   const int s = blockIdx.x, kv = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -32,6 +67,10 @@ __global__ __launch_bounds__(kWarps * 32) void decode_simt_kernel(DecodeArgs a) 
   const size_t bk = (size_t)b * a.Hkv + kv;
 
   int L = a.lengths[b];
+  for (int i = tid; i < G * D; i += blockDim.x) {
+    const int g = i / D, d = i % D;
+    qs[g][d] = load1(static_cast<const T*>(a.q) + ((size_t)b * a.Hq + kv * G + g) * D + d) * a.scale_log2;
+  }
   if (L < 0 || L > a.m_cap) {
     if (tid == 0 && s == 0 && kv == 0) raise_flag(a.flags, SELKV_DEVERR_LENGTH);
     L = L < 0 ? 0 : a.m_cap;
@@ -44,11 +83,6 @@ __global__ __launch_bounds__(kWarps * 32) void decode_simt_kernel(DecodeArgs a) 
   const int total = L + (app ? 1 : 0);
   const int chunk = ((total + S - 1) / S + 31) / 32 * 32;
   const int lo = s * chunk, hi = min(total, lo + chunk);
-
-  for (int i = tid; i < G * D; i += blockDim.x) {
-    const int g = i / D, d = i % D;
-    qs[g][d] = load1(static_cast<const T*>(a.q) + ((size_t)b * a.Hq + kv * G + g) * D + d) * a.scale_log2;
-  }
   __syncthreads();
 
   const T* Kb = static_cast<const T*>(a.Kc) + bk * a.m_cap * D;
@@ -57,61 +91,61 @@ __global__ __launch_bounds__(kWarps * 32) void decode_simt_kernel(DecodeArgs a) 
   const T* vnw = app ? static_cast<const T*>(a.v_new) + bk * D : nullptr;
   const float* bias = a.bias != nullptr ? a.bias + bk * a.m_cap : nullptr;
 
-  float m[GM], l[GM], o[GM][PER], pg[GM];
+  const int sub = lane / LPR, e0 = (lane % LPR) * 4;
+  // the key of a step whose logit this lane ends with: load `mine` of its row group
+  const int mine = (lane % LPR) / kLow;
+  float m[GM], l[GM], o[GM][4];
 #pragma unroll
   for (int g = 0; g < GM; ++g) {
     m[g] = -INFINITY;
     l[g] = 0.f;
 #pragma unroll
-    for (int e = 0; e < PER; ++e) o[g][e] = 0.f;
+    for (int e = 0; e < 4; ++e) o[g][e] = 0.f;
   }
-  for (int t0 = lo + warp * 32; t0 < hi; t0 += kWarps * 32) {
-    const int key = t0 + lane;
-    const bool valid = key < hi;
-    float sc[GM];
+  for (int t0 = lo + warp * kKeys; t0 < hi; t0 += kWarps * kKeys) {
+    float k[kLoads][4], v[kLoads][4];
 #pragma unroll
-    for (int g = 0; g < GM; ++g) sc[g] = 0.f;
-    if (valid) {
-      const T* kr = key < L ? Kb + (size_t)key * D : kn;
-#pragma unroll 4
-      for (int d = 0; d < D; d += 8) {
-        float x[8];
-        load8(kr + d, x);
+    for (int i = 0; i < kLoads; ++i) {
+      const int key = t0 + i * RPI + sub;
+      if (key < hi) {
+        load4((key < L ? Kb + (size_t)key * D : kn) + e0, k[i]);
+        load4((key < L ? Vb + (size_t)key * D : vnw) + e0, v[i]);
+      } else {
 #pragma unroll
-        for (int g = 0; g < GM; ++g) {
-          if (g < G) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) sc[g] = fmaf(qs[g][d + e], x[e], sc[g]);
-          }
-        }
+        for (int e = 0; e < 4; ++e) k[i][e] = v[i][e] = 0.f;
       }
     }
-    const float bv = (valid && key < L && bias != nullptr) ? bias[key] * kLog2e : 0.f;
+    const int key = t0 + mine * RPI + sub;
+    const bool valid = key < hi;
+    const float bv = (key < min(hi, L) && bias != nullptr) ? bias[key] * kLog2e : 0.f;
 #pragma unroll
     for (int g = 0; g < GM; ++g) {
       if (g >= G) break;
-      const float v = valid ? sc[g] + bv : -INFINITY;
-      const float mn = fmaxf(m[g], warp_max(v));
+      const float4 q = *reinterpret_cast<const float4*>(&qs[g][e0]);
+      float part[kLoads];
+#pragma unroll
+      for (int i = 0; i < kLoads; ++i)
+        part[i] = fmaf(k[i][3], q.w, fmaf(k[i][2], q.z, fmaf(k[i][1], q.y, k[i][0] * q.x)));
+      const float dot = spread_sum<LPR>(part, lane);
+      const float x = valid ? dot + bv : -INFINITY;
+      float mx = x;
+#pragma unroll
+      for (int d = kLow; d < 32; d <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+      const float mn = fmaxf(m[g], mx);
       const float corr = exp2f(m[g] - mn);
-      const float p = exp2f(v - mn);
-      l[g] = l[g] * corr + warp_sum(p);
+      const float p = exp2f(x - mn);
+      float ps = p;
 #pragma unroll
-      for (int e = 0; e < PER; ++e) o[g][e] *= corr;
+      for (int d = kLow; d < 32; d <<= 1) ps += __shfl_xor_sync(0xffffffffu, ps, d);
+      l[g] = l[g] * corr + ps;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) o[g][e] *= corr;
       m[g] = mn;
-      pg[g] = p;
-    }
-    const int nk = min(32, hi - t0);
-    for (int k = 0; k < nk; ++k) {
-      const int key2 = t0 + k;
-      const T* vr = key2 < L ? Vb + (size_t)key2 * D : vnw;
-      float v[PER];
-      if constexpr (PER == 4) load4(vr + lane * 4, v); else load2(vr + lane * 2, v);
 #pragma unroll
-      for (int g = 0; g < GM; ++g) {
-        if (g >= G) break;
-        const float pk = __shfl_sync(0xffffffffu, pg[g], k);
+      for (int i = 0; i < kLoads; ++i) {
+        const float pi = __shfl_sync(0xffffffffu, p, sub * LPR + i * kLow);
 #pragma unroll
-        for (int e = 0; e < PER; ++e) o[g][e] = fmaf(pk, v[e], o[g][e]);
+        for (int e = 0; e < 4; ++e) o[g][e] = fmaf(pi, v[i][e], o[g][e]);
       }
     }
   }
@@ -123,8 +157,12 @@ __global__ __launch_bounds__(kWarps * 32) void decode_simt_kernel(DecodeArgs a) 
       wm[warp][g] = m[g];
       wl[warp][g] = l[g];
     }
+    // the row groups of a warp share its max and sum: their outputs are added
 #pragma unroll
-    for (int e = 0; e < PER; ++e) wo[warp][g][lane * PER + e] = o[g][e];
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+      for (int d = LPR; d < 32; d <<= 1) o[g][e] += __shfl_xor_sync(0xffffffffu, o[g][e], d);
+    if (sub == 0) *reinterpret_cast<float4*>(&wo[warp][g][e0]) = make_float4(o[g][0], o[g][1], o[g][2], o[g][3]);
   }
   __syncthreads();
   write_split_partial<kWarps>(a, b, kv, s, &wo[0][0][0], &wm[0][0], &wl[0][0], GM, D, false);
@@ -137,12 +175,11 @@ __global__ __launch_bounds__(kWarps * 32) void decode_simt_kernel(DecodeArgs a) 
 template <typename T, int D>
 cudaError_t launch_t(const DecodeArgs& a, cudaStream_t st) {
   const dim3 grid(a.splits, a.Hkv, a.B);
-  const int th = kWarps * 32;
-  if (a.G <= 1) decode_simt_kernel<T, D, 1><<<grid, th, 0, st>>>(a);
-  else if (a.G <= 2) decode_simt_kernel<T, D, 2><<<grid, th, 0, st>>>(a);
-  else if (a.G <= 4) decode_simt_kernel<T, D, 4><<<grid, th, 0, st>>>(a);
-  else if (a.G <= 8) decode_simt_kernel<T, D, 8><<<grid, th, 0, st>>>(a);
-  else decode_simt_kernel<T, D, 16><<<grid, th, 0, st>>>(a);
+  if (a.G <= 1) decode_simt_kernel<T, D, 1><<<grid, warps_of(1) * 32, 0, st>>>(a);
+  else if (a.G <= 2) decode_simt_kernel<T, D, 2><<<grid, warps_of(2) * 32, 0, st>>>(a);
+  else if (a.G <= 4) decode_simt_kernel<T, D, 4><<<grid, warps_of(4) * 32, 0, st>>>(a);
+  else if (a.G <= 8) decode_simt_kernel<T, D, 8><<<grid, warps_of(8) * 32, 0, st>>>(a);
+  else decode_simt_kernel<T, D, 16><<<grid, warps_of(16) * 32, 0, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -215,7 +215,7 @@ __host__ __device__ constexpr int rope_coarse(int n_cap) { return n_cap / 256 + 
 
 // Columns per CTA in the CUDA-core row-statistics pass: 512 (few partials to fold), halved down to
 // a tile of 64 while the CTAs would leave SMs empty (one prompt of 1k with 2 KV heads: 4 CTAs of 512
-// columns took 40 us, 32 of 64 take 7).
+// columns took 40 us, 32 of 64 take 8).
 __host__ __device__ constexpr int score_simt_chunk(int B, int Hkv, int n_cap, int R) {
   int chunk = 512;
   while (chunk > 64 && (long long)B * Hkv * ((R + 63) / 64) * ((n_cap + chunk - 1) / chunk) < kPlanSMs) chunk /= 2;

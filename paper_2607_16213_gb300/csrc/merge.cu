@@ -349,6 +349,7 @@ template <typename T, int D>
 #endif
 __global__ __launch_bounds__(32, SELKV_MERGE_MINB) void merge_kernel(CompressArgs a) {
   constexpr int PER = D / 32;  // elements of a row per lane
+  __shared__ unsigned char list[32];
   const int lane = threadIdx.x;
   const int X = blockIdx.x;
   const int kv = blockIdx.y % a.Hkv, b = blockIdx.y / a.Hkv;
@@ -453,30 +454,24 @@ __global__ __launch_bounds__(32, SELKV_MERGE_MINB) void merge_kernel(CompressArg
   for (int e = lo_b; e <= hi_b; ++e) {
     const int eb = e * Bs;
     const int cnt_e = min(Bs, n - eb);
-    uint32_t rem = e == X ? evX : (cnt_e >= 32 ? 0xffffffffu : ((1u << cnt_e) - 1u));
+    const uint32_t rem = e == X ? evX : (cnt_e >= 32 ? 0xffffffffu : ((1u << cnt_e) - 1u));
     // a and ||v|| of bucket e, one position per lane
     const float Ae = e == X ? AX : (lane < cnt_e ? A[eb + lane] : 0.f);
     const float Ne = e == X ? NX : (lane < cnt_e ? vn[eb + lane] : 0.f);
-    while (rem) {
-      // the (up to) kBatch lowest contributors left in this bucket
-      const int cut = __fns(rem, 0, kBatch + 1);  // position of the (kBatch+1)-th set bit
-      const uint32_t bm = (cut < 0 || cut > 31) ? rem : (rem & ((1u << cut) - 1u));
-      rem &= ~bm;
-      const int cnt = __popc(bm);
+    // the bucket's contributors in order, kBatch of them at a time
+    __syncwarp();
+    if ((rem >> lane) & 1u) list[__popc(rem & ((1u << lane) - 1u))] = (unsigned char)lane;
+    __syncwarp();
+    const int all = __popc(rem);
+    for (int c0 = 0; c0 < all; c0 += kBatch) {
+      const int cnt = min(kBatch, all - c0);
       RowSlice<T, PER> vj[kBatch];
-      {
-        uint32_t r = bm;
 #pragma unroll
-        for (int k = 0; k < kBatch; ++k) {
-          if (r) {
-            vj[k].load(Vb + (size_t)(eb + __ffs(r) - 1) * D + lane * PER);
-            r &= r - 1u;
-          } else {
-            vj[k].zero();
-          }
-        }
+      for (int k = 0; k < kBatch; ++k) {
+        if (k < cnt) vj[k].load(Vb + (size_t)(eb + list[c0 + k]) * D + lane * PER);
+        else vj[k].zero();
       }
-      const int ob = own < cnt ? (int)__fns(bm, 0, own + 1) : -1;  // bit of the owned contributor
+      const int ob = own < cnt ? list[c0 + own] : -1;  // lane of the owned contributor
       const float ak = __shfl_sync(0xffffffffu, Ae, ob < 0 ? 0 : ob);
       const float nk = __shfl_sync(0xffffffffu, Ne, ob < 0 ? 0 : ob);
       float g;

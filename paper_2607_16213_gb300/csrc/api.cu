@@ -31,16 +31,18 @@ bool shape_ok(const selkv_shape* s) {
 
 size_t round256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// Column chunks of the CUDA-core scoring.
 int simt_chunk(const selkv_shape& s, int R) { return score_simt_chunk(s.batch, s.num_kv_heads, s.n_cap, R); }
+size_t simt_chunks(const selkv_shape& s, int R) { return ((size_t)s.n_cap + simt_chunk(s, R) - 1) / simt_chunk(s, R); }
 
-// Key slices of the scoring's first pass (one row-statistics partial per slice and row).
-int score_chunks(const selkv_shape& s, int R) {
-  return score_uses_tc(s.dtype, s.head_dim, R) ? score_tc_splits(s.batch, s.num_kv_heads, s.n_cap, R, kPlanSMs)
-                                               : (int)(((size_t)s.n_cap + simt_chunk(s, R) - 1) / simt_chunk(s, R));
+// Row-statistics partials of the scoring's first pass, in rows of R.
+size_t score_partials(const selkv_shape& s, int R) {
+  if (score_uses_tc(s.dtype, s.head_dim, R)) return score_tc_partials(s.batch, s.num_kv_heads);
+  return (size_t)s.batch * s.num_kv_heads * simt_chunks(s, R);
 }
 
 struct CompressPlan {
-  size_t seq_n, seq_m, rowpart, rowstat, attn, vnorm, rope_tab, mcount, score, kflag, slot, kmask, kept_pos, tau, atau, ratio, select, total;
+  size_t seq_n, seq_m, seq_t1, rowpart, rowstat, attn, vnorm, rope_tab, mcount, score, kflag, slot, kmask, kept_pos, tau, atau, ratio, select, total;
   size_t ev_pos, cos_invn, cos_rank, cos_order, cos_cnt, cos_seg;
   int nchunks, R;
 };
@@ -55,10 +57,11 @@ CompressPlan plan_compress(const selkv_shape& s) {
   };
   const size_t B = s.batch, Hkv = s.num_kv_heads, n = s.n_cap;
   p.R = (s.num_q_heads / s.num_kv_heads) * s.obs_window;
-  p.nchunks = score_chunks(s, p.R);
+  p.nchunks = (int)simt_chunks(s, p.R);
   p.seq_n = take(B * 4);
   p.seq_m = take(B * 4);
-  p.rowpart = take(B * Hkv * (size_t)p.nchunks * p.R * sizeof(float2));
+  p.seq_t1 = take(B * 4);
+  p.rowpart = take(score_partials(s, p.R) * p.R * sizeof(float2));
   p.rowstat = take(B * Hkv * (size_t)p.R * sizeof(float2));
   p.attn = take(B * Hkv * n * 4);
   p.vnorm = take(B * Hkv * n * 4);
@@ -90,7 +93,7 @@ CompressPlan plan_compress(const selkv_shape& s) {
 }
 
 struct ScorePlan {
-  size_t seq_n, seq_m, rowpart, rowstat, total;
+  size_t seq_n, seq_m, seq_t1, rowpart, rowstat, total;
   int nchunks, R;
 };
 
@@ -104,10 +107,11 @@ ScorePlan plan_score(const selkv_shape& s) {
   };
   const size_t B = s.batch, Hkv = s.num_kv_heads;
   p.R = (s.num_q_heads / s.num_kv_heads) * s.obs_window;
-  p.nchunks = score_chunks(s, p.R);
+  p.nchunks = (int)simt_chunks(s, p.R);
   p.seq_n = take(B * 4);
   p.seq_m = take(B * 4);
-  p.rowpart = take(B * Hkv * (size_t)p.nchunks * p.R * sizeof(float2));
+  p.seq_t1 = take(B * 4);
+  p.rowpart = take(score_partials(s, p.R) * p.R * sizeof(float2));
   p.rowstat = take(B * Hkv * (size_t)p.R * sizeof(float2));
   p.total = off;
   return p;
@@ -145,14 +149,14 @@ T* at(void* ws, size_t off) {
 void note_launches(int kernels) { g_launches += (uint64_t)kernels; }
 
 // Kernels one selkv_compress call enqueues, mirroring the launch code: set-up; the scoring's two
-// passes and the fold of the row statistics between them; the selection (pooling with each KV
+// passes and, on CUDA cores, the fold of the row statistics between them; the selection (pooling with each KV
 // head's top-k, then, in the shared mode only, the union and its trim, with the compaction in
 // the last of them); the RoPE tables when repositioning;
 // the routing and merge (bucket: one kernel for bf16 and buckets of 32, else route and merge, plus
 // the kept-row copy unless the merge does it; cosine: the copy and the cosine kernels); the bias,
 // which the one kernel writes itself in the per-head mode.
 int compress_kernel_count(const CompressArgs& a) {
-  int k = 1 + 3;
+  int k = 1 + (score_uses_tc(a.dtype, a.D, a.R) ? 2 : 3);
   k += a.per_head ? 1 : 2;
   if (a.rope != SELKV_ROPE_OFF) k += 1;
   if (a.use_kmask) return k + 1 + (a.rope != SELKV_ROPE_OFF ? 1 : 0) + (a.per_head ? 0 : 1);
@@ -264,6 +268,7 @@ selkv_status selkv_compress(const selkv_shape* shape, const int32_t* n_len, doub
     if (m - p.recent < 0 || m > s.m_cap || m > n) return SELKV_ERR_INVALID_ARG;
     tab.n[b] = n;
     tab.m[b] = m;
+    tab.t1[b] = b > 0 ? tab.t1[b - 1] + score_tc_tiles1(tab.n[b - 1]) : 0;
   }
   const CompressPlan plan = plan_compress(s);
   if (workspace == nullptr || !aligned(workspace, 256)) return SELKV_ERR_WORKSPACE;
@@ -304,6 +309,7 @@ selkv_status selkv_compress(const selkv_shape* shape, const int32_t* n_len, doub
   a.flags = at<uint32_t>(workspace, 0);
   a.seq_n = at<int32_t>(workspace, plan.seq_n);
   a.seq_m = at<int32_t>(workspace, plan.seq_m);
+  a.seq_t1 = at<int32_t>(workspace, plan.seq_t1);
   a.rowpart = at<float2>(workspace, plan.rowpart);
   a.rowstat = at<float2>(workspace, plan.rowstat);
   a.attn = (debug && debug->attn) ? debug->attn : at<float>(workspace, plan.attn);
@@ -345,7 +351,7 @@ selkv_status selkv_compress(const selkv_shape* shape, const int32_t* n_len, doub
   const SelectWs sw = carve_select_ws(at<char>(workspace, plan.select), s.batch, s.num_kv_heads, s.n_cap);
   cudaError_t e = launch_setup(a, tab, st);
   // the scoring also takes the value norms
-  if (e == cudaSuccess) e = score_uses_tc(a.dtype, a.D, a.R) ? launch_score_tc(a, st) : launch_score_simt(a, st);
+  if (e == cudaSuccess) e = score_uses_tc(a.dtype, a.D, a.R) ? launch_score_tc(a, tab, st) : launch_score_simt(a, st);
   if (e == cudaSuccess)
     e = launch_select_grid(a, sw, st);
   if (e == cudaSuccess) e = launch_merge(a, st);
@@ -375,6 +381,7 @@ selkv_status selkv_score(const selkv_shape* shape, const int32_t* n_len, const v
     if (n < s.obs_window || n > s.n_cap) return SELKV_ERR_INVALID_ARG;
     tab.n[b] = n;
     tab.m[b] = 0;
+    tab.t1[b] = b > 0 ? tab.t1[b - 1] + score_tc_tiles1(tab.n[b - 1]) : 0;
   }
   const ScorePlan plan = plan_score(s);
   if (workspace == nullptr || !aligned(workspace, 256)) return SELKV_ERR_WORKSPACE;
@@ -399,6 +406,7 @@ selkv_status selkv_score(const selkv_shape* shape, const int32_t* n_len, const v
   a.flags = at<uint32_t>(workspace, 0);
   a.seq_n = at<int32_t>(workspace, plan.seq_n);
   a.seq_m = at<int32_t>(workspace, plan.seq_m);
+  a.seq_t1 = at<int32_t>(workspace, plan.seq_t1);
   a.rowpart = at<float2>(workspace, plan.rowpart);
   a.rowstat = at<float2>(workspace, plan.rowstat);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
@@ -406,11 +414,11 @@ selkv_status selkv_score(const selkv_shape* shape, const int32_t* n_len, const v
   int kernels = 0;
   if (passes & SELKV_SCORE_ROWSTATS) {  // the column-sum pass reuses the table of its row-statistics call
     e = launch_seq_setup(a, tab, st);
-    kernels += 3;
+    kernels += score_uses_tc(a.dtype, a.D, a.R) ? 2 : 3;
   }
   if (passes & SELKV_SCORE_COLSUMS) kernels += 1;
   if (e == cudaSuccess)
-    e = score_uses_tc(a.dtype, a.D, a.R) ? launch_score_tc(a, st, passes) : launch_score_simt(a, st, passes);
+    e = score_uses_tc(a.dtype, a.D, a.R) ? launch_score_tc(a, tab, st, passes) : launch_score_simt(a, st, passes);
   g_launches += (uint64_t)kernels;
   return e == cudaSuccess ? SELKV_OK : cuda_fail(e);
 }

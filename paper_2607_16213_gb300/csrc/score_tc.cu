@@ -4,8 +4,8 @@
 // (row r = g W + i is query head kv G + g at position p = n_b - W + i, which sees keys j <= p:
 // the causal re-pass of Sec. 3.1).  With s'_rj = log2(e) q_r . k_j / sqrt(d):
 //   pass 1: per row, over a slice of the keys: (max_j s'_rj, sum_j 2^(s'_rj - max)),
-//   (fold)  M_r, Z_r over the slices (rowstat_reduce_kernel),
-//   pass 2: a_j = sum_r 2^(s'_rj - M_r) / (G Z_r) = sum_r 2^(s'_rj - M_r - log2(G Z_r))
+//   pass 2: M_r, Z_r over the slices, then
+//           a_j = sum_r 2^(s'_rj - M_r) / (G Z_r) = sum_r 2^(s'_rj - M_r - log2(G Z_r))
 //           (Eq. 5's a, mean over the group).
 // Both passes are one kernel: a TMA producer warp streams K tiles (and the group's Q once)
 // into shared memory with 128-byte swizzling; one thread issues tcgen05.mma (bf16 in, fp32
@@ -33,6 +33,9 @@ namespace {
 constexpr uint32_t kTmemCols = 512;  // two accumulators of up to 256 fp32 columns
 #ifndef SELKV_P1_KEYS
 #define SELKV_P1_KEYS 256  // pass 1: keys per tile (the MMA's N), a multiple of 32
+#endif
+#ifndef SELKV_NORM_P1
+#define SELKV_NORM_P1 4    // eighths of a sequence's value norms taken in pass 1
 #endif
 #ifndef SELKV_P1_CPW
 #define SELKV_P1_CPW 2     // pass 1: 32-column accumulator chunks per epilogue warp and tile
@@ -66,9 +69,10 @@ __host__ __device__ constexpr int cta_threads(int pass, bool norms) {
 // lanes as a butterfly per value does.  The copies are marked for early eviction from L2.
 constexpr int kNormChunk = 4096;  // bytes per copy
 __host__ __device__ constexpr int norm_ring(int pass) { return norm_warps(pass) * norm_stages(pass) * kNormChunk; }
+// `used` counts the copies this warp has taken from its ring; false after a timed-out wait.
 template <int D, int PASS>
-__device__ __forceinline__ void norm_rows(const __nv_bfloat16* V, float* norm, int row_lo, int row_hi, int w,
-                                          unsigned char* ring, uint64_t* bars, uint32_t* flags) {
+__device__ __forceinline__ bool norm_rows(const __nv_bfloat16* V, float* norm, int row_lo, int row_hi, int w,
+                                          unsigned char* ring, uint64_t* bars, uint32_t* flags, int& used) {
   constexpr int LPR = D / 8, RPL = 32 / LPR, kGroups = kNormChunk / 512;  // lanes per row, rows per group of lanes
   constexpr int kNormStages = norm_stages(PASS), nw = norm_warps(PASS);
   constexpr int kRows = RPL * kGroups;                     // rows per chunk
@@ -80,7 +84,7 @@ __device__ __forceinline__ void norm_rows(const __nv_bfloat16* V, float* norm, i
   const int chunks = first < row_hi ? (row_hi - first + stride - 1) / stride : 0;
   const uint64_t pol = l2_evict_first_policy();
   auto load = [&](int c) {
-    const int r0 = first + c * stride, st = c % kNormStages;
+    const int r0 = first + c * stride, st = (used + c) % kNormStages;
     const uint32_t bytes = (uint32_t)min(kRows, row_hi - r0) * D * 2;
     mbar_arrive_expect_tx(&bars[st], bytes);
     bulk_load_hint(ring + st * kNormChunk, V + (size_t)r0 * D, bytes, &bars[st], pol);
@@ -88,14 +92,14 @@ __device__ __forceinline__ void norm_rows(const __nv_bfloat16* V, float* norm, i
   if (lane == 0)
     for (int c = 0; c < min(chunks, kNormStages); ++c) load(c);
   for (int c = 0; c < chunks; ++c) {
-    const int st = c % kNormStages, r0 = first + c * stride;
-    if (!__all_sync(0xffffffffu, mbar_wait(&bars[st], (c / kNormStages) & 1))) {
+    const int st = (used + c) % kNormStages, r0 = first + c * stride;
+    if (!__all_sync(0xffffffffu, mbar_wait(&bars[st], ((used + c) / kNormStages) & 1))) {
       if (lane == 0) {
         raise_flag(flags, SELKV_DEVERR_TIMEOUT);
         for (int k = c; k < min(chunks, c + kNormStages); ++k)  // (bounded) let the copies in flight land
-          mbar_wait(&bars[k % kNormStages], (k / kNormStages) & 1);
+          mbar_wait(&bars[(used + k) % kNormStages], ((used + k) / kNormStages) & 1);
       }
-      return;
+      return false;
     }
     const uint4* src = reinterpret_cast<const uint4*>(ring + st * kNormChunk) + lane;
     float q[kGroups];
@@ -134,6 +138,8 @@ __device__ __forceinline__ void norm_rows(const __nv_bfloat16* V, float* norm, i
     const int row = r0 + k0 * RPL + sub;
     if ((lane % (LPR / kGroups)) == 0 && row < row_hi) norm[row] = sqrtf(q[0]);
   }
+  used += chunks;
+  return true;
 }
 
 #ifndef SELKV_P2_PIPE
@@ -190,17 +196,77 @@ struct SCfg {
   static constexpr int kKTile = kKeys * D * 2;           // one K tile
   static constexpr int kQBytes = kRows * D * 2;
   static constexpr int kRing = kStages * kKTile;
-  // barriers | -(M + log2(G Z)) of up to 512 rows | pass 1: [parts][128] float2, pass 2: [2][4][128] float
+  // barriers | -(M + log2(G Z)) and window place of up to 512 rows | pass 1: [parts][128] float2, pass 2: [2][4][128] float
   static constexpr int kHead = 384;  // barriers and flags
-  static constexpr int kMisc = kHead + 256 * 8 + (kP1Parts * 128 * 8 > 4096 ? kP1Parts * 128 * 8 : 4096);
+  static constexpr int kMisc = kHead + 512 * 8 + (kP1Parts * 128 * 8 > 4096 ? kP1Parts * 128 * 8 : 4096);
   static constexpr int kSmem = 1024 + kQBytes + kRing + kMisc + norm_ring(PASS);
   static_assert(kSmem <= 232448, "227 KB of shared memory");
 };
 
+// One CTA's share of a pass: `cnt` consecutive key tiles of the list of all (unit, tile) pairs, in
+// unit order (unit = sequence b, KV head kv), as pieces of one unit each.  Every role of the CTA
+// walks the same pieces.
+struct Walk {
+  int u, t, left;              // the piece's unit and first tile, tiles left from there
+  int b, kv, n, ntiles, nt;    // its sequence, head and length; the unit's tiles; the piece's tiles
+  __device__ __forceinline__ void open(const CompressArgs& a, int keys) {
+    if (left <= 0) return;
+    b = u / a.Hkv;
+    kv = u - b * a.Hkv;
+    n = a.seq_n[b];
+    ntiles = (n + keys - 1) / keys;
+    nt = min(left, ntiles - t);
+  }
+  __device__ __forceinline__ void next(const CompressArgs& a, int keys) {
+    left -= nt;
+    ++u;
+    t = 0;
+    open(a, keys);
+  }
+};
+
+// Fold of pass 1's partials of a unit's row r: -(M + log2(G Z)), the row's whole normaliser as one
+// exponent offset (2^(s' - M) / (G Z) = 2^(s' - (M + log2(G Z)))).  The partials of unit u are
+// those of the pass-1 CTA groups c_first..c_last that held tiles of it, at c + u.
+__device__ __forceinline__ float fold_row_tc(const CompressArgs& a, const Walk& w, int r) {
+  const int T1 = (w.n + SELKV_P1_KEYS - 1) / SELKV_P1_KEYS;
+  int c0, c1;
+  if (a.p1_split > 0) {
+    const int per = (T1 + a.p1_split - 1) / a.p1_split;
+    c0 = w.u * a.p1_split;
+    c1 = c0 + (T1 - 1) / per;
+  } else {
+    const int g = a.seq_t1[w.b] * a.Hkv + w.kv * T1;
+    c0 = g / a.p1_per;
+    c1 = (g + T1 - 1) / a.p1_per;
+  }
+  const float2* part = a.rowpart + ((size_t)c0 + w.u) * a.R + r;
+  const int nch = c1 - c0 + 1;
+  float M = -INFINITY, Z = 0.f;
+  constexpr int kAhead = 8;  // partials loaded together
+  for (int c = 0; c < nch; c += kAhead) {
+    float2 p[kAhead];
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i)
+      p[i] = c + i < nch ? part[(size_t)(c + i) * a.R] : make_float2(-INFINITY, 0.f);
+    float m = M;
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) m = fmaxf(m, p[i].x);
+    if (m == -INFINITY) continue;
+    Z *= exp2f(M - m);
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) Z += p[i].y * exp2f(p[i].x - m);
+    M = m;
+  }
+  const float y = 1.f / ((float)a.G * Z);
+  return y > 0.f ? -(M - log2f(y)) : -INFINITY;
+}
+
 template <int D, int PASS, int HALVES>
 __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
                                                                         const __grid_constant__ CUtensorMap tmK,
-                                                                        CompressArgs a) {
+                                                                        CompressArgs a,
+                                                                        const __grid_constant__ ScoreWalk walk) {
   using C = SCfg<D, PASS, HALVES>;
   constexpr int kEpiWarps = epi_warps(PASS);
   constexpr int kProducerWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1;
@@ -215,8 +281,9 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
   uint64_t* empty = full + kStages;
   uint64_t* tfull = empty + kStages;
   uint64_t* tempty = tfull + 2;
-  uint64_t* qbar = tempty + 2;
-  uint64_t* done = qbar + 1;
+  uint64_t* qbar = tempty + 2;    // the piece's Q is in
+  uint64_t* qfree = qbar + 1;     // the piece's MMAs have read it
+  uint64_t* done = qfree + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   // pass 2: per lane quarter and column-sum buffer, "the other three parts' sums are in" and
@@ -224,30 +291,24 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
   uint64_t* cs_full = reinterpret_cast<uint64_t*>(misc + 128);  // [4][2]
   uint64_t* cs_empty = cs_full + 8;                              // [4][2]
   // the norm warps' copies, and their ring
+  static_assert((2 * kStages + 7) * 8 + 8 <= 128, "barriers and flags before the column sums'");
   constexpr int kNormBars = norm_warps(PASS) * norm_stages(PASS);
   static_assert(kNormBars <= 16, "norm barriers fit");
   uint64_t* nbar = reinterpret_cast<uint64_t*>(misc + 256);
   unsigned char* nring = misc + C::kMisc;
   float* rneg = reinterpret_cast<float*>(misc + C::kHead);               // pass 2: -(M + log2(G Z)) per row
-  float* colpart = reinterpret_cast<float*>(misc + C::kHead + 256 * 8);  // pass 1: [parts][128] float2; pass 2: [2][4][128]
+  int* rwin = reinterpret_cast<int*>(misc + C::kHead + 512 * 4);         // pass 2: r mod W per row, its place in the window
+  float* colpart = reinterpret_cast<float*>(misc + C::kHead + 512 * 8);  // pass 1: [parts][128] float2; pass 2: [2][4][128]
 
-  const int kv = blockIdx.y, b = blockIdx.z;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n = a.seq_n[b];
   const int R = a.R;
   const int Rp = (R + 15) & ~15;              // N of the pass-2 MMAs over all halves
   const int MT = (R + 127) / 128;             // 128-row halves of the R rows
   const int h = PASS == 1 ? (int)blockIdx.x % MT : 0;           // pass 1: this CTA's rows
-  const int split = PASS == 1 ? (int)blockIdx.x / MT : (int)blockIdx.x;
-  const int nsplit = PASS == 1 ? (int)gridDim.x / MT : (int)gridDim.x;
+  const int group = PASS == 1 ? (int)blockIdx.x / MT : (int)blockIdx.x;  // CTAs with the same tiles
   const int Rq = PASS == 1 ? 128 : (HALVES == 2 ? 512 : (R > 128 ? 256 : 128));  // Q rows staged (whole boxes)
-  const int ntiles_all = (n + kKeys - 1) / kKeys;
-  const int per = (ntiles_all + nsplit - 1) / nsplit;
-  const int t_begin = split * per;
-  const int nt = max(0, min(ntiles_all, t_begin + per) - t_begin);
-  const size_t bk = (size_t)b * a.Hkv + kv;
-  const int krow0 = (int)(bk * a.n_cap) + t_begin * kKeys;
-  const int qrow0 = (b * a.Hq + kv * a.G) * a.W + h * 128;
+  Walk w0{walk.u0[group], walk.t0[group], walk.cnt[group], 0, 0, 0, 0, 0};
+  w0.open(a, kKeys);
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) {
@@ -259,6 +320,7 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
       mbar_init(&tempty[i], kEpiWarps);
     }
     mbar_init(qbar, 1);
+    mbar_init(qfree, 1);
     mbar_init(done, 1);
     for (int i = 0; i < kNormBars; ++i) mbar_init(&nbar[i], 1);
     if (PASS == 2) {
@@ -271,74 +333,93 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
     fence_mbar_init();
   }
   if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
-  if (PASS == 2)
-    for (int r = threadIdx.x; r < 256 * HALVES; r += blockDim.x) {
-      // 2^(s' - M) / (G Z) = 2^(s' - (M + log2(G Z))): the normaliser joins the exponent
-      const float2 st = r < R ? a.rowstat[bk * R + r] : make_float2(0.f, 0.f);
-      rneg[r] = st.y > 0.f ? -(st.x - log2f(st.y)) : -INFINITY;
-    }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
   if (warp == kProducerWarp) {
-    if (lane == 0 && nt > 0) {
+    if (lane == 0) {
       prefetch_tensormap(&tmQ);
       prefetch_tensormap(&tmK);
-      mbar_arrive_expect_tx(qbar, C::kBoxes * Rq * 128);
-      for (int bx = 0; bx < C::kBoxes; ++bx)
-        for (int r0 = 0; r0 < Rq; r0 += 128) tma_load_2d(Qs + (bx * Rq + r0) * 128, &tmQ, bx * 64, qrow0 + r0, qbar);
-      int issued = 0;
-      for (int t = 0; t < nt; ++t) {
-        const int st = t % kStages;
-        if (!mbar_wait(&empty[st], ((t / kStages) & 1) ^ 1) || *abort_flag) {
-          *abort_flag = 1;
-          raise_flag(a.flags, SELKV_DEVERR_TIMEOUT);
-          break;
-        }
-        mbar_arrive_expect_tx(&full[st], C::kKTile);
-        for (int bx = 0; bx < C::kBoxes; ++bx)
-          tma_load_2d(Ks + st * C::kKTile + bx * kKeys * 128, &tmK, bx * 64, krow0 + t * kKeys, &full[st]);
-        issued = t + 1;
-      }
-      for (int t = max(0, issued - kStages); t < issued; ++t) mbar_wait(&full[t % kStages], (t / kStages) & 1);
-      mbar_wait(qbar, 0);
-    }
-  } else if (warp == kMmaWarp) {
-    if (lane == 0 && nt > 0) {
-      bool ok = mbar_wait(qbar, 0);
-      const uint32_t qbase = smem_u32(Qs);
-      int u = 0;  // accumulator use: one per (key tile, row half)
-      for (int t = 0; ok && t < nt; ++t) {
-        const int st = t % kStages;
-        if (!mbar_wait(&full[st], (t / kStages) & 1) || *abort_flag) {
-          ok = false;
-          break;
-        }
-        const uint32_t kbase = smem_u32(Ks + st * C::kKTile);
-        for (int ph = 0; ph < HALVES; ++ph, ++u) {
-          const int buf = u & 1;
-          if (!mbar_wait(&tempty[buf], ((u >> 1) & 1) ^ 1) || *abort_flag) {
+      int tt = 0;      // tiles issued, over all pieces
+      int pieces = 0;  // pieces whose Q is issued
+      bool ok = true;
+      for (Walk w = w0; ok && w.left > 0; w.next(a, kKeys)) {
+        const int krow0 = (int)((size_t)w.u * a.n_cap) + w.t * kKeys;
+        const int qrow0 = (w.b * a.Hq + w.kv * a.G) * a.W + h * 128;
+        for (int t = 0; t <= w.nt; ++t) {
+          // Q after the piece's first tile, which can be loaded while the last piece's MMAs still read theirs
+          if (t == 1) {
+            if (pieces > 0) ok = mbar_wait(qfree, (pieces - 1) & 1);
+            if (!ok || *abort_flag) {
+              ok = false;
+              break;
+            }
+            mbar_arrive_expect_tx(qbar, C::kBoxes * Rq * 128);
+            for (int bx = 0; bx < C::kBoxes; ++bx)
+              for (int r0 = 0; r0 < Rq; r0 += 128) tma_load_2d(Qs + (bx * Rq + r0) * 128, &tmQ, bx * 64, qrow0 + r0, qbar);
+            ++pieces;
+          }
+          if (t == w.nt) break;
+          const int st = tt % kStages;
+          if (!mbar_wait(&empty[st], ((tt / kStages) & 1) ^ 1) || *abort_flag) {
             ok = false;
             break;
           }
-          tc_fence_after();
-          const uint32_t idesc = PASS == 1 ? umma_idesc_bf16(128, kKeys) : umma_idesc_bf16(128, min(256, Rp - ph * 256));
-#pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks) {
-            const uint32_t koff = (ks >> 2) * (kKeys * 128) + (ks & 3) * 32;
-            const uint32_t qoff = (ks >> 2) * (Rq * 128) + (ks & 3) * 32 + ph * 256 * 128;
-            if (PASS == 1) {
-              umma_bf16(tmem + buf * 256, umma_desc_sw128(qbase + qoff), umma_desc_sw128(kbase + koff), idesc, ks > 0);
-            } else {
-              umma_bf16(tmem + buf * 256, umma_desc_sw128(kbase + koff), umma_desc_sw128(qbase + qoff), idesc, ks > 0);
-            }
-          }
-          umma_commit(&tfull[buf]);
+          mbar_arrive_expect_tx(&full[st], C::kKTile);
+          for (int bx = 0; bx < C::kBoxes; ++bx)
+            tma_load_2d(Ks + st * C::kKTile + bx * kKeys * 128, &tmK, bx * 64, krow0 + t * kKeys, &full[st]);
+          ++tt;
         }
-        if (!ok) break;
-        umma_commit(&empty[st]);
+      }
+      if (!ok) {
+        *abort_flag = 1;
+        raise_flag(a.flags, SELKV_DEVERR_TIMEOUT);
+      }
+      for (int t = max(0, tt - kStages); t < tt; ++t) mbar_wait(&full[t % kStages], (t / kStages) & 1);
+      if (pieces > 0) mbar_wait(qbar, (pieces - 1) & 1);
+    }
+  } else if (warp == kMmaWarp) {
+    if (lane == 0 && w0.left > 0) {
+      bool ok = true;
+      const uint32_t qbase = smem_u32(Qs);
+      int u = 0;   // accumulator use: one per (key tile, row half)
+      int tt = 0;  // tiles, over all pieces
+      int pieces = 0;
+      for (Walk w = w0; ok && w.left > 0; w.next(a, kKeys), ++pieces) {
+        ok = mbar_wait(qbar, pieces & 1) && !*abort_flag;
+        for (int t = 0; ok && t < w.nt; ++t, ++tt) {
+          const int st = tt % kStages;
+          if (!mbar_wait(&full[st], (tt / kStages) & 1) || *abort_flag) {
+            ok = false;
+            break;
+          }
+          const uint32_t kbase = smem_u32(Ks + st * C::kKTile);
+          for (int ph = 0; ph < HALVES; ++ph, ++u) {
+            const int buf = u & 1;
+            if (!mbar_wait(&tempty[buf], ((u >> 1) & 1) ^ 1) || *abort_flag) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t idesc = PASS == 1 ? umma_idesc_bf16(128, kKeys) : umma_idesc_bf16(128, min(256, Rp - ph * 256));
+#pragma unroll
+            for (int ks = 0; ks < D / 16; ++ks) {
+              const uint32_t koff = (ks >> 2) * (kKeys * 128) + (ks & 3) * 32;
+              const uint32_t qoff = (ks >> 2) * (Rq * 128) + (ks & 3) * 32 + ph * 256 * 128;
+              if (PASS == 1) {
+                umma_bf16(tmem + buf * 256, umma_desc_sw128(qbase + qoff), umma_desc_sw128(kbase + koff), idesc, ks > 0);
+              } else {
+                umma_bf16(tmem + buf * 256, umma_desc_sw128(kbase + koff), umma_desc_sw128(qbase + qoff), idesc, ks > 0);
+              }
+            }
+            umma_commit(&tfull[buf]);
+          }
+          if (!ok) break;
+          umma_commit(&empty[st]);
+        }
+        umma_commit(qfree);
       }
       if (!ok) {
         *abort_flag = 1;
@@ -349,12 +430,20 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
     }
   } else if (warp > kMmaWarp) {
     // ---------------- value norms: this CTA's share of the pass's rows ----------------
-    const int n1 = n / 2;
-    const int lo = PASS == 1 ? 0 : n1, hi = PASS == 1 ? n1 : n;
-    const int share = ((hi - lo + (int)gridDim.x - 1) / (int)gridDim.x + 15) & ~15;
-    const int r_lo = lo + (int)blockIdx.x * share;
-    norm_rows<D, PASS>(static_cast<const __nv_bfloat16*>(a.V) + bk * a.n_cap * D, a.vnorm + bk * a.n_cap, r_lo,
-                 min(hi, r_lo + share), warp - kMmaWarp - 1, nring, nbar, a.flags);
+    // a piece takes the rows of its share of the unit's tiles, pass 1's row halves a part of them each
+    int used = 0;
+    for (Walk w = w0; w.left > 0; w.next(a, kKeys)) {
+      const int n1 = (int)((long long)w.n * SELKV_NORM_P1 / 8);
+      const int lo = PASS == 1 ? 0 : n1, hi = PASS == 1 ? n1 : w.n;
+      auto edge = [&](int t) { return lo + (int)((long long)(hi - lo) * t / w.ntiles); };
+      const int e0 = edge(w.t), len = edge(w.t + w.nt) - e0;
+      const int parts = PASS == 1 ? MT : 1;
+      const size_t row0 = (size_t)w.u * a.n_cap;
+      if (!norm_rows<D, PASS>(static_cast<const __nv_bfloat16*>(a.V) + row0 * D, a.vnorm + row0,
+                              e0 + (int)((long long)len * h / parts), e0 + (int)((long long)len * (h + 1) / parts),
+                              warp - kMmaWarp - 1, nring, nbar, a.flags, used))
+        break;
+    }
   } else {
     // ---------------- epilogue: warps 0-15 ----------------
     const int q = warp & 3, part = warp >> 2;  // lane quarter of TMEM, and which part of the work
@@ -375,127 +464,56 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
     if (PASS == 1) {
       const int r = h * 128 + q * 32 + lane;    // query row owned by this thread
       const bool row_ok = r < R;
-      const int p = n - a.W + (r % a.W);        // its last visible key
-      float m_run = -INFINITY, l_run = 0.f;     // running max (base 2, scaled) and sum
-      for (int t = 0; t < nt; ++t) {
-        const int buf = t & 1;
-        const bool ok = warp_wait(&tfull[buf], (t >> 1) & 1);
-        tc_fence_after();
-        constexpr int kCols = 32 * SELKV_P1_CPW;           // this warp's keys of the tile
-        const int key0 = (t_begin + t) * kKeys + part * kCols;
-        const bool full_quarter = key0 + kCols - 1 <= n - a.W;  // every row sees every key of the part
-        // (pass 1 reads the accumulator 32 columns at a time, each load waited for before its
-        // arithmetic: pipelined loads measured slower here, 16-column ones because the running
-        // max then needs a correction every 16 keys, 32-column ones by half a microsecond)
-        if (ok) {
-#pragma unroll 1
-          for (int c = 0; c < kCols; c += 32) {
-            float v[32];
-            tmem_ld32(tmem + lane_base + buf * 256 + part * kCols + c, v);
-            float cm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-            if (full_quarter && row_ok) {
-#pragma unroll
-              for (int i = 0; i < 32; ++i) cm[i & 3] = fmaxf(cm[i & 3], v[i]);
-            } else {
-#pragma unroll
-              for (int i = 0; i < 32; ++i) {
-                v[i] = (row_ok && key0 + c + i <= p) ? v[i] : -INFINITY;
-                cm[i & 3] = fmaxf(cm[i & 3], v[i]);
-              }
-            }
-            // the scale is positive, so max(v) * scale is the max of the scaled logits
-            const float mn = fmaxf(m_run, fmaxf(fmaxf(cm[0], cm[1]), fmaxf(cm[2], cm[3])) * sc);
-            if (mn != -INFINITY) {
-              // 2^(v sc - mn), pairs packed; sums in four interleaved lanes as (0,1) and (2,3)
-              const uint64_t sc2 = pack_f2(sc, sc), nm2 = pack_f2(-mn, -mn);
-              uint64_t s01 = pack_f2(0.f, 0.f), s23 = s01;
-#pragma unroll
-              for (int i = 0; i < 32; i += 4) {
-                float x0, x1, x2, x3;
-                unpack_f2(ffma2(pack_f2(v[i], v[i + 1]), sc2, nm2), x0, x1);
-                unpack_f2(ffma2(pack_f2(v[i + 2], v[i + 3]), sc2, nm2), x2, x3);
-                s01 = fadd2(s01, pack_f2(ex2_approx(x0), ex2_approx(x1)));
-                s23 = fadd2(s23, pack_f2(ex2_approx(x2), ex2_approx(x3)));
-              }
-              float s0, s1, s2, s3;
-              unpack_f2(s01, s0, s1);
-              unpack_f2(s23, s2, s3);
-              l_run = l_run * ex2_approx(m_run - mn) + ((s0 + s1) + (s2 + s3));
-              m_run = mn;
-            }
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&tempty[buf]);
-      }
-      // fold the key parts of each row in part order (parts 1.. via shared memory)
-      float2* st4 = reinterpret_cast<float2*>(colpart);  // [parts][128]
-      if (part > 0) st4[part * 128 + q * 32 + lane] = make_float2(m_run, l_run);
-      named_bar_sync(1, kEpiWarps * 32);
-      if (part == 0 && row_ok) {
-        float2 o[kP1Parts];
-        o[0] = make_float2(m_run, l_run);
-#pragma unroll
-        for (int k = 1; k < kP1Parts; ++k) o[k] = st4[k * 128 + q * 32 + lane];
-        float M = o[0].x;
-#pragma unroll
-        for (int k = 1; k < kP1Parts; ++k) M = fmaxf(M, o[k].x);
-        float L = 0.f;
-        if (M != -INFINITY) {
-#pragma unroll
-          for (int k = 0; k < kP1Parts; ++k) L += o[k].y * ex2_approx(o[k].x - M);
-        }
-        a.rowpart[(bk * a.nchunks + split) * R + r] = make_float2(M, L);
-      }
-    } else {
-      const int klane = q * 32 + lane;   // key owned by this thread within the tile
-      int u = 0;                         // accumulator use, as counted by the MMA thread
-      for (int t = 0; t < nt; ++t) {
-        const int key0 = (t_begin + t) * kKeys;
-        const int j = key0 + klane;
-        const int jrel = j - (n - a.W);  // > 0: only rows with (r mod W) >= jrel see key j
-        // every key of this warp is seen by every row: the whole tile is unmasked
-        const bool unmasked = key0 + q * 32 + 31 <= n - a.W;
-        float acc = 0.f;
-        for (int ph = 0; ph < HALVES; ++ph, ++u) {
-          const int buf = u & 1;
-          const bool ok = warp_wait(&tfull[buf], (u >> 1) & 1);
+      int tt = 0;  // tiles, over all pieces
+      for (Walk w = w0; w.left > 0; w.next(a, kKeys)) {
+        const int n = w.n, t_begin = w.t, nt = w.nt;
+        const int p = n - a.W + (r % a.W);        // its last visible key
+        float m_run = -INFINITY, l_run = 0.f;     // running max (base 2, scaled) and sum
+        for (int t = 0; t < nt; ++t, ++tt) {
+          const int buf = tt & 1;
+          const bool ok = warp_wait(&tfull[buf], (tt >> 1) & 1);
           tc_fence_after();
-          // this part's 64 rows of the half: accumulator columns from c0, rows from r_lo
-          const int c0 = part * 64, r_lo = ph * 256 + c0, r_hi = min(R, r_lo + 64);
-          const uint32_t tcol = tmem + lane_base + buf * 256 + c0;
-          if (ok && SELKV_P2_PIPE && r_hi - r_lo == 64 && unmasked) {
-            acc += colsum64(tcol, smem_u32(rneg + r_lo), sc);
-          } else if (ok) {
+          constexpr int kCols = 32 * SELKV_P1_CPW;           // this warp's keys of the tile
+          const int key0 = (t_begin + t) * kKeys + part * kCols;
+          const bool full_quarter = key0 + kCols - 1 <= n - a.W;  // every row sees every key of the part
+          // (pass 1 reads the accumulator 32 columns at a time, each load waited for before its
+          // arithmetic: pipelined loads measured slower here, 16-column ones because the running
+          // max then needs a correction every 16 keys, 32-column ones by half a microsecond)
+          if (ok) {
 #pragma unroll 1
-            for (int c = r_lo; c < r_hi; c += 32) {
+            for (int c = 0; c < kCols; c += 32) {
               float v[32];
-              tmem_ld32(tcol + (c - r_lo), v);
-              const int cnt = min(32, r_hi - c);
-              if (jrel <= 0 && cnt == 32) {
-                // sum over rows of 2^(v sc - M_r - log2(G Z_r)), pairs of rows packed; four
-                // interleaved partial sums as (0,1) and (2,3)
-                const uint64_t sc2 = pack_f2(sc, sc);
-                uint64_t a01 = pack_f2(0.f, 0.f), a23 = a01;
+              tmem_ld32(tmem + lane_base + buf * 256 + part * kCols + c, v);
+              float cm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+              if (full_quarter && row_ok) {
 #pragma unroll
-                for (int i = 0; i < 32; i += 4) {
-                  const float4 nm = *reinterpret_cast<const float4*>(&rneg[c + i]);  // rows c+i .. c+i+3
-                  float x0, x1, x2, x3;
-                  unpack_f2(ffma2(pack_f2(v[i], v[i + 1]), sc2, pack_f2(nm.x, nm.y)), x0, x1);
-                  unpack_f2(ffma2(pack_f2(v[i + 2], v[i + 3]), sc2, pack_f2(nm.z, nm.w)), x2, x3);
-                  a01 = fadd2(a01, pack_f2(ex2_approx(x0), ex2_approx(x1)));
-                  a23 = fadd2(a23, pack_f2(ex2_approx(x2), ex2_approx(x3)));
-                }
-                float s0, s1, s2, s3;
-                unpack_f2(a01, s0, s1);
-                unpack_f2(a23, s2, s3);
-                acc += (s0 + s1) + (s2 + s3);
+                for (int i = 0; i < 32; ++i) cm[i & 3] = fmaxf(cm[i & 3], v[i]);
               } else {
 #pragma unroll
-                for (int i = 0; i < 32; ++i)
-                  if (i < cnt && (jrel <= 0 || (c + i) % a.W >= jrel))
-                    acc += ex2_approx(fmaf(v[i], sc, rneg[c + i]));
+                for (int i = 0; i < 32; ++i) {
+                  v[i] = (row_ok && key0 + c + i <= p) ? v[i] : -INFINITY;
+                  cm[i & 3] = fmaxf(cm[i & 3], v[i]);
+                }
+              }
+              // the scale is positive, so max(v) * scale is the max of the scaled logits
+              const float mn = fmaxf(m_run, fmaxf(fmaxf(cm[0], cm[1]), fmaxf(cm[2], cm[3])) * sc);
+              if (mn != -INFINITY) {
+                // 2^(v sc - mn), pairs packed; sums in four interleaved lanes as (0,1) and (2,3)
+                const uint64_t sc2 = pack_f2(sc, sc), nm2 = pack_f2(-mn, -mn);
+                uint64_t s01 = pack_f2(0.f, 0.f), s23 = s01;
+#pragma unroll
+                for (int i = 0; i < 32; i += 4) {
+                  float x0, x1, x2, x3;
+                  unpack_f2(ffma2(pack_f2(v[i], v[i + 1]), sc2, nm2), x0, x1);
+                  unpack_f2(ffma2(pack_f2(v[i + 2], v[i + 3]), sc2, nm2), x2, x3);
+                  s01 = fadd2(s01, pack_f2(ex2_approx(x0), ex2_approx(x1)));
+                  s23 = fadd2(s23, pack_f2(ex2_approx(x2), ex2_approx(x3)));
+                }
+                float s0, s1, s2, s3;
+                unpack_f2(s01, s0, s1);
+                unpack_f2(s23, s2, s3);
+                l_run = l_run * ex2_approx(m_run - mn) + ((s0 + s1) + (s2 + s3));
+                m_run = mn;
               }
             }
           }
@@ -503,30 +521,127 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
           __syncwarp();
           if (lane == 0) mbar_arrive(&tempty[buf]);
         }
-        // The four row quarters' column sums of key j meet in shared memory (two buffers,
-        // alternating by tile): parts 1-3 leave theirs and go on, part 0 adds them to its own in
-        // quarter order and writes a_j.  A part reuses a buffer only once part 0 has read it.
-        const int cb = t & 1;
-        float* cs = colpart + cb * 512;  // [4][128]
-        uint64_t* cfull = &cs_full[q * 2 + cb];
-        uint64_t* cempty = &cs_empty[q * 2 + cb];
-        // bounded wait of every lane (each lane acquires what it then reads or overwrites)
-        auto lane_wait = [&](uint64_t* bar, uint32_t parity) {
-          if (*abort_flag) return;
-          if (!mbar_wait(bar, parity)) {
-            *abort_flag = 1;
-            raise_flag(a.flags, SELKV_DEVERR_TIMEOUT);
+        // fold the key parts of each row in part order (parts 1.. via shared memory)
+        float2* st4 = reinterpret_cast<float2*>(colpart);  // [parts][128]
+        if (part > 0) st4[part * 128 + q * 32 + lane] = make_float2(m_run, l_run);
+        named_bar_sync(1, kEpiWarps * 32);
+        if (part == 0 && row_ok) {
+          float2 o[kP1Parts];
+          o[0] = make_float2(m_run, l_run);
+#pragma unroll
+          for (int k = 1; k < kP1Parts; ++k) o[k] = st4[k * 128 + q * 32 + lane];
+          float M = o[0].x;
+#pragma unroll
+          for (int k = 1; k < kP1Parts; ++k) M = fmaxf(M, o[k].x);
+          float L = 0.f;
+          if (M != -INFINITY) {
+#pragma unroll
+            for (int k = 0; k < kP1Parts; ++k) L += o[k].y * ex2_approx(o[k].x - M);
           }
-        };
-        if (part > 0) {
-          if (t >= 2) lane_wait(cempty, ((t >> 1) - 1) & 1);
-          cs[part * 128 + klane] = acc;
-          mbar_arrive(cfull);
-        } else {
-          lane_wait(cfull, (t >> 1) & 1);
-          const float sum = ((acc + cs[128 + klane]) + cs[256 + klane]) + cs[384 + klane];
-          mbar_arrive(cempty);
-          if (j < n) a.attn[bk * a.n_cap + j] = sum;
+          a.rowpart[((size_t)group + w.u) * R + r] = make_float2(M, L);
+        }
+        if (w.left > nt) named_bar_sync(1, kEpiWarps * 32);  // the next piece's states replace these
+      }
+    } else {
+      const int klane = q * 32 + lane;   // key owned by this thread within the tile
+      int u = 0;                         // accumulator use, as counted by the MMA thread
+      int tt = 0;                        // tiles, over all pieces
+      for (Walk w = w0; w.left > 0; w.next(a, kKeys)) {
+        const int n = w.n, t_begin = w.t, nt = w.nt;
+        float* attn = a.attn + (size_t)w.u * a.n_cap;
+        static_assert(kEpiWarps * 32 >= 256 * HALVES, "a thread per row");
+        {
+          // (Q of the piece and its first tiles are on their way meanwhile)
+          const int r = threadIdx.x;
+          const float x = r < R ? fold_row_tc(a, w, r) : -INFINITY;
+          if (w.left < w0.left) named_bar_sync(1, kEpiWarps * 32);  // the last piece's rows are done with
+          if (r < 256 * HALVES) {
+            rneg[r] = x;
+            rwin[r] = r % a.W;
+          }
+          named_bar_sync(1, kEpiWarps * 32);
+        }
+        for (int t = 0; t < nt; ++t, ++tt) {
+          const int key0 = (t_begin + t) * kKeys;
+          const int j = key0 + klane;
+          const int jrel = j - (n - a.W);  // > 0: only rows with (r mod W) >= jrel see key j
+          // every key of this warp is seen by every row: the whole tile is unmasked
+          const bool unmasked = key0 + q * 32 + 31 <= n - a.W;
+          float acc = 0.f;
+          for (int ph = 0; ph < HALVES; ++ph, ++u) {
+            const int buf = u & 1;
+            const bool ok = warp_wait(&tfull[buf], (u >> 1) & 1);
+            tc_fence_after();
+            // this part's 64 rows of the half: accumulator columns from c0, rows from r_lo
+            const int c0 = part * 64, r_lo = ph * 256 + c0, r_hi = min(R, r_lo + 64);
+            const uint32_t tcol = tmem + lane_base + buf * 256 + c0;
+            if (ok && SELKV_P2_PIPE && r_hi - r_lo == 64 && unmasked) {
+              acc += colsum64(tcol, smem_u32(rneg + r_lo), sc);
+            } else if (ok) {
+#pragma unroll 1
+              for (int c = r_lo; c < r_hi; c += 32) {
+                float v[32];
+                tmem_ld32(tcol + (c - r_lo), v);
+                const int cnt = min(32, r_hi - c);
+                if (unmasked && cnt == 32) {
+                  // sum over rows of 2^(v sc - M_r - log2(G Z_r)), pairs of rows packed; four
+                  // interleaved partial sums as (0,1) and (2,3)
+                  const uint64_t sc2 = pack_f2(sc, sc);
+                  uint64_t a01 = pack_f2(0.f, 0.f), a23 = a01;
+#pragma unroll
+                  for (int i = 0; i < 32; i += 4) {
+                    const float4 nm = *reinterpret_cast<const float4*>(&rneg[c + i]);  // rows c+i .. c+i+3
+                    float x0, x1, x2, x3;
+                    unpack_f2(ffma2(pack_f2(v[i], v[i + 1]), sc2, pack_f2(nm.x, nm.y)), x0, x1);
+                    unpack_f2(ffma2(pack_f2(v[i + 2], v[i + 3]), sc2, pack_f2(nm.z, nm.w)), x2, x3);
+                    a01 = fadd2(a01, pack_f2(ex2_approx(x0), ex2_approx(x1)));
+                    a23 = fadd2(a23, pack_f2(ex2_approx(x2), ex2_approx(x3)));
+                  }
+                  float s0, s1, s2, s3;
+                  unpack_f2(a01, s0, s1);
+                  unpack_f2(a23, s2, s3);
+                  acc += (s0 + s1) + (s2 + s3);
+                } else {
+                  // the end of a sequence (or rows that do not fill the chunk); the places of the rows
+                  // in the window come from a table (a division per row and key made the last tile
+                  // of a unit cost as much as a dozen others)
+                  float s4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                  for (int i = 0; i < 32; ++i)
+                    if (i < cnt && rwin[c + i] >= jrel) s4[i & 3] += ex2_approx(fmaf(v[i], sc, rneg[c + i]));
+                  acc += (s4[0] + s4[1]) + (s4[2] + s4[3]);
+                }
+              }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&tempty[buf]);
+          }
+          // The four row quarters' column sums of key j meet in shared memory (two buffers,
+          // alternating by tile): parts 1-3 leave theirs and go on, part 0 adds them to its own in
+          // quarter order and writes a_j.  A part reuses a buffer only once part 0 has read it.
+          const int cb = tt & 1;
+          float* cs = colpart + cb * 512;  // [4][128]
+          uint64_t* cfull = &cs_full[q * 2 + cb];
+          uint64_t* cempty = &cs_empty[q * 2 + cb];
+          // bounded wait of every lane (each lane acquires what it then reads or overwrites)
+          auto lane_wait = [&](uint64_t* bar, uint32_t parity) {
+            if (*abort_flag) return;
+            if (!mbar_wait(bar, parity)) {
+              *abort_flag = 1;
+              raise_flag(a.flags, SELKV_DEVERR_TIMEOUT);
+            }
+          };
+          if (part > 0) {
+            if (tt >= 2) lane_wait(cempty, ((tt >> 1) - 1) & 1);
+            cs[part * 128 + klane] = acc;
+            mbar_arrive(cfull);
+          } else {
+            lane_wait(cfull, (tt >> 1) & 1);
+            const float sum = ((acc + cs[128 + klane]) + cs[256 + klane]) + cs[384 + klane];
+            mbar_arrive(cempty);
+            if (j < n) attn[j] = sum;
+          }
         }
       }
     }
@@ -539,18 +654,52 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
   }
 }
 
-// Splits of the keys of one (sequence, KV head): enough CTAs for one per SM, each CTA
-// owning `row_parts` x (a slice of `keys`-key tiles).
-int splits_for(int B, int Hkv, int n_cap, int num_sms, int row_parts, int keys) {
-  const int units = B * Hkv * row_parts;
-  const int tiles = (n_cap + keys - 1) / keys;
-  int s = num_sms / units;
-  if (s > tiles) s = tiles;
-  return s < 1 ? 1 : s;
+// Shares of a pass's key tiles: `groups` CTAs (of `row_parts` each in pass 1) with the same number of
+// consecutive tiles of all units, which crosses from one unit to the next; or, where it is no more tiles
+// for the longest unit, every unit cut into the same number of splits, with no crossing.  A fixed grid of
+// splits per unit left SMs idle where the units did not divide them (32 heads: 128 of 152 CTAs) or had
+// unequal lengths (8 ragged prompts of 32k: passes 131 + 146 us, now 100 + 101; 64 of 8k: 233 + 284, now
+// 214 + 232).  A crossing costs a reload of Q while the epilogue works on the two tiles in flight.
+int plan_walk(const CompressArgs& a, const SeqTable& tab, int row_parts, int keys, ScoreWalk& w, int& split, int& per) {
+  const int groups = kPlanSMs / row_parts;
+  const int units = a.B * a.Hkv;
+  auto tiles = [&](int b) { return (tab.n[b] + keys - 1) / keys; };
+  long long total = 0;
+  int longest = 0;
+  for (int b = 0; b < a.B; ++b) {
+    total += (long long)tiles(b) * a.Hkv;
+    longest = tiles(b) > longest ? tiles(b) : longest;
+  }
+  per = (int)((total + groups - 1) / groups);
+  split = units <= groups ? groups / units : 0;
+  if (split > longest) split = longest;
+  if (split > 0 && (longest + split - 1) / split > per) split = 0;
+  int used = 0;
+  if (split > 0) {
+    for (int u = 0; u < units; ++u) {
+      const int T = tiles(u / a.Hkv), p = (T + split - 1) / split;
+      for (int k = 0; k < split; ++k, ++used) {
+        w.u0[used] = u;
+        w.t0[used] = k * p;
+        w.cnt[used] = T - k * p < p ? (T - k * p > 0 ? T - k * p : 0) : p;
+      }
+    }
+  } else {
+    int b = 0;
+    long long before = 0;  // tiles of the sequences before b
+    for (long long g = 0; g < total; g += per, ++used) {
+      while (g >= before + (long long)tiles(b) * a.Hkv) before += (long long)tiles(b++) * a.Hkv;
+      const int T = tiles(b), in = (int)(g - before);
+      w.u0[used] = b * a.Hkv + in / T;
+      w.t0[used] = in % T;
+      w.cnt[used] = (int)(total - g < per ? total - g : per);
+    }
+  }
+  return used;
 }
 
 template <int D, int HALVES>
-cudaError_t launch_tc_t(const CompressArgs& a, cudaStream_t st, int passes) {
+cudaError_t launch_tc_t(CompressArgs a, const SeqTable& tab, cudaStream_t st, int passes) {
   using C1 = SCfg<D, 1>;
   using C2 = SCfg<D, 2, HALVES>;
   CUtensorMap tq, tk1, tk2;
@@ -559,19 +708,21 @@ cudaError_t launch_tc_t(const CompressArgs& a, cudaStream_t st, int passes) {
       !encode_rows_bf16(&tk2, a.K, (uint64_t)a.B * a.Hkv * a.n_cap, D, C2::kKeys))
     return cudaErrorInvalidValue;
   const int MT = (a.R + 127) / 128;
-  const dim3 grid1(a.nchunks * MT, a.Hkv, a.B);
-  const dim3 grid2(splits_for(a.B, a.Hkv, a.n_cap, kPlanSMs, 1, C2::kKeys), a.Hkv, a.B);
+  ScoreWalk w1{}, w2{};
+  int split2, per2;
+  const int groups1 = plan_walk(a, tab, MT, C1::kKeys, w1, a.p1_split, a.p1_per);
+  const int groups2 = plan_walk(a, tab, 1, C2::kKeys, w2, split2, per2);
   auto k1 = score_tc_kernel<D, 1, 1>;
   auto k2 = score_tc_kernel<D, 2, HALVES>;
   cudaError_t e = set_smem_once<score_tc_kernel<D, 1, 1>>(C1::kSmem);
   if (e == cudaSuccess) e = set_smem_once<score_tc_kernel<D, 2, HALVES>>(C2::kSmem);
   if (e != cudaSuccess) return e;
   if (passes & kScoreRowstats) {
-    k1<<<grid1, cta_threads(1, a.V != nullptr), C1::kSmem, st>>>(tq, tk1, a);
-    e = launch_rowstat_reduce(a, st);
+    k1<<<groups1 * MT, cta_threads(1, a.V != nullptr), C1::kSmem, st>>>(tq, tk1, a, w1);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  if (passes & kScoreColsums) k2<<<grid2, cta_threads(2, a.V != nullptr), C2::kSmem, st>>>(tq, tk2, a);
+  if (passes & kScoreColsums) k2<<<groups2, cta_threads(2, a.V != nullptr), C2::kSmem, st>>>(tq, tk2, a, w2);
   return cudaGetLastError();
 }
 
@@ -581,13 +732,15 @@ cudaError_t launch_tc_t(const CompressArgs& a, cudaStream_t st, int passes) {
 // in the column-sum pass); wider groups take the CUDA-core path.
 bool score_uses_tc(int dtype, int D, int R) { return dtype == SELKV_BF16 && (D == 64 || D == 128) && R >= 1 && R <= 512; }
 
-int score_tc_splits(int B, int Hkv, int n_cap, int R, int num_sms) {
-  return splits_for(B, Hkv, n_cap, num_sms, (R + 127) / 128, SCfg<128, 1>::kKeys);
-}
+// Row-statistics partials of pass 1: one per CTA group and unit it holds tiles of, at (group + unit),
+// which is another for every such pair (both only grow along the list of tiles).
+size_t score_tc_partials(int B, int Hkv) { return (size_t)B * Hkv + kPlanSMs; }
 
-cudaError_t launch_score_tc(const CompressArgs& a, cudaStream_t st, int passes) {
-  if (a.R > 256) return a.D == 128 ? launch_tc_t<128, 2>(a, st, passes) : launch_tc_t<64, 2>(a, st, passes);
-  return a.D == 128 ? launch_tc_t<128, 1>(a, st, passes) : launch_tc_t<64, 1>(a, st, passes);
+int score_tc_tiles1(int n) { return (n + SELKV_P1_KEYS - 1) / SELKV_P1_KEYS; }
+
+cudaError_t launch_score_tc(const CompressArgs& a, const SeqTable& tab, cudaStream_t st, int passes) {
+  if (a.R > 256) return a.D == 128 ? launch_tc_t<128, 2>(a, tab, st, passes) : launch_tc_t<64, 2>(a, tab, st, passes);
+  return a.D == 128 ? launch_tc_t<128, 1>(a, tab, st, passes) : launch_tc_t<64, 1>(a, tab, st, passes);
 }
 
 }  // namespace selkv

@@ -133,12 +133,14 @@ __device__ __forceinline__ float warp_max(float v) {
 struct SeqTable {
   int32_t n[SELKV_MAX_BATCH];  // prefill length n_b
   int32_t m[SELKV_MAX_BATCH];  // budget m_b = floor(rho * n_b)
+  int32_t t1[SELKV_MAX_BATCH];  // tensor-core scoring, pass 1: key tiles of the sequences before b (one KV head)
 };
 
 struct CompressArgs {
   int dtype, B, Hq, Hkv, G, D, W, n_cap, m_cap;
   int R;          // observation rows per KV head: G * W
   int nchunks;    // column chunks of the row-statistics pass
+  int p1_split, p1_per;  // tensor-core scoring: how pass 1 cut the tiles (splits per unit, or 0 and tiles per CTA)
   int row_chunk;  // columns of a chunk (CUDA-core scoring)
   float alpha;
   int pool_kernel, bucket, recent, gate_mode, empty_bucket;
@@ -167,7 +169,8 @@ struct CompressArgs {
   uint32_t* flags;
   int32_t* seq_n;
   int32_t* seq_m;
-  float2* rowpart;   // [B][Hkv][nchunks][R] (max, sum) of 2^(s' - max) per column chunk
+  int32_t* seq_t1;   // [B] SeqTable::t1
+  float2* rowpart;   // (max, sum) of 2^(s' - max): [B][Hkv][nchunks][R] per column chunk; tensor cores: [pieces][R]
   float2* rowstat;   // [B][Hkv][R] (M, 1 / (G * Z))
   float* attn;       // [B][Hkv][n_cap]
   float* vnorm;      // [B][Hkv][n_cap]
@@ -204,6 +207,12 @@ struct CompressArgs {
 // not depend on which device answers (GB300: 152 SMs).
 constexpr int kPlanSMs = 152;
 
+// Where each CTA (group) of a tensor-core scoring pass starts in the list of (unit, key tile) pairs,
+// and how many tiles it takes.
+struct ScoreWalk {
+  int32_t u0[kPlanSMs], t0[kPlanSMs], cnt[kPlanSMs];
+};
+
 // Selection unit of (b, kv): the sequence in the shared mode, the KV head in the per-head mode.
 __host__ __device__ __forceinline__ size_t sel_unit(const CompressArgs& a, int b, int kv) {
   return a.per_head ? (size_t)b * a.Hkv + kv : (size_t)b;
@@ -237,10 +246,11 @@ cudaError_t launch_select_grid(const CompressArgs& a, const SelectWs& w, cudaStr
 
 // Scoring: tensor-core path for bf16 with G W <= 256 rows, CUDA-core path otherwise.
 bool score_uses_tc(int dtype, int D, int R);
-int score_tc_splits(int B, int Hkv, int n_cap, int R, int num_sms);  // pass-1 key splits
-// passes: bit 0 = row statistics (pass 1 and their fold), bit 1 = column sums (pass 2)
+size_t score_tc_partials(int B, int Hkv);  // rows of R partials that pass 1 leaves
+int score_tc_tiles1(int n);                // pass-1 key tiles of n keys
+// passes: bit 0 = row statistics (pass 1; on CUDA cores also their fold), bit 1 = column sums (pass 2)
 constexpr int kScoreRowstats = 1, kScoreColsums = 2, kScoreAll = 3;
-cudaError_t launch_score_tc(const CompressArgs& a, cudaStream_t s, int passes = kScoreAll);
+cudaError_t launch_score_tc(const CompressArgs& a, const SeqTable& tab, cudaStream_t s, int passes = kScoreAll);
 cudaError_t launch_score_simt(const CompressArgs& a, cudaStream_t s, int passes = kScoreAll);
 cudaError_t launch_seq_setup(const CompressArgs& a, const SeqTable& tab, cudaStream_t s);
 cudaError_t launch_rowstat_reduce(const CompressArgs& a, cudaStream_t s);

@@ -12,9 +12,9 @@
 // accumulate, N = 256 so each instruction carries a full-width product) into one of two
 // tensor-memory accumulators; sixteen epilogue warps (four per scheduler) read the
 // accumulator with tcgen05.ld and reduce it while the next tile is multiplied.  Pass 1 puts
-// 128 query rows in the accumulator lanes (M = 128) and 256 keys in its columns, so a CTA
-// owns one half of the R rows; an epilogue thread owns a row and a quarter of each tile's
-// keys, and the four quarter states of a row are folded at the end.  Pass 2 puts 128 keys in
+// 128 query rows in the accumulator lanes (M = 128) and 256 keys in its columns; a CTA owns 128
+// rows, or two such halves in turn on the same keys; an epilogue thread owns a row (of each half) and
+// a quarter of each tile's keys, and the four quarter states of a row are folded at the end.  Pass 2 puts 128 keys in
 // the lanes and the R rows in the columns; an epilogue thread owns a key and a quarter of the
 // rows, and the four quarters' column sums of a key are added in shared memory in a fixed
 // order before a_j is written.
@@ -23,6 +23,8 @@
 // protocol of its epilogue warps, lets issued copies and MMAs finish (bounded) and frees its
 // tensor memory before leaving.
 #include <cudaTypedefs.h>
+
+#include <type_traits>
 
 #include "ptx.cuh"
 #include "selkv_internal.cuh"
@@ -33,9 +35,6 @@ namespace {
 constexpr uint32_t kTmemCols = 512;  // two accumulators of up to 256 fp32 columns
 #ifndef SELKV_P1_KEYS
 #define SELKV_P1_KEYS 256  // pass 1: keys per tile (the MMA's N), a multiple of 32
-#endif
-#ifndef SELKV_NORM_P1
-#define SELKV_NORM_P1 4    // eighths of a sequence's value norms taken in pass 1
 #endif
 #ifndef SELKV_P1_CPW
 #define SELKV_P1_CPW 2     // pass 1: 32-column accumulator chunks per epilogue warp and tile
@@ -52,15 +51,15 @@ static_assert(kP1Parts * 32 * SELKV_P1_CPW == SELKV_P1_KEYS && kP1Parts >= 1, "p
 // 50 + 51 us become 62 + 56 us.  All rows in pass 1 make it wait for HBM (73 + 51 us).  Pass 2
 // has shared memory for three warps of two copies in flight, which bounds its share (three
 // quarters of the rows there: 57 + 72 us with two warps).
-__host__ __device__ constexpr int norm_warps(int pass) { return pass == 1 ? 4 : 3; }
-__host__ __device__ constexpr int norm_stages(int pass) { return pass == 1 ? 3 : 2; }
-static_assert(4 * kP1Parts + 2 + norm_warps(1) <= 32 && SELKV_P1_KEYS <= 256, "pass-1 warps per CTA");
+__host__ __device__ constexpr int norm_warps(int pass, int halves) { return pass == 1 && halves == 1 ? 4 : 3; }
+__host__ __device__ constexpr int norm_stages(int pass, int halves) { return pass == 1 && halves == 1 ? 3 : 2; }
+static_assert(4 * kP1Parts + 2 + norm_warps(1, 1) <= 32 && SELKV_P1_KEYS <= 256, "pass-1 warps per CTA");
 __host__ __device__ constexpr int epi_warps(int pass) { return pass == 1 ? 4 * kP1Parts : 16; }
-__host__ __device__ constexpr int cta_threads(int pass, bool norms) {
-  return (epi_warps(pass) + 2 + (norms ? norm_warps(pass) : 0)) * 32;
+__host__ __device__ constexpr int cta_threads(int pass, int halves, bool norms) {
+  return (epi_warps(pass) + 2 + (norms ? norm_warps(pass, halves) : 0)) * 32;
 }
 
-// Value norms of rows [row_lo, row_hi) by warp `w` of norm_warps(PASS).  The rows of a (sequence,
+// Value norms of rows [row_lo, row_hi) by warp `w` of norm_warps.  The rows of a (sequence,
 // KV head) are contiguous, so lane 0 streams them as 4 KB bulk copies into the warp's own ring
 // (bytes in flight cost no registers; with 4 KB in registers per warp the round trips of eight
 // warps made pass 1 277 us for 64 x 8k where this takes 235).  D / 8 lanes take a row, 16 bytes a
@@ -68,13 +67,15 @@ __host__ __device__ constexpr int cta_threads(int pass, bool norms) {
 // sums of a chunk's 8 row groups share it (each level keeps half of the values), pairing the
 // lanes as a butterfly per value does.  The copies are marked for early eviction from L2.
 constexpr int kNormChunk = 4096;  // bytes per copy
-__host__ __device__ constexpr int norm_ring(int pass) { return norm_warps(pass) * norm_stages(pass) * kNormChunk; }
+__host__ __device__ constexpr int norm_ring(int pass, int halves) {
+  return norm_warps(pass, halves) * norm_stages(pass, halves) * kNormChunk;
+}
 // `used` counts the copies this warp has taken from its ring; false after a timed-out wait.
-template <int D, int PASS>
+template <int D, int PASS, int HALVES>
 __device__ __forceinline__ bool norm_rows(const __nv_bfloat16* V, float* norm, int row_lo, int row_hi, int w,
                                           unsigned char* ring, uint64_t* bars, uint32_t* flags, int& used) {
   constexpr int LPR = D / 8, RPL = 32 / LPR, kGroups = kNormChunk / 512;  // lanes per row, rows per group of lanes
-  constexpr int kNormStages = norm_stages(PASS), nw = norm_warps(PASS);
+  constexpr int kNormStages = norm_stages(PASS, HALVES), nw = norm_warps(PASS, HALVES);
   constexpr int kRows = RPL * kGroups;                     // rows per chunk
   static_assert(kRows * D * 2 == kNormChunk, "a chunk is whole rows");
   const int lane = threadIdx.x & 31, sub = lane / LPR;
@@ -191,15 +192,15 @@ template <int D, int PASS, int HALVES = 1>
 struct SCfg {
   static constexpr int kKeys = PASS == 1 ? SELKV_P1_KEYS : 128;        // keys per tile
   static constexpr int kStages = PASS == 1 ? 2 : (HALVES == 2 ? 2 : 4);  // K tiles in flight
-  static constexpr int kRows = PASS == 1 ? 128 : 256 * HALVES;          // Q rows staged per CTA
+  static constexpr int kRows = (PASS == 1 ? 128 : 256) * HALVES;        // Q rows staged per CTA
   static constexpr int kBoxes = D / 64;                  // 128-byte-wide boxes per row
   static constexpr int kKTile = kKeys * D * 2;           // one K tile
   static constexpr int kQBytes = kRows * D * 2;
   static constexpr int kRing = kStages * kKTile;
   // barriers | -(M + log2(G Z)) and window place of up to 512 rows | pass 1: [parts][128] float2, pass 2: [2][4][128] float
   static constexpr int kHead = 384;  // barriers and flags
-  static constexpr int kMisc = kHead + 512 * 8 + (kP1Parts * 128 * 8 > 4096 ? kP1Parts * 128 * 8 : 4096);
-  static constexpr int kSmem = 1024 + kQBytes + kRing + kMisc + norm_ring(PASS);
+  static constexpr int kMisc = kHead + (PASS == 1 ? 0 : 512 * 8) + (kP1Parts * 128 * 8 > 4096 ? kP1Parts * 128 * 8 : 4096);
+  static constexpr int kSmem = 1024 + kQBytes + kRing + kMisc + norm_ring(PASS, HALVES);
   static_assert(kSmem <= 232448, "227 KB of shared memory");
 };
 
@@ -262,8 +263,26 @@ __device__ __forceinline__ float fold_row_tc(const CompressArgs& a, const Walk& 
   return y > 0.f ? -(M - log2f(y)) : -INFINITY;
 }
 
+// Pass 1: the sum of 2^(v sc - ref) over a row's 32 keys; pairs packed, four interleaved partial sums.
+__device__ __forceinline__ float rowsum32(const float (&v)[32], float sc, float ref) {
+  const uint64_t sc2 = pack_f2(sc, sc), nm2 = pack_f2(-ref, -ref);
+  uint64_t s01 = pack_f2(0.f, 0.f), s23 = s01;
+#pragma unroll
+  for (int i = 0; i < 32; i += 4) {
+    float x0, x1, x2, x3;
+    unpack_f2(ffma2(pack_f2(v[i], v[i + 1]), sc2, nm2), x0, x1);
+    unpack_f2(ffma2(pack_f2(v[i + 2], v[i + 3]), sc2, nm2), x2, x3);
+    s01 = fadd2(s01, pack_f2(ex2_approx(x0), ex2_approx(x1)));
+    s23 = fadd2(s23, pack_f2(ex2_approx(x2), ex2_approx(x3)));
+  }
+  float s0, s1, s2, s3;
+  unpack_f2(s01, s0, s1);
+  unpack_f2(s23, s2, s3);
+  return (s0 + s1) + (s2 + s3);
+}
+
 template <int D, int PASS, int HALVES>
-__global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
+__global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
                                                                         const __grid_constant__ CUtensorMap tmK,
                                                                         CompressArgs a,
                                                                         const __grid_constant__ ScoreWalk walk) {
@@ -292,21 +311,23 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
   uint64_t* cs_empty = cs_full + 8;                              // [4][2]
   // the norm warps' copies, and their ring
   static_assert((2 * kStages + 7) * 8 + 8 <= 128, "barriers and flags before the column sums'");
-  constexpr int kNormBars = norm_warps(PASS) * norm_stages(PASS);
+  constexpr int kNormBars = norm_warps(PASS, HALVES) * norm_stages(PASS, HALVES);
   static_assert(kNormBars <= 16, "norm barriers fit");
   uint64_t* nbar = reinterpret_cast<uint64_t*>(misc + 256);
   unsigned char* nring = misc + C::kMisc;
   float* rneg = reinterpret_cast<float*>(misc + C::kHead);               // pass 2: -(M + log2(G Z)) per row
   int* rwin = reinterpret_cast<int*>(misc + C::kHead + 512 * 4);         // pass 2: r mod W per row, its place in the window
-  float* colpart = reinterpret_cast<float*>(misc + C::kHead + 512 * 8);  // pass 1: [parts][128] float2; pass 2: [2][4][128]
+  float* colpart = reinterpret_cast<float*>(misc + C::kHead + (PASS == 1 ? 0 : 512 * 8));  // pass 1: [parts][128] float2; pass 2: [2][4][128]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int R = a.R;
   const int Rp = (R + 15) & ~15;              // N of the pass-2 MMAs over all halves
-  const int MT = (R + 127) / 128;             // 128-row halves of the R rows
+  constexpr int kP1Rows = 128 * HALVES;
+  const int MT = (R + kP1Rows - 1) / kP1Rows;  // pass 1: row parts of the R rows, a CTA each
   const int h = PASS == 1 ? (int)blockIdx.x % MT : 0;           // pass 1: this CTA's rows
   const int group = PASS == 1 ? (int)blockIdx.x / MT : (int)blockIdx.x;  // CTAs with the same tiles
-  const int Rq = PASS == 1 ? 128 : (HALVES == 2 ? 512 : (R > 128 ? 256 : 128));  // Q rows staged (whole boxes)
+  const int nph = PASS == 1 ? min(HALVES, (R - h * kP1Rows + 127) / 128) : HALVES;  // row halves in use
+  const int Rq = PASS == 1 ? kP1Rows : (HALVES == 2 ? 512 : (R > 128 ? 256 : 128));  // Q rows staged (whole boxes)
   Walk w0{walk.u0[group], walk.t0[group], walk.cnt[group], 0, 0, 0, 0, 0};
   w0.open(a, kKeys);
 
@@ -347,7 +368,7 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
       bool ok = true;
       for (Walk w = w0; ok && w.left > 0; w.next(a, kKeys)) {
         const int krow0 = (int)((size_t)w.u * a.n_cap) + w.t * kKeys;
-        const int qrow0 = (w.b * a.Hq + w.kv * a.G) * a.W + h * 128;
+        const int qrow0 = (w.b * a.Hq + w.kv * a.G) * a.W + h * kP1Rows;
         for (int t = 0; t <= w.nt; ++t) {
           // Q after the piece's first tile, which can be loaded while the last piece's MMAs still read theirs
           if (t == 1) {
@@ -396,7 +417,7 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
             break;
           }
           const uint32_t kbase = smem_u32(Ks + st * C::kKTile);
-          for (int ph = 0; ph < HALVES; ++ph, ++u) {
+          for (int ph = 0; ph < nph; ++ph, ++u) {
             const int buf = u & 1;
             if (!mbar_wait(&tempty[buf], ((u >> 1) & 1) ^ 1) || *abort_flag) {
               ok = false;
@@ -407,7 +428,7 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks) {
               const uint32_t koff = (ks >> 2) * (kKeys * 128) + (ks & 3) * 32;
-              const uint32_t qoff = (ks >> 2) * (Rq * 128) + (ks & 3) * 32 + ph * 256 * 128;
+              const uint32_t qoff = (ks >> 2) * (Rq * 128) + (ks & 3) * 32 + ph * (PASS == 1 ? 128 : 256) * 128;
               if (PASS == 1) {
                 umma_bf16(tmem + buf * 256, umma_desc_sw128(qbase + qoff), umma_desc_sw128(kbase + koff), idesc, ks > 0);
               } else {
@@ -433,13 +454,13 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
     // a piece takes the rows of its share of the unit's tiles, pass 1's row halves a part of them each
     int used = 0;
     for (Walk w = w0; w.left > 0; w.next(a, kKeys)) {
-      const int n1 = (int)((long long)w.n * SELKV_NORM_P1 / 8);
+      const int n1 = w.n / 2;
       const int lo = PASS == 1 ? 0 : n1, hi = PASS == 1 ? n1 : w.n;
       auto edge = [&](int t) { return lo + (int)((long long)(hi - lo) * t / w.ntiles); };
       const int e0 = edge(w.t), len = edge(w.t + w.nt) - e0;
       const int parts = PASS == 1 ? MT : 1;
       const size_t row0 = (size_t)w.u * a.n_cap;
-      if (!norm_rows<D, PASS>(static_cast<const __nv_bfloat16*>(a.V) + row0 * D, a.vnorm + row0,
+      if (!norm_rows<D, PASS, HALVES>(static_cast<const __nv_bfloat16*>(a.V) + row0 * D, a.vnorm + row0,
                               e0 + (int)((long long)len * h / parts), e0 + (int)((long long)len * (h + 1) / parts),
                               warp - kMmaWarp - 1, nring, nbar, a.flags, used))
         break;
@@ -462,83 +483,87 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
       return __shfl_sync(0xffffffffu, ok, 0) != 0;
     };
     if (PASS == 1) {
-      const int r = h * 128 + q * 32 + lane;    // query row owned by this thread
-      const bool row_ok = r < R;
-      int tt = 0;  // tiles, over all pieces
+      int u = 0;  // accumulator use, as counted by the MMA thread
       for (Walk w = w0; w.left > 0; w.next(a, kKeys)) {
         const int n = w.n, t_begin = w.t, nt = w.nt;
-        const int p = n - a.W + (r % a.W);        // its last visible key
-        float m_run = -INFINITY, l_run = 0.f;     // running max (base 2, scaled) and sum
-        for (int t = 0; t < nt; ++t, ++tt) {
-          const int buf = tt & 1;
-          const bool ok = warp_wait(&tfull[buf], (tt >> 1) & 1);
-          tc_fence_after();
+        // this thread's query row in each half, its last visible key, and its running max (base 2,
+        // scaled) and sum
+        int r[HALVES], p[HALVES];
+        float m_run[HALVES], l_run[HALVES];
+#pragma unroll
+        for (int ph = 0; ph < HALVES; ++ph) {
+          r[ph] = h * kP1Rows + ph * 128 + q * 32 + lane;
+          p[ph] = n - a.W + (r[ph] % a.W);
+          m_run[ph] = -INFINITY;
+          l_run[ph] = 0.f;
+        }
+        for (int t = 0; t < nt; ++t) {
           constexpr int kCols = 32 * SELKV_P1_CPW;           // this warp's keys of the tile
           const int key0 = (t_begin + t) * kKeys + part * kCols;
           const bool full_quarter = key0 + kCols - 1 <= n - a.W;  // every row sees every key of the part
-          // (pass 1 reads the accumulator 32 columns at a time, each load waited for before its
-          // arithmetic: pipelined loads measured slower here, 16-column ones because the running
-          // max then needs a correction every 16 keys, 32-column ones by half a microsecond)
-          if (ok) {
+#pragma unroll
+          for (int ph = 0; ph < HALVES; ++ph) {
+            if (ph >= nph) break;
+            const int buf = u & 1;
+            const bool ok = warp_wait(&tfull[buf], (u >> 1) & 1);
+            ++u;
+            tc_fence_after();
+            // (pass 1 reads the accumulator 32 columns at a time, each load waited for before its
+            // arithmetic: pipelined loads measured slower here, and leaving the max out of the chunks where
+            // the last one still serves as a reference changed nothing)
+            if (ok) {
 #pragma unroll 1
-            for (int c = 0; c < kCols; c += 32) {
-              float v[32];
-              tmem_ld32(tmem + lane_base + buf * 256 + part * kCols + c, v);
-              float cm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-              if (full_quarter && row_ok) {
+              for (int c = 0; c < kCols; c += 32) {
+                float v[32];
+                tmem_ld32(tmem + lane_base + buf * 256 + part * kCols + c, v);
+                float cm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                if (full_quarter) {
 #pragma unroll
-                for (int i = 0; i < 32; ++i) cm[i & 3] = fmaxf(cm[i & 3], v[i]);
-              } else {
+                  for (int i = 0; i < 32; ++i) cm[i & 3] = fmaxf(cm[i & 3], v[i]);
+                } else {
 #pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                  v[i] = (row_ok && key0 + c + i <= p) ? v[i] : -INFINITY;
-                  cm[i & 3] = fmaxf(cm[i & 3], v[i]);
+                  for (int i = 0; i < 32; ++i) {
+                    v[i] = key0 + c + i <= p[ph] ? v[i] : -INFINITY;
+                    cm[i & 3] = fmaxf(cm[i & 3], v[i]);
+                  }
                 }
-              }
-              // the scale is positive, so max(v) * scale is the max of the scaled logits
-              const float mn = fmaxf(m_run, fmaxf(fmaxf(cm[0], cm[1]), fmaxf(cm[2], cm[3])) * sc);
-              if (mn != -INFINITY) {
-                // 2^(v sc - mn), pairs packed; sums in four interleaved lanes as (0,1) and (2,3)
-                const uint64_t sc2 = pack_f2(sc, sc), nm2 = pack_f2(-mn, -mn);
-                uint64_t s01 = pack_f2(0.f, 0.f), s23 = s01;
-#pragma unroll
-                for (int i = 0; i < 32; i += 4) {
-                  float x0, x1, x2, x3;
-                  unpack_f2(ffma2(pack_f2(v[i], v[i + 1]), sc2, nm2), x0, x1);
-                  unpack_f2(ffma2(pack_f2(v[i + 2], v[i + 3]), sc2, nm2), x2, x3);
-                  s01 = fadd2(s01, pack_f2(ex2_approx(x0), ex2_approx(x1)));
-                  s23 = fadd2(s23, pack_f2(ex2_approx(x2), ex2_approx(x3)));
+                // the scale is positive, so max(v) * scale is the max of the scaled logits
+                const float mn = fmaxf(m_run[ph], fmaxf(fmaxf(cm[0], cm[1]), fmaxf(cm[2], cm[3])) * sc);
+                if (mn != -INFINITY) {
+                  const float s = rowsum32(v, sc, mn);
+                  l_run[ph] = l_run[ph] * ex2_approx(m_run[ph] - mn) + s;
+                  m_run[ph] = mn;
                 }
-                float s0, s1, s2, s3;
-                unpack_f2(s01, s0, s1);
-                unpack_f2(s23, s2, s3);
-                l_run = l_run * ex2_approx(m_run - mn) + ((s0 + s1) + (s2 + s3));
-                m_run = mn;
               }
             }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&tempty[buf]);
           }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&tempty[buf]);
         }
         // fold the key parts of each row in part order (parts 1.. via shared memory)
         float2* st4 = reinterpret_cast<float2*>(colpart);  // [parts][128]
-        if (part > 0) st4[part * 128 + q * 32 + lane] = make_float2(m_run, l_run);
-        named_bar_sync(1, kEpiWarps * 32);
-        if (part == 0 && row_ok) {
-          float2 o[kP1Parts];
-          o[0] = make_float2(m_run, l_run);
 #pragma unroll
-          for (int k = 1; k < kP1Parts; ++k) o[k] = st4[k * 128 + q * 32 + lane];
-          float M = o[0].x;
+        for (int ph = 0; ph < HALVES; ++ph) {
+          if (ph >= nph) break;
+          if (ph > 0) named_bar_sync(1, kEpiWarps * 32);  // the first half's states are read
+          if (part > 0) st4[part * 128 + q * 32 + lane] = make_float2(m_run[ph], l_run[ph]);
+          named_bar_sync(1, kEpiWarps * 32);
+          if (part == 0 && r[ph] < R) {
+            float2 o[kP1Parts];
+            o[0] = make_float2(m_run[ph], l_run[ph]);
 #pragma unroll
-          for (int k = 1; k < kP1Parts; ++k) M = fmaxf(M, o[k].x);
-          float L = 0.f;
-          if (M != -INFINITY) {
+            for (int k = 1; k < kP1Parts; ++k) o[k] = st4[k * 128 + q * 32 + lane];
+            float M = o[0].x;
 #pragma unroll
-            for (int k = 0; k < kP1Parts; ++k) L += o[k].y * ex2_approx(o[k].x - M);
+            for (int k = 1; k < kP1Parts; ++k) M = fmaxf(M, o[k].x);
+            float L = 0.f;
+            if (M != -INFINITY) {
+#pragma unroll
+              for (int k = 0; k < kP1Parts; ++k) L += o[k].y * ex2_approx(o[k].x - M);
+            }
+            a.rowpart[((size_t)group + w.u) * R + r[ph]] = make_float2(M, L);
           }
-          a.rowpart[((size_t)group + w.u) * R + r] = make_float2(M, L);
         }
         if (w.left > nt) named_bar_sync(1, kEpiWarps * 32);  // the next piece's states replace these
       }
@@ -658,8 +683,8 @@ __global__ __launch_bounds__(cta_threads(PASS, true), 1) void score_tc_kernel(co
 // consecutive tiles of all units, which crosses from one unit to the next; or, where it is no more tiles
 // for the longest unit, every unit cut into the same number of splits, with no crossing.  A fixed grid of
 // splits per unit left SMs idle where the units did not divide them (32 heads: 128 of 152 CTAs) or had
-// unequal lengths (8 ragged prompts of 32k: passes 131 + 146 us, now 100 + 101; 64 of 8k: 233 + 284, now
-// 214 + 232).  A crossing costs a reload of Q while the epilogue works on the two tiles in flight.
+// unequal lengths (8 ragged prompts of 32k: passes 131 + 146 us, now 91 + 101; 64 of 8k: 233 + 284, now
+// 195 + 229).  A crossing costs a reload of Q while the epilogue works on the two tiles in flight.
 int plan_walk(const CompressArgs& a, const SeqTable& tab, int row_parts, int keys, ScoreWalk& w, int& split, int& per) {
   const int groups = kPlanSMs / row_parts;
   const int units = a.B * a.Hkv;
@@ -698,31 +723,31 @@ int plan_walk(const CompressArgs& a, const SeqTable& tab, int row_parts, int key
   return used;
 }
 
-template <int D, int HALVES>
+template <int D, int H1, int H2>
 cudaError_t launch_tc_t(CompressArgs a, const SeqTable& tab, cudaStream_t st, int passes) {
-  using C1 = SCfg<D, 1>;
-  using C2 = SCfg<D, 2, HALVES>;
+  using C1 = SCfg<D, 1, H1>;
+  using C2 = SCfg<D, 2, H2>;
   CUtensorMap tq, tk1, tk2;
   if (!encode_rows_bf16(&tq, a.Q, (uint64_t)a.B * a.Hq * a.W, D, 128) ||
       !encode_rows_bf16(&tk1, a.K, (uint64_t)a.B * a.Hkv * a.n_cap, D, C1::kKeys) ||
       !encode_rows_bf16(&tk2, a.K, (uint64_t)a.B * a.Hkv * a.n_cap, D, C2::kKeys))
     return cudaErrorInvalidValue;
-  const int MT = (a.R + 127) / 128;
+  const int MT = (a.R + 128 * H1 - 1) / (128 * H1);
   ScoreWalk w1{}, w2{};
   int split2, per2;
   const int groups1 = plan_walk(a, tab, MT, C1::kKeys, w1, a.p1_split, a.p1_per);
   const int groups2 = plan_walk(a, tab, 1, C2::kKeys, w2, split2, per2);
-  auto k1 = score_tc_kernel<D, 1, 1>;
-  auto k2 = score_tc_kernel<D, 2, HALVES>;
-  cudaError_t e = set_smem_once<score_tc_kernel<D, 1, 1>>(C1::kSmem);
-  if (e == cudaSuccess) e = set_smem_once<score_tc_kernel<D, 2, HALVES>>(C2::kSmem);
+  auto k1 = score_tc_kernel<D, 1, H1>;
+  auto k2 = score_tc_kernel<D, 2, H2>;
+  cudaError_t e = set_smem_once<score_tc_kernel<D, 1, H1>>(C1::kSmem);
+  if (e == cudaSuccess) e = set_smem_once<score_tc_kernel<D, 2, H2>>(C2::kSmem);
   if (e != cudaSuccess) return e;
   if (passes & kScoreRowstats) {
-    k1<<<groups1 * MT, cta_threads(1, a.V != nullptr), C1::kSmem, st>>>(tq, tk1, a, w1);
+    k1<<<groups1 * MT, cta_threads(1, H1, a.V != nullptr), C1::kSmem, st>>>(tq, tk1, a, w1);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  if (passes & kScoreColsums) k2<<<groups2, cta_threads(2, a.V != nullptr), C2::kSmem, st>>>(tq, tk2, a, w2);
+  if (passes & kScoreColsums) k2<<<groups2, cta_threads(2, H2, a.V != nullptr), C2::kSmem, st>>>(tq, tk2, a, w2);
   return cudaGetLastError();
 }
 
@@ -739,8 +764,24 @@ size_t score_tc_partials(int B, int Hkv) { return (size_t)B * Hkv + kPlanSMs; }
 int score_tc_tiles1(int n) { return (n + SELKV_P1_KEYS - 1) / SELKV_P1_KEYS; }
 
 cudaError_t launch_score_tc(const CompressArgs& a, const SeqTable& tab, cudaStream_t st, int passes) {
-  if (a.R > 256) return a.D == 128 ? launch_tc_t<128, 2>(a, tab, st, passes) : launch_tc_t<64, 2>(a, tab, st, passes);
-  return a.D == 128 ? launch_tc_t<128, 1>(a, tab, st, passes) : launch_tc_t<64, 1>(a, tab, st, passes);
+  // Pass 1 with two 128-row halves per CTA reads a tile's keys once for both, where two CTAs with a half
+  // each read them twice (from L2, or HBM where they drift apart: 8 x 32k 100 -> 90 us, 64 x 8k 215 ->
+  // 197); but a CTA's share is then twice as coarse.  From 8 tiles (16 accumulators) a CTA on, unless
+  // rounding to whole tiles makes it longer (16k: 8 accumulators against 7, 18.9 against 16.4 us).
+  long long total = 0;
+  for (int b = 0; b < a.B; ++b) total += (long long)score_tc_tiles1(tab.n[b]) * a.Hkv;
+  auto accs = [&](int halves) {  // accumulators of the longest share
+    const int groups = kPlanSMs / ((a.R + 128 * halves - 1) / (128 * halves));
+    return (total + groups - 1) / groups * halves;
+  };
+  const bool both = a.R > 128 && accs(2) >= 16 && accs(2) <= accs(1);
+  auto go = [&](auto d, auto h2) {
+    constexpr int D = decltype(d)::value, H2 = decltype(h2)::value;
+    return both ? launch_tc_t<D, 2, H2>(a, tab, st, passes) : launch_tc_t<D, 1, H2>(a, tab, st, passes);
+  };
+  using std::integral_constant;
+  if (a.R > 256) return a.D == 128 ? go(integral_constant<int, 128>{}, integral_constant<int, 2>{}) : go(integral_constant<int, 64>{}, integral_constant<int, 2>{});
+  return a.D == 128 ? go(integral_constant<int, 128>{}, integral_constant<int, 1>{}) : go(integral_constant<int, 64>{}, integral_constant<int, 1>{});
 }
 
 }  // namespace selkv

@@ -210,11 +210,11 @@ struct SCfg {
 struct Walk {
   int u, t, left;              // the piece's unit and first tile, tiles left from there
   int b, kv, n, ntiles, nt;    // its sequence, head and length; the unit's tiles; the piece's tiles
-  __device__ __forceinline__ void open(const CompressArgs& a, int keys) {
+  __device__ __forceinline__ void open(const CompressArgs& a, int keys, int len = 0) {
     if (left <= 0) return;
     b = u / a.Hkv;
     kv = u - b * a.Hkv;
-    n = a.seq_n[b];
+    n = len > 0 ? len : a.seq_n[b];
     ntiles = (n + keys - 1) / keys;
     nt = min(left, ntiles - t);
   }
@@ -226,23 +226,33 @@ struct Walk {
   }
 };
 
-// Fold of pass 1's partials of a unit's row r: -(M + log2(G Z)), the row's whole normaliser as one
-// exponent offset (2^(s' - M) / (G Z) = 2^(s' - (M + log2(G Z)))).  The partials of unit u are
-// those of the pass-1 CTA groups c_first..c_last that held tiles of it, at c + u.
-__device__ __forceinline__ float fold_row_tc(const CompressArgs& a, const Walk& w, int r) {
-  const int T1 = (w.n + SELKV_P1_KEYS - 1) / SELKV_P1_KEYS;
+// The partials that pass 1 left of unit u (T1 of its tiles, the first one `before` tiles into the list
+// of all): one from each CTA group that held tiles of it, at first .. first + count - 1.
+struct Partials {
+  int first, count;
+};
+__host__ __device__ __forceinline__ Partials partials_of(int split, int per, int u, int before, int T1) {
   int c0, c1;
-  if (a.p1_split > 0) {
-    const int per = (T1 + a.p1_split - 1) / a.p1_split;
-    c0 = w.u * a.p1_split;
-    c1 = c0 + (T1 - 1) / per;
+  if (split > 0) {
+    const int p = (T1 + split - 1) / split;
+    c0 = u * split;
+    c1 = c0 + (T1 - 1) / p;
   } else {
-    const int g = a.seq_t1[w.b] * a.Hkv + w.kv * T1;
-    c0 = g / a.p1_per;
-    c1 = (g + T1 - 1) / a.p1_per;
+    c0 = before / per;
+    c1 = (before + T1 - 1) / per;
   }
-  const float2* part = a.rowpart + ((size_t)c0 + w.u) * a.R + r;
-  const int nch = c1 - c0 + 1;
+  return {c0 + u, c1 - c0 + 1};
+}
+__device__ __forceinline__ Partials partials_of(const CompressArgs& a, const Walk& w) {
+  const int T1 = (w.n + SELKV_P1_KEYS - 1) / SELKV_P1_KEYS;
+  return partials_of(a.p1_split, a.p1_per, w.u, a.p1_split > 0 ? 0 : a.seq_t1[w.b] * a.Hkv + w.kv * T1, T1);
+}
+
+// Fold of the partials of row r: -(M + log2(G Z)), the row's whole normaliser as one exponent offset
+// (2^(s' - M) / (G Z) = 2^(s' - (M + log2(G Z)))).
+__device__ __forceinline__ float fold_row_tc(const CompressArgs& a, const Partials& ps, int r) {
+  const float2* part = a.rowpart + (size_t)ps.first * a.R + r;
+  const int nch = ps.count;
   float M = -INFINITY, Z = 0.f;
   constexpr int kAhead = 8;  // partials loaded together
   for (int c = 0; c < nch; c += kAhead) {
@@ -329,7 +339,7 @@ __global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_k
   const int nph = PASS == 1 ? min(HALVES, (R - h * kP1Rows + 127) / 128) : HALVES;  // row halves in use
   const int Rq = PASS == 1 ? kP1Rows : (HALVES == 2 ? 512 : (R > 128 ? 256 : 128));  // Q rows staged (whole boxes)
   Walk w0{walk.u0[group], walk.t0[group], walk.cnt[group], 0, 0, 0, 0, 0};
-  w0.open(a, kKeys);
+  w0.open(a, kKeys, walk.n[group]);
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) {
@@ -346,8 +356,8 @@ __global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_k
     for (int i = 0; i < kNormBars; ++i) mbar_init(&nbar[i], 1);
     if (PASS == 2) {
       for (int i = 0; i < 8; ++i) {
-        mbar_init(&cs_full[i], 3 * 32);
-        mbar_init(&cs_empty[i], 32);
+        mbar_init(&cs_full[i], 3);
+        mbar_init(&cs_empty[i], 1);
       }
     }
     *abort_flag = 0;
@@ -578,7 +588,9 @@ __global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_k
         {
           // (Q of the piece and its first tiles are on their way meanwhile)
           const int r = threadIdx.x;
-          const float x = r < R ? fold_row_tc(a, w, r) : -INFINITY;
+          // the first unit's partials from the table: its chain of loads is not hidden by earlier tiles
+          const Partials ps = w.left == w0.left ? Partials{walk.part0[group], walk.parts[group]} : partials_of(a, w);
+          const float x = r < R ? fold_row_tc(a, ps, r) : -INFINITY;
           if (w.left < w0.left) named_bar_sync(1, kEpiWarps * 32);  // the last piece's rows are done with
           if (r < 256 * HALVES) {
             rneg[r] = x;
@@ -660,11 +672,13 @@ __global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_k
           if (part > 0) {
             if (tt >= 2) lane_wait(cempty, ((tt >> 1) - 1) & 1);
             cs[part * 128 + klane] = acc;
-            mbar_arrive(cfull);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(cfull);
           } else {
             lane_wait(cfull, (tt >> 1) & 1);
             const float sum = ((acc + cs[128 + klane]) + cs[256 + klane]) + cs[384 + klane];
-            mbar_arrive(cempty);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(cempty);
             if (j < n) attn[j] = sum;
           }
         }
@@ -683,8 +697,8 @@ __global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_k
 // consecutive tiles of all units, which crosses from one unit to the next; or, where it is no more tiles
 // for the longest unit, every unit cut into the same number of splits, with no crossing.  A fixed grid of
 // splits per unit left SMs idle where the units did not divide them (32 heads: 128 of 152 CTAs) or had
-// unequal lengths (8 ragged prompts of 32k: passes 131 + 146 us, now 91 + 101; 64 of 8k: 233 + 284, now
-// 195 + 229).  A crossing costs a reload of Q while the epilogue works on the two tiles in flight.
+// unequal lengths (8 ragged prompts of 32k: passes 131 + 146 us, now 91 + 96; 64 of 8k: 233 + 284, now
+// 195 + 221).  A crossing costs a reload of Q while the epilogue works on the two tiles in flight.
 int plan_walk(const CompressArgs& a, const SeqTable& tab, int row_parts, int keys, ScoreWalk& w, int& split, int& per) {
   const int groups = kPlanSMs / row_parts;
   const int units = a.B * a.Hkv;
@@ -720,6 +734,16 @@ int plan_walk(const CompressArgs& a, const SeqTable& tab, int row_parts, int key
       w.cnt[used] = (int)(total - g < per ? total - g : per);
     }
   }
+  for (int c = 0; c < used; ++c) {
+    const int b = w.u0[c] / a.Hkv;
+    w.n[c] = tab.n[b];
+    // (pass 2, after pass 1 has been planned)
+    const int T1 = score_tc_tiles1(tab.n[b]);
+    const Partials ps = a.p1_per > 0 ? partials_of(a.p1_split, a.p1_per, w.u0[c], tab.t1[b] * a.Hkv + w.u0[c] % a.Hkv * T1, T1)
+                                     : Partials{0, 0};
+    w.part0[c] = ps.first;
+    w.parts[c] = ps.count;
+  }
   return used;
 }
 
@@ -735,7 +759,10 @@ cudaError_t launch_tc_t(CompressArgs a, const SeqTable& tab, cudaStream_t st, in
   const int MT = (a.R + 128 * H1 - 1) / (128 * H1);
   ScoreWalk w1{}, w2{};
   int split2, per2;
-  const int groups1 = plan_walk(a, tab, MT, C1::kKeys, w1, a.p1_split, a.p1_per);
+  int split1, per1;
+  const int groups1 = plan_walk(a, tab, MT, C1::kKeys, w1, split1, per1);
+  a.p1_split = split1;
+  a.p1_per = per1;
   const int groups2 = plan_walk(a, tab, 1, C2::kKeys, w2, split2, per2);
   auto k1 = score_tc_kernel<D, 1, H1>;
   auto k2 = score_tc_kernel<D, 2, H2>;

@@ -211,6 +211,8 @@ constexpr int kPlanSMs = 152;
 // and how many tiles it takes.
 struct ScoreWalk {
   int32_t u0[kPlanSMs], t0[kPlanSMs], cnt[kPlanSMs];
+  int32_t n[kPlanSMs];                      // length of the first unit's sequence
+  int32_t part0[kPlanSMs], parts[kPlanSMs];  // pass 2: the first unit's partials of pass 1
 };
 
 // Selection unit of (b, kv): the sequence in the shared mode, the KV head in the per-head mode.

@@ -153,13 +153,12 @@ void note_launches(int kernels) { g_launches += (uint64_t)kernels; }
 // head's top-k, then, in the shared mode only, the union and its trim, with the compaction in
 // the last of them); the RoPE tables when repositioning;
 // the routing and merge (bucket: one kernel for bf16 and buckets of 32, else route and merge, plus
-// the kept-row copy unless the merge does it; cosine: the copy and the cosine kernels); the bias,
-// which the one kernel writes itself in the per-head mode.
+// the kept-row copy unless the merge does it; cosine: the copy and the cosine kernels); the bias.
 int compress_kernel_count(const CompressArgs& a) {
   int k = 1 + (score_uses_tc(a.dtype, a.D, a.R) ? 2 : 3);
   k += a.per_head ? 1 : 2;
   if (a.rope != SELKV_ROPE_OFF) k += 1;
-  if (a.use_kmask) return k + 1 + (a.rope != SELKV_ROPE_OFF ? 1 : 0) + (a.per_head ? 0 : 1);
+  if (a.use_kmask) return k + 1 + (a.rope != SELKV_ROPE_OFF ? 1 : 0) + 1;
   if (a.routing == SELKV_ROUTE_COSINE)
     k += 1 + (a.m_cap > 0 ? cosine_kernels(a.dtype, a.D) : 0);
   else

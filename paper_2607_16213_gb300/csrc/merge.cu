@@ -536,17 +536,17 @@ __global__ __launch_bounds__(32, SELKV_MERGE_MINB) void merge_kernel(CompressArg
 
 // bias[b][kv][slot] = alpha * ln(mean over KV heads of R[b][kv][slot])   (Sec. 3.6, GQA);
 // per-head mode: alpha * ln R[b][kv][slot] of each head, no averaging (Sec. 3.6, MHA).  The
-// count variant uses ln(1 + M) of the merge counts M instead of ln R.
+// count variant uses ln(1 + M) of the merge counts M instead of ln R.  Grid (slots, B, KV heads in the
+// per-head mode: 19 us with one thread for all 32 heads of a slot).  Always the call's last kernel: a
+// decode may load rows of K_c and V_c while it runs, so it writes none of them.
 __global__ __launch_bounds__(256) void bias_kernel(CompressArgs a) {
   const int b = blockIdx.y;
   const int slot = blockIdx.x * blockDim.x + threadIdx.x;
   if (slot >= a.seq_m[b]) return;
   const float* src = a.bias_count ? a.mcount : a.ratio;
   if (a.per_head) {
-    for (int kv = 0; kv < a.Hkv; ++kv) {
-      const size_t o = ((size_t)b * a.Hkv + kv) * a.m_cap + slot;
-      a.bias[o] = a.alpha * (a.bias_count ? log1pf(src[o]) : logf(src[o]));
-    }
+    const size_t o = ((size_t)b * a.Hkv + blockIdx.z) * a.m_cap + slot;
+    a.bias[o] = a.alpha * (a.bias_count ? log1pf(src[o]) : logf(src[o]));
     return;
   }
   float s = 0.f;
@@ -554,6 +554,11 @@ __global__ __launch_bounds__(256) void bias_kernel(CompressArgs a) {
   const float mean = s / (float)a.Hkv;
   const float bias = a.alpha * (a.bias_count ? log1pf(mean) : logf(mean));
   for (int kv = 0; kv < a.Hkv; ++kv) a.bias[((size_t)b * a.Hkv + kv) * a.m_cap + slot] = bias;
+}
+
+cudaError_t launch_bias(const CompressArgs& a, cudaStream_t s) {
+  bias_kernel<<<dim3((a.m_cap + 255) / 256, a.B, a.per_head ? a.Hkv : 1), 256, 0, s>>>(a);
+  return cudaGetLastError();
 }
 
 template <typename T, int D>
@@ -587,11 +592,9 @@ cudaError_t launch_merge(const CompressArgs& a, cudaStream_t s) {
       if (a.D == 128) launch_copy_t<__nv_bfloat16, 128>(a, s);
       else launch_copy_t<__nv_bfloat16, 64>(a, s);
     }
-    if (a.m_cap < 1) return cudaErrorInvalidConfiguration;  // no slot to launch for
     const cudaError_t e = launch_merge_mma(a, s);
-    if (e != cudaSuccess || a.per_head) return e;
-    bias_kernel<<<dim3((a.m_cap + 255) / 256, a.B), 256, 0, s>>>(a);
-    return cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return launch_bias(a, s);
   }
   if (a.routing == SELKV_ROUTE_BUCKET)
     route_kernel<<<dim3((a.nbk + kWarpsPerCta - 1) / kWarpsPerCta, a.B), kWarpsPerCta * 32, 0, s>>>(a);
@@ -606,8 +609,7 @@ cudaError_t launch_merge(const CompressArgs& a, cudaStream_t s) {
     const cudaError_t e = launch_route_cosine(a, s);
     if (e != cudaSuccess) return e;
   }
-  bias_kernel<<<dim3((a.m_cap + 255) / 256, a.B), 256, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_bias(a, s);
 }
 
 }  // namespace selkv

@@ -441,12 +441,8 @@ __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_
       const size_t s = (size_t)bk * a.m_cap + slot0 + __popc(below);
       const float ratio = lane == tl && a_tau > 0.f ? tot / a_tau : 1.f;
       const float count = lane == tl ? (float)merged : 0.f;
-      if (a.per_head) {
-        a.bias[s] = a.alpha * (a.bias_count ? log1pf(count) : logf(ratio));
-      } else {
-        a.ratio[s] = ratio;
-        a.mcount[s] = count;
-      }
+      a.ratio[s] = ratio;
+      a.mcount[s] = count;
       if (a.dbg_ratio) a.dbg_ratio[s] = ratio;
       const size_t o = row_base + X * 32 + lane;
       if (a.dbg_target) a.dbg_target[o] = -1;

@@ -30,12 +30,6 @@ __device__ __forceinline__ PartialView partial_view(const DecodeArgs& a) {
   return {a.partial, decode_record_floats(a.G, a.splits, a.D), a.G, a.splits, a.D};
 }
 
-// Griddepcontrol (programmatic dependent launch): a no-op for kernels launched without it.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch_dependents() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // Fold NW warp states (max wm[w*rs+g], sum wl[w*rs+g], output wo[(w*rs+g)*ld+d]) of heads
 // g < G into this split's partial.  An aborted CTA leaves an empty partial.
 template <int NW>

@@ -48,6 +48,7 @@ __device__ __forceinline__ void argmax_lanes(float& v, int& idx) {
 }
 
 __global__ __launch_bounds__(kWarpsPerCta * 32) void route_kernel(CompressArgs a) {
+  chain_begin();
   const int lane = threadIdx.x & 31;
   const int X = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5), b = blockIdx.y;
   const int n = a.seq_n[b], Bs = a.bucket;
@@ -76,6 +77,7 @@ __global__ __launch_bounds__(kWarpsPerCta * 32) void route_kernel(CompressArgs a
 // positions stay accurate to fp32 rounding.
 constexpr int kRopeRowsPerThread = 8;
 __global__ void rope_table_kernel(CompressArgs a) {
+  chain_begin();
   const int half = a.D / 2, rows = a.rope_hi + 256;
   const int groups = (rows + kRopeRowsPerThread - 1) / kRopeRowsPerThread;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -174,6 +176,7 @@ __device__ __forceinline__ uint4 pack16<float>(const float* x) {
 // elements pair with the ones d/2 further on (the pairs (f, f + d/2)).
 template <typename T, int D>
 __global__ __launch_bounds__(256) void copy_kernel(CompressArgs a) {
+  chain_begin();
   constexpr int kPieces = D * (int)sizeof(T) / 16;  // 16-byte pieces per row
   constexpr int kEpp = 16 / (int)sizeof(T);          // elements per piece
   const int b = blockIdx.y;
@@ -348,6 +351,7 @@ template <typename T, int D>
 #define SELKV_MERGE_MINB 32  // one-warp merge CTAs resident per SM (32: the most an SM holds)
 #endif
 __global__ __launch_bounds__(32, SELKV_MERGE_MINB) void merge_kernel(CompressArgs a) {
+  chain_begin();
   constexpr int PER = D / 32;  // elements of a row per lane
   __shared__ unsigned char list[32];
   const int lane = threadIdx.x;
@@ -540,6 +544,7 @@ __global__ __launch_bounds__(32, SELKV_MERGE_MINB) void merge_kernel(CompressArg
 // per-head mode: 19 us with one thread for all 32 heads of a slot).  Always the call's last kernel: a
 // decode may load rows of K_c and V_c while it runs, so it writes none of them.
 __global__ __launch_bounds__(256) void bias_kernel(CompressArgs a) {
+  pdl_wait();
   const int b = blockIdx.y;
   const int slot = blockIdx.x * blockDim.x + threadIdx.x;
   if (slot >= a.seq_m[b]) return;
@@ -557,7 +562,7 @@ __global__ __launch_bounds__(256) void bias_kernel(CompressArgs a) {
 }
 
 cudaError_t launch_bias(const CompressArgs& a, cudaStream_t s) {
-  bias_kernel<<<dim3((a.m_cap + 255) / 256, a.B, a.per_head ? a.Hkv : 1), 256, 0, s>>>(a);
+  launch_chained(bias_kernel, dim3((a.m_cap + 255) / 256, a.B, a.per_head ? a.Hkv : 1), 256, 0, s, a);
   return cudaGetLastError();
 }
 
@@ -565,14 +570,14 @@ template <typename T, int D>
 void launch_copy_t(const CompressArgs& a, cudaStream_t s) {
   constexpr int kPieces = D * (int)sizeof(T) / 16;
   const size_t copy_threads = (size_t)a.Hkv * a.m_cap * 2 * kPieces;
-  copy_kernel<T, D><<<dim3((unsigned)((copy_threads + 255) / 256), a.B), 256, 0, s>>>(a);
+  launch_chained(copy_kernel<T, D>, dim3((unsigned)((copy_threads + 255) / 256), a.B), 256, 0, s, a);
 }
 
 template <typename T, int D>
 void launch_merge_t(const CompressArgs& a, cudaStream_t s) {
   // with the bucket routing and no repositioning the merge warps copy the kept rows themselves
   if (!merge_copies_kept_rows(a)) launch_copy_t<T, D>(a, s);
-  if (a.routing == SELKV_ROUTE_BUCKET) merge_kernel<T, D><<<dim3(a.nbk, a.B * a.Hkv), 32, 0, s>>>(a);
+  if (a.routing == SELKV_ROUTE_BUCKET) launch_chained(merge_kernel<T, D>, dim3(a.nbk, a.B * a.Hkv), 32, 0, s, a);
 }
 
 }  // namespace
@@ -585,7 +590,7 @@ cudaError_t launch_merge(const CompressArgs& a, cudaStream_t s) {
   if (a.rope != SELKV_ROPE_OFF) {
     const int groups = (a.rope_hi + 256 + kRopeRowsPerThread - 1) / kRopeRowsPerThread;
     const int threads = a.D / 2 * groups;
-    rope_table_kernel<<<(threads + 127) / 128, 128, 0, s>>>(a);
+    launch_chained(rope_table_kernel, (threads + 127) / 128, 128, 0, s, a);
   }
   if (a.use_kmask) {
     if (a.rope != SELKV_ROPE_OFF) {
@@ -597,7 +602,7 @@ cudaError_t launch_merge(const CompressArgs& a, cudaStream_t s) {
     return launch_bias(a, s);
   }
   if (a.routing == SELKV_ROUTE_BUCKET)
-    route_kernel<<<dim3((a.nbk + kWarpsPerCta - 1) / kWarpsPerCta, a.B), kWarpsPerCta * 32, 0, s>>>(a);
+    launch_chained(route_kernel, dim3((a.nbk + kWarpsPerCta - 1) / kWarpsPerCta, a.B), kWarpsPerCta * 32, 0, s, a);
   if (a.dtype == SELKV_BF16) {
     if (a.D == 128) launch_merge_t<__nv_bfloat16, 128>(a, s);
     else launch_merge_t<__nv_bfloat16, 64>(a, s);

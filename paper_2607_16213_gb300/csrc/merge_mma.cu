@@ -132,6 +132,7 @@ __device__ __forceinline__ void copy_keys(const CompressArgs& a, int bk, size_t 
 template <int D>
 __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_constant__ CUtensorMap tmV,
                                                                   CompressArgs a, int seg, int walks) {
+  chain_begin();
   using C = MCfg<D>;
   using bf16 = __nv_bfloat16;
   constexpr int PER = D / 32;        // elements of a row per lane
@@ -491,7 +492,7 @@ cudaError_t launch_t(const CompressArgs& a, cudaStream_t s) {
   const int walks = (nb + seg - 1) / seg;
   // with repositioning copy_kernel writes the keys
   const int keys = a.rope == SELKV_ROPE_OFF ? (a.m_cap + kKeySlots - 1) / kKeySlots : 0;
-  merge_mma_kernel<D><<<dim3(walks + keys, units), 32, MCfg<D>::kSmem, s>>>(tv, a, seg, walks);
+  launch_chained(merge_mma_kernel<D>, dim3(walks + keys, units), 32, MCfg<D>::kSmem, s, tv, a, seg, walks);
   return cudaGetLastError();
 }
 

@@ -206,6 +206,21 @@ __device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t 
 }
 __device__ __forceinline__ void bulk_store_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
+// Griddepcontrol (programmatic dependent launch): a no-op for kernels launched without it.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// First thing in every kernel of a compression but the first (nothing to wait for) and the last
+// (which lets no kernel of the caller's start early): wait for the kernels before, then let the next
+// one be launched while this one runs.  Every thread of every CTA comes through here, so a kernel that
+// has got past it knows that all kernels but its predecessor have completed, and that the
+// predecessor has too.
+__device__ __forceinline__ void chain_begin() {
+  pdl_wait();
+  pdl_launch_dependents();
+}
+
 // ---- tcgen05 (5th-generation tensor cores, accumulators in tensor memory) ----------------
 // Instruction descriptor, kind::f16: bf16 A and B (both K-major), fp32 D, M x N tile.
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {

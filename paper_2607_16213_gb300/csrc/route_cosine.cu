@@ -90,6 +90,7 @@ __device__ __forceinline__ uint64_t fmul2(uint64_t x, uint64_t y) {
 
 template <int D>
 __global__ __launch_bounds__(kThreads, 1) void cos_tc_kernel(const __grid_constant__ CUtensorMap tmB, CompressArgs a) {
+  chain_begin();
   using C = CosCfg<D>;
   const int kv = blockIdx.y, b = blockIdx.z;
   const int n = a.seq_n[b], m = a.seq_m[b], ne = n - m;
@@ -289,6 +290,7 @@ __global__ __launch_bounds__(kThreads, 1) void cos_tc_kernel(const __grid_consta
 constexpr int kSimtRows = 8;
 template <typename T, int D>
 __global__ __launch_bounds__(kSimtRows * 32) void cos_simt_kernel(CompressArgs a) {
+  chain_begin();
   const int kv = blockIdx.y, b = blockIdx.z;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int e = blockIdx.x * kSimtRows + warp;  // evicted rank
@@ -328,6 +330,7 @@ __global__ __launch_bounds__(kSimtRows * 32) void cos_simt_kernel(CompressArgs a
 constexpr int kRankSlots = 2048;
 
 __global__ __launch_bounds__(32) void cos_rank_kernel(CompressArgs a) {
+  chain_begin();
   const int c = blockIdx.x, s0 = blockIdx.y * kRankSlots;
   const int bk = blockIdx.z, b = bk / a.Hkv;
   const int n = a.seq_n[b], m = a.seq_m[b];
@@ -368,6 +371,7 @@ __global__ __launch_bounds__(32) void cos_rank_kernel(CompressArgs a) {
 }
 
 __global__ __launch_bounds__(256) void cos_colscan_kernel(CompressArgs a) {
+  chain_begin();
   const int bk = blockIdx.y, b = bk / a.Hkv;
   const int slot = blockIdx.x * blockDim.x + threadIdx.x;
   if (slot >= a.seq_m[b]) return;
@@ -385,6 +389,7 @@ __global__ __launch_bounds__(256) void cos_colscan_kernel(CompressArgs a) {
 }
 
 __global__ __launch_bounds__(1024) void cos_slotscan_kernel(CompressArgs a) {
+  chain_begin();
   const int bk = blockIdx.x, b = bk / a.Hkv;
   const int m = a.seq_m[b];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -427,6 +432,7 @@ __global__ __launch_bounds__(1024) void cos_slotscan_kernel(CompressArgs a) {
 }
 
 __global__ __launch_bounds__(256) void cos_scatter_kernel(CompressArgs a) {
+  chain_begin();
   const int bk = blockIdx.y, b = bk / a.Hkv;
   const int n = a.seq_n[b];
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -450,6 +456,7 @@ constexpr int kBatch = 8;  // contributor rows in flight per lane
 
 template <typename T, int D>
 __global__ __launch_bounds__(kMergeWarps * 32) void cos_merge_kernel(CompressArgs a) {
+  chain_begin();
   constexpr int PER = D / 32;
   const int bk = blockIdx.y, b = bk / a.Hkv, kv = bk % a.Hkv;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -520,18 +527,18 @@ cudaError_t launch_argmax_tc(const CompressArgs& a, cudaStream_t st) {
   if (!encode_rows_bf16(&tb, a.Vc, (uint64_t)a.B * a.Hkv * a.m_cap, D, kCols)) return cudaErrorInvalidValue;
   cudaError_t e = set_smem_once<cos_tc_kernel<D>>(C::kSmem);
   if (e != cudaSuccess) return e;
-  cos_tc_kernel<D><<<dim3((a.n_cap + 127) / 128, a.Hkv, a.B), kThreads, C::kSmem, st>>>(tb, a);
+  launch_chained(cos_tc_kernel<D>, dim3((a.n_cap + 127) / 128, a.Hkv, a.B), kThreads, C::kSmem, st, tb, a);
   return cudaGetLastError();
 }
 
 template <typename T, int D>
 void launch_rest(const CompressArgs& a, cudaStream_t st) {
   const unsigned bkn = (unsigned)(a.B * a.Hkv);
-  cos_rank_kernel<<<dim3(a.cos_chunks, (a.m_cap + kRankSlots - 1) / kRankSlots, bkn), 32, 0, st>>>(a);
-  cos_colscan_kernel<<<dim3((a.m_cap + 255) / 256, bkn), 256, 0, st>>>(a);
-  cos_slotscan_kernel<<<bkn, 1024, 0, st>>>(a);
-  cos_scatter_kernel<<<dim3((a.n_cap + 255) / 256, bkn), 256, 0, st>>>(a);
-  cos_merge_kernel<T, D><<<dim3((a.m_cap + kMergeWarps - 1) / kMergeWarps, bkn), kMergeWarps * 32, 0, st>>>(a);
+  launch_chained(cos_rank_kernel, dim3(a.cos_chunks, (a.m_cap + kRankSlots - 1) / kRankSlots, bkn), 32, 0, st, a);
+  launch_chained(cos_colscan_kernel, dim3((a.m_cap + 255) / 256, bkn), 256, 0, st, a);
+  launch_chained(cos_slotscan_kernel, bkn, 1024, 0, st, a);
+  launch_chained(cos_scatter_kernel, dim3((a.n_cap + 255) / 256, bkn), 256, 0, st, a);
+  launch_chained(cos_merge_kernel<T, D>, dim3((a.m_cap + kMergeWarps - 1) / kMergeWarps, bkn), kMergeWarps * 32, 0, st, a);
 }
 
 }  // namespace
@@ -549,10 +556,10 @@ cudaError_t launch_route_cosine(const CompressArgs& a, cudaStream_t st) {
   } else {
     const dim3 grid((a.n_cap + kSimtRows - 1) / kSimtRows, a.Hkv, a.B);
     if (a.D == 128) {
-      cos_simt_kernel<float, 128><<<grid, kSimtRows * 32, 0, st>>>(a);
+      launch_chained(cos_simt_kernel<float, 128>, grid, kSimtRows * 32, 0, st, a);
       launch_rest<float, 128>(a, st);
     } else {
-      cos_simt_kernel<float, 64><<<grid, kSimtRows * 32, 0, st>>>(a);
+      launch_chained(cos_simt_kernel<float, 64>, grid, kSimtRows * 32, 0, st, a);
       launch_rest<float, 64>(a, st);
     }
   }

@@ -11,6 +11,7 @@
 // tile code, so pass 2 sees bit-identical scores.
 #include <algorithm>
 
+#include "ptx.cuh"
 #include "selkv_internal.cuh"
 
 namespace selkv {
@@ -85,6 +86,7 @@ __device__ __forceinline__ float reduce16_sum(float v) {
 // over the chunk's visible columns.
 template <typename T, int D>
 __global__ __launch_bounds__(256) void rowstats_kernel(CompressArgs a) {
+  chain_begin();
   __shared__ __align__(16) float Qs[kDc][kTile + 4];
   __shared__ __align__(16) float Ks[kDc][kTile + 4];
   const int chunk = blockIdx.x, r0 = blockIdx.y * kTile, bk = blockIdx.z;
@@ -152,13 +154,17 @@ __device__ __forceinline__ void fold_row(const CompressArgs& a, int idx) {
   a.rowstat[idx] = make_float2(M, 1.f / ((float)a.G * Z));
 }
 
-__global__ void rowstat_reduce_kernel(CompressArgs a) { fold_row(a, blockIdx.x * blockDim.x + threadIdx.x); }
+__global__ void rowstat_reduce_kernel(CompressArgs a) {
+  chain_begin();
+  fold_row(a, blockIdx.x * blockDim.x + threadIdx.x);
+}
 
 // The fold in the first `fold_blocks` CTAs and ||v_j|| of Eq. 1 in the others: two kernels' work
 // that does not depend on one another in one launch.  D / 8 lanes per row (at most 16), each
 // loading 8 elements at a time.
 template <typename T, int D>
 __global__ __launch_bounds__(256) void fold_norm_kernel(CompressArgs a, int fold_blocks) {
+  chain_begin();
   if ((int)blockIdx.x < fold_blocks) {
     fold_row(a, blockIdx.x * blockDim.x + threadIdx.x);
     return;
@@ -198,6 +204,7 @@ __global__ __launch_bounds__(256) void fold_norm_kernel(CompressArgs a, int fold
 // Pass 2: grid (column tile, b * Hkv); a_j = sum_r 2^(s'_rj - M_r) / (G Z_r).
 template <typename T, int D>
 __global__ __launch_bounds__(256) void colsum_kernel(CompressArgs a) {
+  chain_begin();
   __shared__ __align__(16) float Qs[kDc][kTile + 4];
   __shared__ __align__(16) float Ks[kDc][kTile + 4];
   __shared__ float red[16][kTile];
@@ -239,17 +246,17 @@ template <typename T, int D>
 cudaError_t launch_score_t(const CompressArgs& a, cudaStream_t s, int passes) {
   const int row_tiles = (a.R + kTile - 1) / kTile;
   if (passes & kScoreRowstats) {
-    rowstats_kernel<T, D><<<dim3(a.nchunks, row_tiles, a.B * a.Hkv), 256, 0, s>>>(a);
+    launch_chained(rowstats_kernel<T, D>, dim3(a.nchunks, row_tiles, a.B * a.Hkv), 256, 0, s, a);
     if (a.V == nullptr) {
       launch_rowstat_reduce(a, s);
     } else {
       const size_t rows = (size_t)a.B * a.Hkv * a.n_cap;
       const int fold = (a.B * a.Hkv * a.R + 255) / 256, norm = (int)std::min<size_t>((rows + 15) / 16, 152 * 8);
-      fold_norm_kernel<T, D><<<fold + norm, 256, 0, s>>>(a, fold);
+      launch_chained(fold_norm_kernel<T, D>, fold + norm, 256, 0, s, a, fold);
     }
   }
   if (passes & kScoreColsums)
-    colsum_kernel<T, D><<<dim3((a.n_cap + kTile - 1) / kTile, a.B * a.Hkv), 256, 0, s>>>(a);
+    launch_chained(colsum_kernel<T, D>, dim3((a.n_cap + kTile - 1) / kTile, a.B * a.Hkv), 256, 0, s, a);
   return cudaGetLastError();
 }
 
@@ -257,7 +264,7 @@ cudaError_t launch_score_t(const CompressArgs& a, cudaStream_t s, int passes) {
 
 cudaError_t launch_rowstat_reduce(const CompressArgs& a, cudaStream_t s) {
   const int nrows = a.B * a.Hkv * a.R;
-  rowstat_reduce_kernel<<<(nrows + 255) / 256, 256, 0, s>>>(a);
+  launch_chained(rowstat_reduce_kernel, (nrows + 255) / 256, 256, 0, s, a);
   return cudaGetLastError();
 }
 

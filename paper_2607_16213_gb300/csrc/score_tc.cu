@@ -364,6 +364,7 @@ __global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_k
     fence_mbar_init();
   }
   if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
+  chain_begin();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -770,11 +771,11 @@ cudaError_t launch_tc_t(CompressArgs a, const SeqTable& tab, cudaStream_t st, in
   if (e == cudaSuccess) e = set_smem_once<score_tc_kernel<D, 2, H2>>(C2::kSmem);
   if (e != cudaSuccess) return e;
   if (passes & kScoreRowstats) {
-    k1<<<groups1 * MT, cta_threads(1, H1, a.V != nullptr), C1::kSmem, st>>>(tq, tk1, a, w1);
+    launch_chained(k1, groups1 * MT, cta_threads(1, H1, a.V != nullptr), C1::kSmem, st, tq, tk1, a, w1);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  if (passes & kScoreColsums) k2<<<groups2, cta_threads(2, H2, a.V != nullptr), C2::kSmem, st>>>(tq, tk2, a, w2);
+  if (passes & kScoreColsums) launch_chained(k2, groups2, cta_threads(2, H2, a.V != nullptr), C2::kSmem, st, tq, tk2, a, w2);
   return cudaGetLastError();
 }
 

@@ -1,4 +1,5 @@
 // Per-call set-up: sequence table, output lengths.
+#include "ptx.cuh"
 #include "selkv_internal.cuh"
 
 namespace selkv {
@@ -6,6 +7,7 @@ namespace {
 
 // Sequence table and output lengths.
 __global__ void setup_kernel(SeqTable tab, CompressArgs a) {
+  pdl_launch_dependents();
   for (int b = threadIdx.x; b < a.B; b += blockDim.x) {
     a.seq_n[b] = tab.n[b];
     a.seq_m[b] = tab.m[b];
@@ -16,6 +18,7 @@ __global__ void setup_kernel(SeqTable tab, CompressArgs a) {
 
 // Sequence table alone (the scoring entry point).
 __global__ void seq_setup_kernel(SeqTable tab, int32_t* seq_n, int32_t* seq_m, int32_t* seq_t1, int B) {
+  pdl_launch_dependents();
   for (int b = threadIdx.x; b < B; b += blockDim.x) {
     seq_n[b] = tab.n[b];
     seq_m[b] = tab.m[b];

@@ -339,6 +339,7 @@ __device__ __forceinline__ void compact(const CompressArgs& a, Shared<NT>& sh, c
 // the pooling kernel (0: any, from the arguments).
 template <int POOL, int NT>
 __global__ __launch_bounds__(NT) void topk_kernel(CompressArgs a, SelectWs w, int near_keys) {
+  chain_begin();
   __shared__ Shared<NT> sh;
   extern __shared__ uint32_t dyn_keys[];
   const int u = blockIdx.y, b = u / a.Hkv, lane = threadIdx.x & 31;
@@ -408,6 +409,7 @@ __global__ __launch_bounds__(NT) void topk_kernel(CompressArgs a, SelectWs w, in
 // Grid (cluster size, B).
 template <int NT>
 __global__ __launch_bounds__(NT) void trim_kernel(CompressArgs a, SelectWs w, int near_keys) {
+  chain_begin();
   __shared__ Shared<NT> sh;
   __shared__ RadixCut cut[32];
   extern __shared__ uint32_t dyn_keys[];
@@ -512,13 +514,15 @@ cudaError_t launch_clusters(const CompressArgs& a, const SelectWs& w, int units,
   cfg.blockDim = dim3(NT);
   cfg.dynamicSmemBytes = near_keys ? (size_t)span * 4 : 0;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = cs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // (as launch_chained)
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, Kern, a, w, near_keys);
 }
 

@@ -347,6 +347,7 @@ selkv_status selkv_compress(const selkv_shape* shape, const int32_t* n_len, doub
     a.dbg_ratio = debug->ratio;
   }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  a.chain = may_chain(st);
   const SelectWs sw = carve_select_ws(at<char>(workspace, plan.select), s.batch, s.num_kv_heads, s.n_cap);
   cudaError_t e = launch_setup(a, tab, st);
   // the scoring also takes the value norms
@@ -409,6 +410,7 @@ selkv_status selkv_score(const selkv_shape* shape, const int32_t* n_len, const v
   a.rowpart = at<float2>(workspace, plan.rowpart);
   a.rowstat = at<float2>(workspace, plan.rowstat);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  a.chain = may_chain(st);
   cudaError_t e = cudaSuccess;
   int kernels = 0;
   if (passes & SELKV_SCORE_ROWSTATS) {  // the column-sum pass reuses the table of its row-statistics call

@@ -562,7 +562,7 @@ __global__ __launch_bounds__(256) void bias_kernel(CompressArgs a) {
 }
 
 cudaError_t launch_bias(const CompressArgs& a, cudaStream_t s) {
-  launch_chained(bias_kernel, dim3((a.m_cap + 255) / 256, a.B, a.per_head ? a.Hkv : 1), 256, 0, s, a);
+  launch_chained(a.chain, bias_kernel, dim3((a.m_cap + 255) / 256, a.B, a.per_head ? a.Hkv : 1), 256, 0, s, a);
   return cudaGetLastError();
 }
 
@@ -570,14 +570,14 @@ template <typename T, int D>
 void launch_copy_t(const CompressArgs& a, cudaStream_t s) {
   constexpr int kPieces = D * (int)sizeof(T) / 16;
   const size_t copy_threads = (size_t)a.Hkv * a.m_cap * 2 * kPieces;
-  launch_chained(copy_kernel<T, D>, dim3((unsigned)((copy_threads + 255) / 256), a.B), 256, 0, s, a);
+  launch_chained(a.chain, copy_kernel<T, D>, dim3((unsigned)((copy_threads + 255) / 256), a.B), 256, 0, s, a);
 }
 
 template <typename T, int D>
 void launch_merge_t(const CompressArgs& a, cudaStream_t s) {
   // with the bucket routing and no repositioning the merge warps copy the kept rows themselves
   if (!merge_copies_kept_rows(a)) launch_copy_t<T, D>(a, s);
-  if (a.routing == SELKV_ROUTE_BUCKET) launch_chained(merge_kernel<T, D>, dim3(a.nbk, a.B * a.Hkv), 32, 0, s, a);
+  if (a.routing == SELKV_ROUTE_BUCKET) launch_chained(a.chain, merge_kernel<T, D>, dim3(a.nbk, a.B * a.Hkv), 32, 0, s, a);
 }
 
 }  // namespace
@@ -590,7 +590,7 @@ cudaError_t launch_merge(const CompressArgs& a, cudaStream_t s) {
   if (a.rope != SELKV_ROPE_OFF) {
     const int groups = (a.rope_hi + 256 + kRopeRowsPerThread - 1) / kRopeRowsPerThread;
     const int threads = a.D / 2 * groups;
-    launch_chained(rope_table_kernel, (threads + 127) / 128, 128, 0, s, a);
+    launch_chained(a.chain, rope_table_kernel, (threads + 127) / 128, 128, 0, s, a);
   }
   if (a.use_kmask) {
     if (a.rope != SELKV_ROPE_OFF) {
@@ -602,7 +602,7 @@ cudaError_t launch_merge(const CompressArgs& a, cudaStream_t s) {
     return launch_bias(a, s);
   }
   if (a.routing == SELKV_ROUTE_BUCKET)
-    launch_chained(route_kernel, dim3((a.nbk + kWarpsPerCta - 1) / kWarpsPerCta, a.B), kWarpsPerCta * 32, 0, s, a);
+    launch_chained(a.chain, route_kernel, dim3((a.nbk + kWarpsPerCta - 1) / kWarpsPerCta, a.B), kWarpsPerCta * 32, 0, s, a);
   if (a.dtype == SELKV_BF16) {
     if (a.D == 128) launch_merge_t<__nv_bfloat16, 128>(a, s);
     else launch_merge_t<__nv_bfloat16, 64>(a, s);

@@ -492,7 +492,7 @@ cudaError_t launch_t(const CompressArgs& a, cudaStream_t s) {
   const int walks = (nb + seg - 1) / seg;
   // with repositioning copy_kernel writes the keys
   const int keys = a.rope == SELKV_ROPE_OFF ? (a.m_cap + kKeySlots - 1) / kKeySlots : 0;
-  launch_chained(merge_mma_kernel<D>, dim3(walks + keys, units), 32, MCfg<D>::kSmem, s, tv, a, seg, walks);
+  launch_chained(a.chain, merge_mma_kernel<D>, dim3(walks + keys, units), 32, MCfg<D>::kSmem, s, tv, a, seg, walks);
   return cudaGetLastError();
 }
 

@@ -527,18 +527,18 @@ cudaError_t launch_argmax_tc(const CompressArgs& a, cudaStream_t st) {
   if (!encode_rows_bf16(&tb, a.Vc, (uint64_t)a.B * a.Hkv * a.m_cap, D, kCols)) return cudaErrorInvalidValue;
   cudaError_t e = set_smem_once<cos_tc_kernel<D>>(C::kSmem);
   if (e != cudaSuccess) return e;
-  launch_chained(cos_tc_kernel<D>, dim3((a.n_cap + 127) / 128, a.Hkv, a.B), kThreads, C::kSmem, st, tb, a);
+  launch_chained(a.chain, cos_tc_kernel<D>, dim3((a.n_cap + 127) / 128, a.Hkv, a.B), kThreads, C::kSmem, st, tb, a);
   return cudaGetLastError();
 }
 
 template <typename T, int D>
 void launch_rest(const CompressArgs& a, cudaStream_t st) {
   const unsigned bkn = (unsigned)(a.B * a.Hkv);
-  launch_chained(cos_rank_kernel, dim3(a.cos_chunks, (a.m_cap + kRankSlots - 1) / kRankSlots, bkn), 32, 0, st, a);
-  launch_chained(cos_colscan_kernel, dim3((a.m_cap + 255) / 256, bkn), 256, 0, st, a);
-  launch_chained(cos_slotscan_kernel, bkn, 1024, 0, st, a);
-  launch_chained(cos_scatter_kernel, dim3((a.n_cap + 255) / 256, bkn), 256, 0, st, a);
-  launch_chained(cos_merge_kernel<T, D>, dim3((a.m_cap + kMergeWarps - 1) / kMergeWarps, bkn), kMergeWarps * 32, 0, st, a);
+  launch_chained(a.chain, cos_rank_kernel, dim3(a.cos_chunks, (a.m_cap + kRankSlots - 1) / kRankSlots, bkn), 32, 0, st, a);
+  launch_chained(a.chain, cos_colscan_kernel, dim3((a.m_cap + 255) / 256, bkn), 256, 0, st, a);
+  launch_chained(a.chain, cos_slotscan_kernel, bkn, 1024, 0, st, a);
+  launch_chained(a.chain, cos_scatter_kernel, dim3((a.n_cap + 255) / 256, bkn), 256, 0, st, a);
+  launch_chained(a.chain, cos_merge_kernel<T, D>, dim3((a.m_cap + kMergeWarps - 1) / kMergeWarps, bkn), kMergeWarps * 32, 0, st, a);
 }
 
 }  // namespace
@@ -556,10 +556,10 @@ cudaError_t launch_route_cosine(const CompressArgs& a, cudaStream_t st) {
   } else {
     const dim3 grid((a.n_cap + kSimtRows - 1) / kSimtRows, a.Hkv, a.B);
     if (a.D == 128) {
-      launch_chained(cos_simt_kernel<float, 128>, grid, kSimtRows * 32, 0, st, a);
+      launch_chained(a.chain, cos_simt_kernel<float, 128>, grid, kSimtRows * 32, 0, st, a);
       launch_rest<float, 128>(a, st);
     } else {
-      launch_chained(cos_simt_kernel<float, 64>, grid, kSimtRows * 32, 0, st, a);
+      launch_chained(a.chain, cos_simt_kernel<float, 64>, grid, kSimtRows * 32, 0, st, a);
       launch_rest<float, 64>(a, st);
     }
   }

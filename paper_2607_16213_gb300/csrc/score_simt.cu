@@ -246,17 +246,17 @@ template <typename T, int D>
 cudaError_t launch_score_t(const CompressArgs& a, cudaStream_t s, int passes) {
   const int row_tiles = (a.R + kTile - 1) / kTile;
   if (passes & kScoreRowstats) {
-    launch_chained(rowstats_kernel<T, D>, dim3(a.nchunks, row_tiles, a.B * a.Hkv), 256, 0, s, a);
+    launch_chained(a.chain, rowstats_kernel<T, D>, dim3(a.nchunks, row_tiles, a.B * a.Hkv), 256, 0, s, a);
     if (a.V == nullptr) {
       launch_rowstat_reduce(a, s);
     } else {
       const size_t rows = (size_t)a.B * a.Hkv * a.n_cap;
       const int fold = (a.B * a.Hkv * a.R + 255) / 256, norm = (int)std::min<size_t>((rows + 15) / 16, 152 * 8);
-      launch_chained(fold_norm_kernel<T, D>, fold + norm, 256, 0, s, a, fold);
+      launch_chained(a.chain, fold_norm_kernel<T, D>, fold + norm, 256, 0, s, a, fold);
     }
   }
   if (passes & kScoreColsums)
-    launch_chained(colsum_kernel<T, D>, dim3((a.n_cap + kTile - 1) / kTile, a.B * a.Hkv), 256, 0, s, a);
+    launch_chained(a.chain, colsum_kernel<T, D>, dim3((a.n_cap + kTile - 1) / kTile, a.B * a.Hkv), 256, 0, s, a);
   return cudaGetLastError();
 }
 
@@ -264,7 +264,7 @@ cudaError_t launch_score_t(const CompressArgs& a, cudaStream_t s, int passes) {
 
 cudaError_t launch_rowstat_reduce(const CompressArgs& a, cudaStream_t s) {
   const int nrows = a.B * a.Hkv * a.R;
-  launch_chained(rowstat_reduce_kernel, (nrows + 255) / 256, 256, 0, s, a);
+  launch_chained(a.chain, rowstat_reduce_kernel, (nrows + 255) / 256, 256, 0, s, a);
   return cudaGetLastError();
 }
 

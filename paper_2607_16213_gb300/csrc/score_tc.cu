@@ -771,11 +771,11 @@ cudaError_t launch_tc_t(CompressArgs a, const SeqTable& tab, cudaStream_t st, in
   if (e == cudaSuccess) e = set_smem_once<score_tc_kernel<D, 2, H2>>(C2::kSmem);
   if (e != cudaSuccess) return e;
   if (passes & kScoreRowstats) {
-    launch_chained(k1, groups1 * MT, cta_threads(1, H1, a.V != nullptr), C1::kSmem, st, tq, tk1, a, w1);
+    launch_chained(a.chain, k1, groups1 * MT, cta_threads(1, H1, a.V != nullptr), C1::kSmem, st, tq, tk1, a, w1);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  if (passes & kScoreColsums) launch_chained(k2, groups2, cta_threads(2, H2, a.V != nullptr), C2::kSmem, st, tq, tk2, a, w2);
+  if (passes & kScoreColsums) launch_chained(a.chain, k2, groups2, cta_threads(2, H2, a.V != nullptr), C2::kSmem, st, tq, tk2, a, w2);
   return cudaGetLastError();
 }
 

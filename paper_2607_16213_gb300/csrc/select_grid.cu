@@ -522,7 +522,7 @@ cudaError_t launch_clusters(const CompressArgs& a, const SelectWs& w, int units,
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // (as launch_chained)
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = a.chain ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, Kern, a, w, near_keys);
 }
 

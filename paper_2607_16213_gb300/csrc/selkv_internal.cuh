@@ -137,6 +137,7 @@ struct SeqTable {
 };
 
 struct CompressArgs {
+  bool chain;     // launch with launch_chained's early start
   int dtype, B, Hq, Hkv, G, D, W, n_cap, m_cap;
   int R;          // observation rows per KV head: G * W
   int nchunks;    // column chunks of the row-statistics pass
@@ -339,10 +340,18 @@ cudaError_t allow_any_cluster_once() {
   return e;
 }
 
+// Whether the kernels of a call may be brought up early (launch_chained): on the default stream, where
+// nothing else hides their launches.  With several streams, or in a captured graph, the other work
+// does (four streams: 0.176 ms a layer either way), and there a decode graph of 8192 nodes replayed
+// afterwards took 23.2 us a launch in place of 20.9 in some programs.
+inline bool may_chain(cudaStream_t s) { return s == nullptr || s == cudaStreamLegacy; }
+
 // Launch of a kernel that begins with chain_begin (or pdl_wait): it is brought up while its
-// predecessor on the stream still runs, which hides its launch (about 1.7 us a kernel: one layer at 16k 88 -> 76 us, 1k of fp32 64 -> 45).
+// predecessor on the stream still runs, which hides its launch (about 1.7 us a kernel: one layer at
+// 16k 88 -> 76 us, 1k of fp32 64 -> 45).
 template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
+cudaError_t launch_chained(bool chain, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                           const A&... args) {
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -352,7 +361,7 @@ cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t sme
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = chain ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 

@@ -8,10 +8,10 @@
 // |S| |E| d multiply-adds per KV head, run on the tensor cores for bf16 caches.  Kernels, in
 // stream order (after the copy kernel has put the kept rows into V_c and 1 / ||v_i|| into
 // cos_invn):
-//   argmax   a CTA per 128 evicted positions of one (sequence, KV head): their value rows are
+//   argmax   a CTA per 256 evicted positions of one (sequence, KV head): their value rows are
 //            gathered once into shared memory (the MMA's A), 256-slot tiles of the kept rows
-//            stream in by TMA (B), tcgen05.mma accumulates 128 x 256 products in tensor memory,
-//            and sixteen epilogue warps keep each row's running (max s_ji, slot) over a quarter
+//            stream in by TMA (B), tcgen05.mma accumulates 128 x 256 products in tensor memory
+//            for each half of the rows in turn, and sixteen epilogue warps keep each row's running (max s_ji, slot) over a quarter
 //            of each tile's columns; the quarters are folded in column order at the end.  The
 //            row's target, gate g = clamp(s / ||v_j||, 0, 1) and decision are written there.
 //            fp32 caches use a CUDA-core kernel with the same outputs.
@@ -72,12 +72,18 @@ constexpr int kChunkBytes = kCols * 128;   // one 64-element-wide box of a tile
 constexpr int kRingChunks = 4;             // two tiles in flight at d = 128
 constexpr uint32_t kTmemCols = 512;        // two 256-column accumulators
 
+// A CTA takes 256 evicted rows as two halves of 128, an accumulator each, on the same tiles of kept
+// rows: with 128 rows a CTA the tiles came from L2 twice as often, 0.8 GB for one layer at 16k, and the
+// kernel took 141 us; now 124 (95 of it the loads and products alone, 18 the search for the slot of a
+// new maximum).
+constexpr int kRowsPerCta = 256;
+
 template <int D>
 struct CosCfg {
   static constexpr int kBoxes = D / 64;
-  static constexpr int kABytes = 128 * D * 2;
+  static constexpr int kABytes = kRowsPerCta * D * 2;
   static constexpr int kRing = kRingChunks * kChunkBytes;
-  static constexpr int kMisc = 256 + 3 * 128 * 8;
+  static constexpr int kMisc = 256 + kEpiWarps * 64 * 4 + 3 * kRowsPerCta * 8;
   static constexpr int kSmem = 1024 + kABytes + kRing + kMisc;
   static_assert(kSmem <= 227 * 1024, "shared memory per CTA");
 };
@@ -94,12 +100,12 @@ __global__ __launch_bounds__(kThreads, 1) void cos_tc_kernel(const __grid_consta
   using C = CosCfg<D>;
   const int kv = blockIdx.y, b = blockIdx.z;
   const int n = a.seq_n[b], m = a.seq_m[b], ne = n - m;
-  const int r0 = blockIdx.x * 128;
+  const int r0 = blockIdx.x * kRowsPerCta;
   if (r0 >= ne) return;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  unsigned char* As = smem;                 // [kBoxes][128 rows][128 B]
+  unsigned char* As = smem;                 // [kBoxes][256 rows][128 B]
   unsigned char* ring = smem + C::kABytes;  // [kRingChunks][256 rows][128 B]
   unsigned char* misc = ring + C::kRing;
   uint64_t* full = reinterpret_cast<uint64_t*>(misc);
@@ -110,13 +116,15 @@ __global__ __launch_bounds__(kThreads, 1) void cos_tc_kernel(const __grid_consta
   uint64_t* done = abar + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float2* fold = reinterpret_cast<float2*>(misc + 256);  // [3][128] (best, slot) of quarters 1-3
+  float* winv = reinterpret_cast<float*>(misc + 256);  // [epilogue warps][64] 1 / ||v|| of the warp's columns
+  float2* fold = reinterpret_cast<float2*>(winv + kEpiWarps * 64);  // [3][256] (best, slot) of quarters 1-3
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const size_t bk = (size_t)b * a.Hkv + kv;
   const size_t su = sel_unit(a, b, kv);
   const int nt = (m + kCols - 1) / kCols;
   const int nchunks = nt * C::kBoxes;
+  const int nph = ne - r0 > 128 ? 2 : 1;  // halves with rows
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kRingChunks; ++i) {
@@ -163,26 +171,26 @@ __global__ __launch_bounds__(kThreads, 1) void cos_tc_kernel(const __grid_consta
       const uint32_t idesc = umma_idesc_bf16(128, kCols);
       const uint32_t abase = smem_u32(As), rbase = smem_u32(ring);
       for (int t = 0; ok && t < nt; ++t) {
-        const int buf = t & 1;
-        if (!mbar_wait(&tempty[buf], ((t >> 1) & 1) ^ 1) || *abort_flag) {
-          ok = false;
-          break;
-        }
-        for (int bx = 0; bx < C::kBoxes; ++bx) {
-          const int c = t * C::kBoxes + bx, st = c % kRingChunks;
-          if (!mbar_wait(&full[st], (c / kRingChunks) & 1) || *abort_flag) {
+        for (int ph = 0; ok && ph < nph; ++ph) {  // half ph into accumulator ph
+          if (!mbar_wait(&tempty[ph], (t & 1) ^ 1) || *abort_flag) {
             ok = false;
             break;
           }
-          tc_fence_after();
+          for (int bx = 0; bx < C::kBoxes; ++bx) {
+            const int c = t * C::kBoxes + bx, st = c % kRingChunks;
+            if (ph == 0 && (!mbar_wait(&full[st], (c / kRingChunks) & 1) || *abort_flag)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks)
-            umma_bf16(tmem + buf * kCols, umma_desc_sw128(abase + bx * 128 * 128 + ks * 32),
-                      umma_desc_sw128(rbase + st * kChunkBytes + ks * 32), idesc, (bx | ks) > 0);
-          umma_commit(&empty[st]);  // the stage is free once these MMAs have read it
+            for (int ks = 0; ks < 4; ++ks)
+              umma_bf16(tmem + ph * kCols, umma_desc_sw128(abase + bx * kRowsPerCta * 128 + ph * 128 * 128 + ks * 32),
+                        umma_desc_sw128(rbase + st * kChunkBytes + ks * 32), idesc, (bx | ks) > 0);
+            if (ph == nph - 1) umma_commit(&empty[st]);  // the stage is free once these MMAs have read it
+          }
+          if (ok) umma_commit(&tfull[ph]);
         }
-        if (!ok) break;
-        umma_commit(&tfull[buf]);
       }
       if (!ok) {
         *abort_flag = 1;
@@ -195,15 +203,15 @@ __global__ __launch_bounds__(kThreads, 1) void cos_tc_kernel(const __grid_consta
     // ---------------- epilogue: warps 0-15 ----------------
     const int32_t* ev = a.ev_pos + su * a.n_cap;  // evicted positions, ascending
     {
-      // gather the 128 evicted value rows into the swizzled A layout (rows past the evicted
+      // gather the 256 evicted value rows into the swizzled A layout (rows past the evicted
       // count repeat the last one; their results are not written)
       constexpr int kRowChunks = D / 8;  // 16-byte pieces per row
       const __nv_bfloat16* Vb = static_cast<const __nv_bfloat16*>(a.V) + bk * a.n_cap * D;
       const uint32_t abase = smem_u32(As);
-      for (int i = threadIdx.x; i < 128 * kRowChunks; i += kEpiWarps * 32) {
+      for (int i = threadIdx.x; i < kRowsPerCta * kRowChunks; i += kEpiWarps * 32) {
         const int r = i / kRowChunks, ch = i % kRowChunks;
         const int j = ev[min(r0 + r, ne - 1)];
-        cp_async16_cg(abase + (ch >> 3) * (128 * 128) + swz128(r, ch & 7), Vb + (size_t)j * D + ch * 8);
+        cp_async16_cg(abase + (ch >> 3) * (kRowsPerCta * 128) + swz128(r, ch & 7), Vb + (size_t)j * D + ch * 8);
       }
       cp_async_wait_all();
       fence_proxy_async_smem();  // visible to the tensor cores (async proxy)
@@ -212,7 +220,6 @@ __global__ __launch_bounds__(kThreads, 1) void cos_tc_kernel(const __grid_consta
     }
     const int q = warp & 3, part = warp >> 2;  // TMEM lane quarter (rows), column quarter of a tile
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    const float* invn = a.cos_invn + bk * a.cos_mpad;
     auto warp_wait = [&](uint64_t* bar, uint32_t parity) -> bool {
       int ok = 0;
       if (lane == 0) {
@@ -224,57 +231,73 @@ __global__ __launch_bounds__(kThreads, 1) void cos_tc_kernel(const __grid_consta
       }
       return __shfl_sync(0xffffffffu, ok, 0) != 0;
     };
-    float best = -INFINITY;
-    int bcol = -1;
+    float best[2] = {-INFINITY, -INFINITY};
+    int bcol[2] = {-1, -1};
+    // 1 / ||v|| of this warp's 64 columns of a tile, fetched a tile ahead (cos_mpad is whole tiles)
+    const float2* invn = reinterpret_cast<const float2*>(a.cos_invn + bk * a.cos_mpad + part * 64) + lane;
+    float2* wown = reinterpret_cast<float2*>(winv + warp * 64);
+    if (nt > 0) wown[lane] = __ldg(invn);
+    __syncwarp();
     for (int t = 0; t < nt; ++t) {
-      const int buf = t & 1;
-      const bool ok = warp_wait(&tfull[buf], (t >> 1) & 1);
-      tc_fence_after();
-      if (ok) {
+      float2 wnext = make_float2(0.f, 0.f);
+      if (t + 1 < nt) wnext = __ldg(invn + (size_t)(t + 1) * (kCols / 2));
+#pragma unroll
+      for (int ph = 0; ph < 2; ++ph) {
+        if (ph >= nph) break;
+        const bool ok = warp_wait(&tfull[ph], t & 1);
+        tc_fence_after();
+        if (ok) {
 #pragma unroll 1
-        for (int c = 0; c < 64; c += 32) {
-          float v[32];
-          tmem_ld32(tmem + lane_base + buf * kCols + part * 64 + c, v);
-          const int col0 = t * kCols + part * 64 + c;
-          if (col0 >= m) continue;  // uniform across the warp
-          // s = acc / ||v_i||, pairs packed; slots past m take -inf
-          const float4* w4 = reinterpret_cast<const float4*>(invn + col0);
+          for (int c = 0; c < 64; c += 32) {
+            float v[32];
+            tmem_ld32(tmem + lane_base + ph * kCols + part * 64 + c, v);
+            const int col0 = t * kCols + part * 64 + c;
+            if (col0 >= m) continue;  // uniform across the warp
+            // s = acc / ||v_i||, pairs packed; slots past m take -inf
+            const uint32_t w4 = smem_u32(winv + warp * 64 + c);
 #pragma unroll
-          for (int i = 0; i < 32; i += 4) {
-            const float4 w = __ldg(w4 + i / 4);
-            unpack_f2(fmul2(pack_f2(v[i], v[i + 1]), pack_f2(w.x, w.y)), v[i], v[i + 1]);
-            unpack_f2(fmul2(pack_f2(v[i + 2], v[i + 3]), pack_f2(w.z, w.w)), v[i + 2], v[i + 3]);
-          }
-          if (col0 + 32 > m) {
+            for (int k = 0; k < 32; k += 4) {
+              const float4 w = lds_f4(w4 + k * 4);
+              unpack_f2(fmul2(pack_f2(v[k], v[k + 1]), pack_f2(w.x, w.y)), v[k], v[k + 1]);
+              unpack_f2(fmul2(pack_f2(v[k + 2], v[k + 3]), pack_f2(w.z, w.w)), v[k + 2], v[k + 3]);
+            }
+            if (col0 + 32 > m) {
 #pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = col0 + i < m ? v[i] : -INFINITY;
-          }
-          const float cmax = max32(v);
-          if (cmax > best) {  // strictly larger: an equal value at a later slot does not win
-            int first = 31;   // the lowest slot holding the maximum
+              for (int k = 0; k < 32; ++k) v[k] = col0 + k < m ? v[k] : -INFINITY;
+            }
+            const float cmax = max32(v);
+            if (cmax > best[ph]) {  // strictly larger: an equal value at a later slot does not win
+              int first = 31;       // the lowest slot holding the maximum
 #pragma unroll
-            for (int i = 30; i >= 0; --i) first = v[i] == cmax ? i : first;
-            best = cmax;
-            bcol = col0 + first;
+              for (int k = 30; k >= 0; --k) first = v[k] == cmax ? k : first;
+              best[ph] = cmax;
+              bcol[ph] = col0 + first;
+            }
           }
         }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tempty[ph]);
       }
-      tc_fence_before();
+      wown[lane] = wnext;  // (every lane is past its reads: the __syncwarp above)
       __syncwarp();
-      if (lane == 0) mbar_arrive(&tempty[buf]);
     }
     // fold the four column quarters of each row (their columns interleave: compare slots)
     const int r = q * 32 + lane;
-    if (part > 0) fold[(part - 1) * 128 + r] = make_float2(best, __int_as_float(bcol));
-    named_bar_sync(1, kEpiWarps * 32);
-    if (part == 0 && r0 + r < ne) {
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const float2 f = fold[k * 128 + r];
-        argmax_take(best, bcol, f.x, __float_as_int(f.y));
+    for (int ph = 0; ph < 2; ++ph)
+      if (part > 0 && ph < nph) fold[(part - 1) * kRowsPerCta + ph * 128 + r] = make_float2(best[ph], __int_as_float(bcol[ph]));
+    named_bar_sync(1, kEpiWarps * 32);
+#pragma unroll
+    for (int ph = 0; ph < 2; ++ph)
+      if (part == 0 && r0 + ph * 128 + r < ne) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const float2 f = fold[k * kRowsPerCta + ph * 128 + r];
+          argmax_take(best[ph], bcol[ph], f.x, __float_as_int(f.y));
+        }
+        cos_finish(a, b, kv, ev[r0 + ph * 128 + r], best[ph], bcol[ph]);
       }
-      cos_finish(a, b, kv, ev[r0 + r], best, bcol);
-    }
   }
   tc_fence_before();
   __syncthreads();
@@ -527,7 +550,7 @@ cudaError_t launch_argmax_tc(const CompressArgs& a, cudaStream_t st) {
   if (!encode_rows_bf16(&tb, a.Vc, (uint64_t)a.B * a.Hkv * a.m_cap, D, kCols)) return cudaErrorInvalidValue;
   cudaError_t e = set_smem_once<cos_tc_kernel<D>>(C::kSmem);
   if (e != cudaSuccess) return e;
-  launch_chained(a.chain, cos_tc_kernel<D>, dim3((a.n_cap + 127) / 128, a.Hkv, a.B), kThreads, C::kSmem, st, tb, a);
+  launch_chained(a.chain, cos_tc_kernel<D>, dim3((a.n_cap + kRowsPerCta - 1) / kRowsPerCta, a.Hkv, a.B), kThreads, C::kSmem, st, tb, a);
   return cudaGetLastError();
 }
 

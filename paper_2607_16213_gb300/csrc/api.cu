@@ -158,7 +158,7 @@ int compress_kernel_count(const CompressArgs& a) {
   int k = 1 + (score_uses_tc(a.dtype, a.D, a.R) ? 2 : 3);
   k += a.per_head ? 1 : 2;
   if (a.rope != SELKV_ROPE_OFF) k += 1;
-  if (a.use_kmask) return k + 1 + (a.rope != SELKV_ROPE_OFF ? 1 : 0) + 1;
+  if (a.use_kmask) return k + 2;
   if (a.routing == SELKV_ROUTE_COSINE)
     k += 1 + (a.m_cap > 0 ? cosine_kernels(a.dtype, a.D) : 0);
   else

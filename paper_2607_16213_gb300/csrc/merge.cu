@@ -26,6 +26,7 @@
 #include <climits>
 
 #include "ptx.cuh"
+#include "rope.cuh"
 #include "selkv_internal.cuh"
 
 namespace selkv {
@@ -76,12 +77,17 @@ __global__ __launch_bounds__(kWarpsPerCta * 32) void route_kernel(CompressArgs a
 // Angles are reduced modulo 2 pi in fp64 before the sine and cosine, so shifts of 10^5
 // positions stay accurate to fp32 rounding.
 constexpr int kRopeRowsPerThread = 8;
+// The table depends on no other kernel of the call: where it may start early, it is made beside the
+// selection's few clusters, and only its end waits for them.
 __global__ void rope_table_kernel(CompressArgs a) {
-  chain_begin();
+  pdl_launch_dependents();
   const int half = a.D / 2, rows = a.rope_hi + 256;
   const int groups = (rows + kRopeRowsPerThread - 1) / kRopeRowsPerThread;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= half * groups) return;
+  if (i >= half * groups) {
+    pdl_wait();
+    return;
+  }
   const int f = i % half, c0 = (i / half) * kRopeRowsPerThread;
   const double w = pow((double)a.rope_theta, -2.0 * f / a.D);
   const double two_pi = 6.283185307179586;
@@ -93,28 +99,7 @@ __global__ void rope_table_kernel(CompressArgs a) {
     sincosf((float)ang, &sn, &cs);
     a.rope_tab[(size_t)c * half + f] = make_float2(cs, sn);
   }
-}
-
-// (cos, sin) of e w_f for the N consecutive frequencies f0 .. f0 + N - 1 (f0 and N even),
-// from the coarse and the fine row of e.
-template <int N>
-__device__ __forceinline__ void rope_angles(const CompressArgs& a, int f0, int e, float2 (&cs)[N]) {
-  const int half = a.D / 2;
-  const float4* h = reinterpret_cast<const float4*>(a.rope_tab + (size_t)(e >> 8) * half + f0);
-  const float4* l = reinterpret_cast<const float4*>(a.rope_tab + (size_t)(a.rope_hi + (e & 255)) * half + f0);
-#pragma unroll
-  for (int t = 0; t < N / 2; ++t) {
-    const float4 hv = h[t], lv = l[t];
-    cs[2 * t] = make_float2(hv.x * lv.x - hv.y * lv.y, hv.y * lv.x + hv.x * lv.y);
-    cs[2 * t + 1] = make_float2(hv.z * lv.z - hv.w * lv.w, hv.w * lv.z + hv.z * lv.w);
-  }
-}
-
-// Turn the pair (x, y) back by e w_f (from position j to slot j - e).
-__device__ __forceinline__ void rope_back(float& x, float& y, float2 cs) {
-  const float nx = x * cs.x + y * cs.y, ny = y * cs.x - x * cs.y;
-  x = nx;
-  y = ny;
+  pdl_wait();
 }
 
 template <typename T>
@@ -593,10 +578,6 @@ cudaError_t launch_merge(const CompressArgs& a, cudaStream_t s) {
     launch_chained(a.chain, rope_table_kernel, (threads + 127) / 128, 128, 0, s, a);
   }
   if (a.use_kmask) {
-    if (a.rope != SELKV_ROPE_OFF) {
-      if (a.D == 128) launch_copy_t<__nv_bfloat16, 128>(a, s);
-      else launch_copy_t<__nv_bfloat16, 64>(a, s);
-    }
     const cudaError_t e = launch_merge_mma(a, s);
     if (e != cudaSuccess) return e;
     return launch_bias(a, s);

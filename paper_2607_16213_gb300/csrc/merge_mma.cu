@@ -23,6 +23,7 @@
 #include <climits>
 
 #include "ptx.cuh"
+#include "rope.cuh"
 #include "selkv_internal.cuh"
 
 namespace selkv {
@@ -86,8 +87,45 @@ __device__ __forceinline__ int argmax_kept(uint32_t mask, float a, int lane, flo
   return __ffs(__ballot_sync(kFull, ((mask >> lane) & 1u) && key == mx)) - 1;
 }
 
+// Turn the staged key rows back by e w_f, e = position - slot: a lane takes the pairs of two
+// frequencies of a row.
+template <int D>
+__device__ __forceinline__ void turn_rows(const CompressArgs& a, const int (&pos)[kKeySlots / 32], int s0, int rows,
+                                          unsigned char* ring) {
+  constexpr int LP = D / 4, RPI = 32 / LP;  // lanes per row, rows per step
+  const int sub = (int)threadIdx.x / LP, f0 = (int)threadIdx.x % LP * 2;
+  // HALF pairs (f, f + d/2), INTERLEAVED (2 f, 2 f + 1)
+  const bool half = a.rope == SELKV_ROPE_HALF;
+  const int o0 = half ? f0 : 2 * f0, o1 = half ? f0 + D / 2 : 2 * f0 + 2;  // this lane's two 4-byte words
+#pragma unroll
+  for (int i = 0; i < kKeySlots / 32; ++i) {
+#pragma unroll 4
+    for (int k = 0; k < 32; k += RPI) {
+      const int r = i * 32 + k + sub;
+      const int e = max(0, __shfl_sync(kFull, pos[i], k + sub) - (s0 + r));  // kept positions ascend with their slots
+      if (r >= rows) continue;
+      uint32_t* w0 = reinterpret_cast<uint32_t*>(ring + (r * D + o0) * 2);
+      uint32_t* w1 = reinterpret_cast<uint32_t*>(ring + (r * D + o1) * 2);
+      const uint32_t u0 = *w0, u1 = *w1;
+      float x0 = bf16_lo(u0), x1 = bf16_hi(u0), y0 = bf16_lo(u1), y1 = bf16_hi(u1);
+      float2 cs[2];
+      rope_angles<2>(a, f0, e, cs);
+      if (half) {
+        rope_back(x0, y0, cs[0]);
+        rope_back(x1, y1, cs[1]);
+      } else {
+        rope_back(x0, x1, cs[0]);
+        rope_back(y0, y1, cs[1]);
+      }
+      *w0 = pack_bf16(x0, x1);
+      *w1 = pack_bf16(y0, y1);
+    }
+  }
+}
+
 // Key rows of slots [s0, s0 + kKeySlots) of (sequence, KV head) bk, a warp's work: one bulk copy a row
-// into the idle ring, then all of them to the slots, which are consecutive, with one.
+// into the idle ring, then all of them to the slots, which are consecutive, with one; in between, with
+// repositioning, each is turned by the shift from its position to its slot.
 template <int D>
 __device__ __forceinline__ void copy_keys(const CompressArgs& a, int bk, size_t unit, int s0, int m, unsigned char* ring,
                                           uint64_t* bar) {
@@ -122,6 +160,11 @@ __device__ __forceinline__ void copy_keys(const CompressArgs& a, int bk, size_t 
     if (lane == 0) raise_flag(a.flags, SELKV_DEVERR_TIMEOUT);
     mbar_wait(bar, 0);  // (bounded) the copies land before the CTA leaves
     return;
+  }
+  if (a.rope != SELKV_ROPE_OFF) {
+    turn_rows<D>(a, pos, s0, rows, ring);
+    fence_proxy_async_smem();  // the turned rows, before the bulk copy reads them
+    __syncwarp();
   }
   if (lane == 0) {
     bulk_store(static_cast<__nv_bfloat16*>(a.Kc) + ((size_t)bk * a.m_cap + s0) * D, ring, (uint32_t)rows * D * 2);
@@ -209,7 +252,6 @@ __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_
     while (next_e < x1 && issued - consumed < kStages) issue(next_e);
   };
 
-  const bool own_copy = a.rope == SELKV_ROPE_OFF;
   const int mi = lane >> 3, ri = lane & 7, g8 = lane >> 2, c4 = lane & 3;
   const bf16* Vb = static_cast<const bf16*>(a.V) + row_base * D;
   bf16* Vc = static_cast<bf16*>(a.Vc) + (size_t)bk * a.m_cap * D;
@@ -333,7 +375,7 @@ __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_
       }
       unsigned char* tile = smem + (consumed % kStages) * C::kTileBytes;
       const uint32_t T = smem_u32(tile);
-      if (e == X && own_copy) {
+      if (e == X) {
         // the kept rows but the target's, from the tile to their slots
         for (int r = sub; r < nk; r += RPI) {
           const int row = list[r];
@@ -485,13 +527,13 @@ cudaError_t launch_t(const CompressArgs& a, cudaStream_t s) {
   const cudaError_t e = set_smem_once<merge_mma_kernel<D>>(MCfg<D>::kSmem);
   if (e != cudaSuccess) return e;
   // Buckets per warp: up to 8 (a walk starts with two dependent rounds of loads), fewer where the
-  // warps would not fill the SMs.
+  // warps would not fill the SMs: one and a half times what would fill them with walks alone, which
+  // leaves room for the key warps in the same wave (8 heads x 16k: 3 buckets 18 us, 2 or 4 21).
   const int units = a.B * a.Hkv, nb = (a.n_cap + 31) / 32;
-  const long long per = (long long)units * nb / (kPlanSMs * kCtasPerSm);
+  const long long per = (long long)units * nb * 3 / (2 * kPlanSMs * kCtasPerSm);
   const int seg = (int)(per < 1 ? 1 : per > SELKV_MERGE_SEG ? SELKV_MERGE_SEG : per);
   const int walks = (nb + seg - 1) / seg;
-  // with repositioning copy_kernel writes the keys
-  const int keys = a.rope == SELKV_ROPE_OFF ? (a.m_cap + kKeySlots - 1) / kKeySlots : 0;
+  const int keys = (a.m_cap + kKeySlots - 1) / kKeySlots;
   launch_chained(a.chain, merge_mma_kernel<D>, dim3(walks + keys, units), 32, MCfg<D>::kSmem, s, tv, a, seg, walks);
   return cudaGetLastError();
 }

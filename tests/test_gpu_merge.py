@@ -27,14 +27,14 @@ def workload(n, d=128, heads=(8, 2), batch=2, rho=0.25):
                                                 num_kv_heads=heads[1], obs_window=24, rho=rho, ragged=(0.6, 1.0), seed=n)
 
 
-@pytest.mark.parametrize("mode", ["shared", "per_head", "rope", "drop"])
+@pytest.mark.parametrize("mode", ["shared", "per_head", "rope", "rope_pairs", "drop"])
 @pytest.mark.parametrize("n,d,rho", [(64, 128, 0.5), (65, 64, 0.3), (95, 128, 0.3), (257, 64, 0.1), (2049, 128, 0.02),
                                      (4000, 128, 0.008), (4000, 64, 0.6)])
 def test_merge_matches_the_oracle(n, d, rho, mode):
     wl = workload(n, d, rho=rho, batch=1 if n >= 4000 else 2)
     p = O.Params(recent=min(16, int(0.5 * rho * wl.n * 0.6)),
                  select_mode=O.SELECT_PER_HEAD if mode == "per_head" else O.SELECT_SHARED,
-                 rope=O.ROPE_HALF if mode == "rope" else O.ROPE_OFF,
+                 rope={"rope": O.ROPE_HALF, "rope_pairs": O.ROPE_INTERLEAVED}.get(mode, O.ROPE_OFF),
                  empty_bucket=O.EMPTY_DROP if mode == "drop" else O.EMPTY_EXPAND)
     x = synth.gen_layer(wl, 0)
     _, host, _ = run_compress(wl, x, p)

@@ -341,7 +341,21 @@ __global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_k
   Walk w0{walk.u0[group], walk.t0[group], walk.cnt[group], 0, 0, 0, 0, 0};
   w0.open(a, kKeys, walk.n[group]);
 
-  if (threadIdx.x == 0) {
+  // Loads of the producer's lane 0: a tile of keys, and the rows of the piece's Q.
+  auto load_tile = [&](const Walk& w, int t, int st) {
+    const int krow0 = (int)((size_t)w.u * a.n_cap) + w.t * kKeys;
+    mbar_arrive_expect_tx(&full[st], C::kKTile);
+    for (int bx = 0; bx < C::kBoxes; ++bx)
+      tma_load_2d(Ks + st * C::kKTile + bx * kKeys * 128, &tmK, bx * 64, krow0 + t * kKeys, &full[st]);
+  };
+  auto load_q = [&](const Walk& w) {
+    const int qrow0 = (w.b * a.Hq + w.kv * a.G) * a.W + h * kP1Rows;
+    mbar_arrive_expect_tx(qbar, C::kBoxes * Rq * 128);
+    for (int bx = 0; bx < C::kBoxes; ++bx)
+      for (int r0 = 0; r0 < Rq; r0 += 128) tma_load_2d(Qs + (bx * Rq + r0) * 128, &tmQ, bx * 64, qrow0 + r0, qbar);
+  };
+  const int early = w0.left > 0 ? min(kStages, w0.nt) : 0;  // tiles loaded before the CTA is set up
+  if (threadIdx.x == kProducerWarp * 32) {
     for (int i = 0; i < kStages; ++i) {
       mbar_init(&full[i], 1);
       mbar_init(&empty[i], 1);
@@ -362,7 +376,17 @@ __global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_k
     }
     *abort_flag = 0;
     fence_mbar_init();
+    // Q and the first tiles at once: K and Q are inputs of the call, complete before its first kernel
+    // starts, whatever the kernel before this one still does.
+    prefetch_tensormap(&tmQ);
+    prefetch_tensormap(&tmK);
+    if (early > 0) {
+      load_tile(w0, 0, 0);
+      load_q(w0);
+      for (int t = 1; t < early; ++t) load_tile(w0, t, t);
+    }
   }
+  __syncwarp();
   if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
   chain_begin();
   tc_fence_before();
@@ -372,36 +396,31 @@ __global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_k
 
   if (warp == kProducerWarp) {
     if (lane == 0) {
-      prefetch_tensormap(&tmQ);
-      prefetch_tensormap(&tmK);
       int tt = 0;      // tiles issued, over all pieces
       int pieces = 0;  // pieces whose Q is issued
       bool ok = true;
       for (Walk w = w0; ok && w.left > 0; w.next(a, kKeys)) {
-        const int krow0 = (int)((size_t)w.u * a.n_cap) + w.t * kKeys;
-        const int qrow0 = (w.b * a.Hq + w.kv * a.G) * a.W + h * kP1Rows;
         for (int t = 0; t <= w.nt; ++t) {
           // Q after the piece's first tile, which can be loaded while the last piece's MMAs still read theirs
           if (t == 1) {
-            if (pieces > 0) ok = mbar_wait(qfree, (pieces - 1) & 1);
-            if (!ok || *abort_flag) {
+            if (pieces > 0) {
+              if (!mbar_wait(qfree, (pieces - 1) & 1) || *abort_flag) {
+                ok = false;
+                break;
+              }
+              load_q(w);
+            }
+            ++pieces;  // (the first piece's was loaded above)
+          }
+          if (t == w.nt) break;
+          if (tt >= early) {
+            const int st = tt % kStages;
+            if (!mbar_wait(&empty[st], ((tt / kStages) & 1) ^ 1) || *abort_flag) {
               ok = false;
               break;
             }
-            mbar_arrive_expect_tx(qbar, C::kBoxes * Rq * 128);
-            for (int bx = 0; bx < C::kBoxes; ++bx)
-              for (int r0 = 0; r0 < Rq; r0 += 128) tma_load_2d(Qs + (bx * Rq + r0) * 128, &tmQ, bx * 64, qrow0 + r0, qbar);
-            ++pieces;
+            load_tile(w, t, st);
           }
-          if (t == w.nt) break;
-          const int st = tt % kStages;
-          if (!mbar_wait(&empty[st], ((tt / kStages) & 1) ^ 1) || *abort_flag) {
-            ok = false;
-            break;
-          }
-          mbar_arrive_expect_tx(&full[st], C::kKTile);
-          for (int bx = 0; bx < C::kBoxes; ++bx)
-            tma_load_2d(Ks + st * C::kKTile + bx * kKeys * 128, &tmK, bx * 64, krow0 + t * kKeys, &full[st]);
           ++tt;
         }
       }
@@ -775,7 +794,9 @@ cudaError_t launch_tc_t(CompressArgs a, const SeqTable& tab, cudaStream_t st, in
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  if (passes & kScoreColsums) launch_chained(a.chain, k2, groups2, cta_threads(2, H2, a.V != nullptr), C2::kSmem, st, tq, tk2, a, w2);
+  // (alone, pass 2 follows a kernel of the caller's and starts only after it)
+  const bool chain2 = a.chain && (passes & kScoreRowstats);
+  if (passes & kScoreColsums) launch_chained(chain2, k2, groups2, cta_threads(2, H2, a.V != nullptr), C2::kSmem, st, tq, tk2, a, w2);
   return cudaGetLastError();
 }
 

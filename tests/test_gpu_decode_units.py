@@ -1,0 +1,63 @@
+"""Decode of many short caches, whose units the CTAs walk longest first: ragged and equal lengths, empty
+and full caches, more sequences than one warp's lanes, several tokens in a row (the lengths advance
+once per token), against plain torch in 64 bits."""
+import math
+
+import pytest
+import torch
+
+from paper_2607_16213_gb300 import api
+import paper_2607_16213_gb300 as S
+
+from parity import DEC_BF16_MAX, DEC_BF16_MEAN
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_2607_16213_gb300 import build as b
+    b.build()
+    S.library()
+
+
+@pytest.mark.parametrize("B,hq,hkv,d,cap,lens", [
+    (64, 32, 8, 128, 896, "ragged"), (33, 16, 8, 64, 256, "ragged"), (160, 1, 1, 128, 192, "equal"),
+    (300, 8, 2, 128, 128, "ragged"), (77, 32, 2, 64, 2112, "ragged"), (1000, 4, 1, 64, 64, "edges"),
+    (40, 8, 4, 128, 320, "edges")])
+def test_tokens(B, hq, hkv, d, cap, lens):
+    g = torch.Generator(device="cuda").manual_seed(B + cap)
+    if lens == "ragged":
+        n = torch.randint(1, cap - 4, (B,), generator=g, device="cuda")
+    elif lens == "equal":
+        n = torch.full((B,), cap - 5, device="cuda")
+    else:  # around the 64-row steps, empty, and full but for one row
+        n = torch.tensor([0, 1, 63, 64, 65, cap - 4, cap - 1], device="cuda").clamp(max=cap - 1)[torch.arange(B, device="cuda") % 7]
+    n = n.int()
+    K, V = (torch.randn((B, hkv, cap, d), generator=g, device="cuda").bfloat16() for _ in range(2))
+    bias = torch.rand((B, hkv, cap), generator=g, device="cuda")
+    shape = api.make_shape("bf16", B, hq, hkv, d, 32, cap, cap)
+    lengths = torch.zeros(((B + 3) // 4 * 4,), dtype=torch.int32, device="cuda")
+    lengths[:B] = n
+    cache = api.CompressedCache(shape, K, V, bias, lengths)
+    ws = api.Workspace(S.selkv_decode_workspace_size(shape))
+    col = torch.arange(cap, device="cuda")
+    for token in range(3):
+        q = torch.randn((B, hq, d), generator=g, device="cuda").bfloat16()
+        kn, vn = (torch.randn((B, hkv, d), generator=g, device="cuda").bfloat16() for _ in range(2))
+        app = n + 1 <= cap
+        out = api.decode(cache, q, kn, vn, workspace=ws)
+        torch.cuda.synchronize()
+        # the row appended by this token is in the cache now, with bias 0
+        rows = torch.where(app, n + 1, n)
+        s = torch.einsum("bkgd,bknd->bkgn", q.view(B, hkv, hq // hkv, d).double(), K.double()) / math.sqrt(d)
+        s = (s + bias.double()[:, :, None]).masked_fill((col[None] >= rows[:, None])[:, None, None], -math.inf)
+        want = torch.einsum("bkgn,bknd->bkgd", torch.softmax(s, 3), V.double()).reshape(B, hq, d)
+        err = (out.double() - want).abs()
+        assert float(err.max()) <= DEC_BF16_MAX and float(err.mean()) <= DEC_BF16_MEAN
+        at = n.long().clamp(max=cap - 1)
+        b = torch.arange(B, device="cuda")
+        assert torch.equal(K[b, :, at][app], kn[app]) and torch.equal(V[b, :, at][app], vn[app])
+        n = rows.int()
+        assert torch.equal(lengths[:B], n)
+        assert ws.errors() == (0 if bool(app.all()) else S.SELKV_DEVERR_CAPACITY)

@@ -71,8 +71,9 @@ constexpr int kBoxRows = 64;   // TMA box height; split boundaries fall on multi
 constexpr int kHalves = kTile / kBoxRows;
 static_assert(kTile % kBoxRows == 0, "tile is whole boxes");
 
-template <int D>
+template <int D, int TILE = kTile>
 struct Cfg {
+  static constexpr int kTile = TILE, kConsumers = TILE / 16;
   static constexpr int kBoxes = D / 64;                // 128-byte-wide boxes per row
   static constexpr int kBoxBytes = kTile * 128;        // one 128-byte column of a tile
   static constexpr int kPieceBytes = kBoxRows * 128;   // one TMA box: kBoxRows rows x 128 bytes
@@ -675,14 +676,17 @@ __global__ __launch_bounds__(kThreads, SELKV_DEC_MINBLOCKS) void decode_tc_kerne
 // lengths (in 64-row steps), and CTA p takes unit p of that order, then 2P - 1 - p, 2P + p, ..., back
 // and forth, so that a long first unit is followed by a short one and the last, partial round has the
 // shortest.  In sequence order the longest share of a ragged batch carried the launch (64 sequences
-// of 409-819 rows, 8 KV heads: 50.3 us a launch, now 45.8).  The producer streams the next unit's tiles while the consumer warps fold the
+// of 409-819 rows, 8 KV heads: 50.3 us a launch against 45.8).  The producer streams the next unit's tiles while the consumer warps fold the
 // previous one (the ring runs on across units), so the start and drain of a CTA are paid once
 // per CTA instead of once per unit.  Each unit is held whole by one CTA: its fold is its output.
 // The group's queries (and the appended row) are staged in shared memory per unit, so the
 // mma fragments are not held in registers across the tiles.
-template <int D, bool ROWS16>
+template <int D, bool ROWS16, int TILE>
 struct UCfg {
-  using C = Cfg<D>;
+  using C = Cfg<D, TILE>;
+  static constexpr int kConsumers = C::kConsumers;
+  static constexpr int kThreads = (kConsumers + 1) * 32;
+  static constexpr int kCtasPerSm = TILE <= 64 ? 2 : 1;
   static constexpr int kRows = ROWS16 ? 16 : 8;          // group rows a warp state holds
   static constexpr int kFoldLd = D + 8;
   static constexpr int kFoldBytes = kConsumers * kRows * kFoldLd * 4;
@@ -743,12 +747,13 @@ __device__ __forceinline__ void order_by_length(const int* lengths, int B, bool 
   }
 }
 
-template <int D, bool ROWS16>
-__global__ __launch_bounds__(kThreads, 1) void decode_units_kernel(const __grid_constant__ CUtensorMap tmK,
+template <int D, bool ROWS16, int TILE>
+__global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TILE>::kCtasPerSm) void decode_units_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                    const __grid_constant__ CUtensorMap tmV,
                                                                    DecodeArgs a) {
-  using C = Cfg<D>;
-  using U = UCfg<D, ROWS16>;
+  using C = Cfg<D, TILE>;
+  using U = UCfg<D, ROWS16, TILE>;
+  constexpr int kTile = TILE, kConsumers = C::kConsumers, kHalves = TILE / kBoxRows;
   constexpr int NT = D / 8;
   constexpr int KS = D / 16;
   extern __shared__ unsigned char smem_raw[];
@@ -1142,6 +1147,18 @@ __global__ __launch_bounds__(kThreads, 1) void decode_units_kernel(const __grid_
   }
 }
 
+template <int D, bool R16, int TILE>
+cudaError_t launch_units_t(cudaLaunchConfig_t cfg, const CUtensorMap& tk, const CUtensorMap& tv, const DecodeArgs& a) {
+  using U = UCfg<D, R16, TILE>;
+  constexpr auto kern = decode_units_kernel<D, R16, TILE>;
+  const cudaError_t e = set_smem_once<kern>(U::kSmemBytes);
+  if (e != cudaSuccess) return e;
+  cfg.gridDim = dim3(kPlanSMs * U::kCtasPerSm);
+  cfg.blockDim = dim3(U::kThreads);
+  cfg.dynamicSmemBytes = U::kSmemBytes;
+  return cudaLaunchKernelEx(&cfg, kern, tk, tv, a);
+}
+
 template <int D, bool R16>
 cudaError_t launch_tc_t(const DecodeArgs& a, cudaStream_t st) {
   CUtensorMap tk, tv;
@@ -1159,11 +1176,13 @@ cudaError_t launch_tc_t(const DecodeArgs& a, cudaStream_t st) {
   if (SELKV_DEC_UNITS && a.splits == 1 && a.B * a.Hkv > kPlanSMs && a.m_cap <= SELKV_DEC_UNITS_MAX_ROWS) {
     // one split per (b, kv), more units than SMs, short units: persistent CTAs walk the units
     // (with longer units the static walk balances worse than the hardware's CTA scheduling)
-    cudaError_t e = set_smem_once<decode_units_kernel<D, R16>>(UCfg<D, R16>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    cfg.gridDim = dim3(kPlanSMs, 1, 1);
-    cfg.dynamicSmemBytes = UCfg<D, R16>::kSmemBytes;
-    return cudaLaunchKernelEx(&cfg, decode_units_kernel<D, R16>, tk, tv, a);
+    // 64-row tiles let two CTAs share an SM, so that one streams while the other folds a unit and fetches
+    // the next one's queries (512 units of 409-819 rows: 45.7 -> 39.4 us, 2048 of 200-400: 102 -> 80).
+    // With at most one unit for each of those CTAs a fold is paid once, and one CTA per SM balances
+    // better unless the units are short (256 units of 750-1500 rows: 37.1 us, 39.9 with two; 264 of
+    // 350-700: 25.0 and 23.1).
+    const bool one = a.B * a.Hkv <= 2 * kPlanSMs && a.m_cap > 1024;
+    return one ? launch_units_t<D, R16, 128>(cfg, tk, tv, a) : launch_units_t<D, R16, 64>(cfg, tk, tv, a);
   }
   cudaError_t e = set_smem_once<decode_tc_kernel<D, R16>>(Cfg<D>::kSmemBytes);
   if (e != cudaSuccess) return e;

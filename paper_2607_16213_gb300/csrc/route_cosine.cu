@@ -475,7 +475,7 @@ __global__ __launch_bounds__(256) void cos_scatter_kernel(CompressArgs a) {
 
 // ---- gated merge over each slot's contributors (Eq. 5, Eq. 6) ----------------------------
 constexpr int kMergeWarps = 8;
-constexpr int kBatch = 8;  // contributor rows in flight per lane
+constexpr int kBatch = 8;  // contributor rows in flight per lane (16: 44 us for one layer at 16k, 32: 65, 8: 33)
 
 template <typename T, int D>
 __global__ __launch_bounds__(kMergeWarps * 32) void cos_merge_kernel(CompressArgs a) {

@@ -280,7 +280,7 @@ int cosine_kernels(int dtype, int D);  // kernels launch_route_cosine enqueues
 // Chunks of the counting sort for caches of n_cap positions, and the chunk length.
 constexpr int kMaxCosChunks = 32;
 __host__ __device__ constexpr int cos_chunks_for(int n_cap) {
-  return n_cap <= 2048 ? 1 : (n_cap + 2047) / 2048 < kMaxCosChunks ? (n_cap + 2047) / 2048 : kMaxCosChunks;
+  return n_cap <= 1024 ? 1 : (n_cap + 1023) / 1024 < kMaxCosChunks ? (n_cap + 1023) / 1024 : kMaxCosChunks;
 }
 __host__ __device__ constexpr int cos_chunk_len(int n_cap) {
   return ((n_cap + cos_chunks_for(n_cap) - 1) / cos_chunks_for(n_cap) + 31) / 32 * 32;

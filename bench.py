@@ -634,7 +634,7 @@ def measure_scoring(L: Layered, S, api, torch, stream, dev, peaks, peak_src, rep
             "pass1_frac_burst": r1 / burst, "pass2_frac_burst": r2 / burst,
             "achieved": 2 * F / ((p1 + p2) * 1e-6) / 1e12, "frac": 2 * F / ((p1 + p2) * 1e-6) / 1e12 / peak,
             "useful_tflops_stage": stage, "useful_frac_stage": stage / peak,
-            "note": "pass 1 includes the sequence-table upload and the fold of the row statistics; "
+            "note": "pass 1 includes the sequence-table upload, pass 2 the fold of the row statistics; "
                     "achieved = executed flops of both passes over their time; useful = one product "
                     "(what the method needs) over the stage's time; peaks: sustained, and burst beside",
             "traffic": None}

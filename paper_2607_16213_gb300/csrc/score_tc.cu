@@ -47,10 +47,10 @@ static_assert(kP1Parts * 32 * SELKV_P1_CPW == SELKV_P1_KEYS && kP1Parts >= 1, "p
 // Both passes also carry the value norms of Eq. 1 (selkv_compress only) in a few more warps, half
 // of the rows each.  A kernel of its own for them, whether before the passes or beside them on
 // another stream, took all SMs first and cost its whole time (58 us for one layer of 8 x 100k
-// rows); the passes, bound by their epilogues at 60% of HBM, have room for its bytes: with them
-// 50 + 51 us become 62 + 56 us.  All rows in pass 1 make it wait for HBM (73 + 51 us).  Pass 2
-// has shared memory for three warps of two copies in flight, which bounds its share (three
-// quarters of the rows there: 57 + 72 us with two warps).
+// rows); the passes have room for its bytes: 50 + 53 us become 53 + 55.  All rows in pass 1 make it
+// wait for HBM (68 + 58 us with one row half per CTA), all in pass 2 wait for the three warps of
+// two copies in flight that its shared memory holds (50 + 78); shares of 3/8 and 5/8 in pass 1 are
+// within 2% of halves.  Two warps with as many bytes in flight are too slow (59 + 60 us).
 __host__ __device__ constexpr int norm_warps(int pass, int halves) { return pass == 1 && halves == 1 ? 4 : 3; }
 __host__ __device__ constexpr int norm_stages(int pass, int halves) { return pass == 1 && halves == 1 ? 3 : 2; }
 static_assert(4 * kP1Parts + 2 + norm_warps(1, 1) <= 32 && SELKV_P1_KEYS <= 256, "pass-1 warps per CTA");
@@ -62,7 +62,7 @@ __host__ __device__ constexpr int cta_threads(int pass, int halves, bool norms) 
 // Value norms of rows [row_lo, row_hi) by warp `w` of norm_warps.  The rows of a (sequence,
 // KV head) are contiguous, so lane 0 streams them as 4 KB bulk copies into the warp's own ring
 // (bytes in flight cost no registers; with 4 KB in registers per warp the round trips of eight
-// warps made pass 1 277 us for 64 x 8k where this takes 235).  D / 8 lanes take a row, 16 bytes a
+// warps made pass 1 277 us for 64 x 8k where this took 235).  D / 8 lanes take a row, 16 bytes a
 // lane: a lane squares its 8 elements in order and the lanes of a row meet in a butterfly; the
 // sums of a chunk's 8 row groups share it (each level keeps half of the values), pairing the
 // lanes as a butterfly per value does.  The copies are marked for early eviction from L2.

@@ -681,10 +681,24 @@ __global__ __launch_bounds__(kThreads, SELKV_DEC_MINBLOCKS) void decode_tc_kerne
 // per CTA instead of once per unit.  Each unit is held whole by one CTA: its fold is its output.
 // The group's queries (and the appended row) are staged in shared memory per unit, so the
 // mma fragments are not held in registers across the tiles.
+//
+// A warp's state covers the rows that it has with 128-row tiles: with 64-row tiles it takes the even
+// tiles of a unit first, puts that state away and takes the odd ones as a second state.  The running
+// max against which it rounds its weights to bf16, and with it the output, then do not depend on the
+// tile.
 template <int D, bool ROWS16, int TILE>
 struct UCfg {
   using C = Cfg<D, TILE>;
   static constexpr int kConsumers = C::kConsumers;
+  static constexpr int kStates = selkv::kConsumers;    // warp states of a unit
+  static constexpr int kRuns = kStates / kConsumers;   // states a warp goes through, one after the other
+  // the i-th of a unit's nt tiles: every kRuns-th one, kRuns times over
+  __device__ static __forceinline__ int tile_at(int i, int nt) {
+    static_assert(kRuns <= 2, "even tiles, then odd ones");
+    if (kRuns == 1) return i;
+    const int even = (nt + 1) / 2;
+    return i < even ? 2 * i : 2 * (i - even) + 1;
+  }
   static constexpr int kThreads = (kConsumers + 1) * 32;
   static constexpr int kCtasPerSm = TILE <= 64 ? 2 : 1;
   static constexpr int kRows = ROWS16 ? 16 : 8;          // group rows a warp state holds
@@ -694,7 +708,7 @@ struct UCfg {
   static constexpr int kQBytes = 16 * kQLd * 2 + 2 * D * 2;  // queries (16 rows), k_new, v_new
   // ring | fold scratch | queries | full, empty, pre [kStages] | abort | warp (max, sum), appended row
   static constexpr int kSmemBytes =
-      1024 + C::kRingBytes + kFoldBytes + kQBytes + 3 * kStages * 8 + 8 + 2 * (kConsumers + 1) * 16 * 4;
+      1024 + C::kRingBytes + kFoldBytes + kQBytes + 3 * kStages * 8 + 8 + 2 * (kStates + 1) * 16 * 4;
   static_assert((C::kRingBytes + kFoldBytes) % 16 == 0 && kQBytes % 16 == 0, "query rows 16-byte aligned");
 };
 
@@ -754,6 +768,7 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
   using C = Cfg<D, TILE>;
   using U = UCfg<D, ROWS16, TILE>;
   constexpr int kTile = TILE, kConsumers = C::kConsumers, kHalves = TILE / kBoxRows;
+  constexpr int kStates = U::kStates, kRuns = U::kRuns;
   constexpr int NT = D / 8;
   constexpr int KS = D / 16;
   extern __shared__ unsigned char smem_raw[];
@@ -766,9 +781,9 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
   uint64_t* empty = full + kStages;
   uint64_t* pre = empty + kStages;
   volatile int* s_abort = reinterpret_cast<volatile int*>(pre + kStages);
-  float* wm = reinterpret_cast<float*>(pre + kStages + 1);  // [kConsumers][16]
-  float* wl = wm + kConsumers * 16;                         // [kConsumers][16]
-  float* apm = wl + kConsumers * 16;                        // [16] appended row's logit
+  float* wm = reinterpret_cast<float*>(pre + kStages + 1);  // [kStates][16]
+  float* wl = wm + kStates * 16;                            // [kStates][16]
+  float* apm = wl + kStates * 16;                        // [16] appended row's logit
   float* apw = apm + 16;                                    // [16] its weight / the normaliser
   __shared__ int s_pre_n, s_pre_u;  // early loads: tiles, and the unit they are of
   __shared__ float s_inv[16];  // 1 / normaliser per query head of the unit
@@ -807,11 +822,11 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
       const int Lg = min(max(ld_relaxed_gpu(a.lengths + b), 0), a.m_cap);
       const int safe = Lg - 1;
       const int max_pre = Lg >= SELKV_DEC_PRELOAD_MIN * kTile ? min(kStages, SELKV_DEC_PRELOAD) : 0;
-      for (; npre < max_pre && (npre + 1) * kTile <= safe; ++npre) {
+      for (; npre < max_pre && (npre * kRuns + 1) * kTile <= safe; ++npre) {
         unsigned char* base = smem + npre * C::kStageBytes;
         mbar_arrive_expect_tx(&pre[npre], C::kStageBytes);
         for (int h = 0; h < kHalves; ++h) {
-          const int y = (int)(bk * a.m_cap) + npre * kTile + h * kBoxRows;
+          const int y = (int)(bk * a.m_cap) + npre * kRuns * kTile + h * kBoxRows;
 #pragma unroll
           for (int bx = 0; bx < C::kBoxes; ++bx)
             tma_load_2d(base + bx * C::kBoxBytes + h * C::kPieceBytes, &tmK, bx * 64, y, &pre[npre]);
@@ -846,8 +861,8 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
         const int L = min(max(a.lengths[u / a.Hkv], 0), a.m_cap);
         const int nt = (L + kTile - 1) / kTile;
         const int row0 = (int)((size_t)u * a.m_cap);
-        for (int t = 0; t < nt; ++t) {
-          const int tg = issued, st = tg % kStages;
+        for (int i = 0; i < nt; ++i) {
+          const int t = U::tile_at(i, nt), tg = issued, st = tg % kStages;
           if (!mbar_wait(&empty[st], ((tg / kStages) & 1) ^ 1)) {
             *s_abort = 1;
             raise_flag(a.flags, SELKV_DEVERR_TIMEOUT);
@@ -867,7 +882,7 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
               break;
             }
             pre_seen |= 1u << st;
-            if (k == 0 && u == s_pre_u && (t + 1) * kTile <= L) {
+            if (k == 0 && u == s_pre_u && t == i * kRuns && (t + 1) * kTile <= L) {
               mbar_arrive(&full[st]);  // the tile is already in place
               issued = tg + 1;
               continue;
@@ -909,11 +924,7 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
     const bool app = has_new && L + 1 <= a.m_cap;
     const int nt = (L + kTile - 1) / kTile;
     float o[NT][4];
-    float mrow[2] = {-INFINITY, -INFINITY}, lrow[2] = {0.f, 0.f};
-#pragma unroll
-    for (int n8 = 0; n8 < NT; ++n8)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) o[n8][e] = 0.f;
+    float mrow[2], lrow[2];
     {
       const __nv_bfloat16* qg = static_cast<const __nv_bfloat16*>(a.q) + ((size_t)b * a.Hq + (size_t)(u - b * a.Hkv) * G) * D;
       for (int i = tid; i < 16 * (D / 8); i += kCons) {
@@ -947,15 +958,63 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
           dst[n2][e] = (brow != nullptr && key < L) ? __ldg(brow + key) * kLog2e : 0.f;
         }
     };
+    const bool two = kRuns > 1 && nt > 1;  // the warp goes through two states
+    auto clear_state = [&]() {
+      // (a zero that the compiler does not know: with a known one the same launch spills
+      // and takes 44.3 us in place of 41.2 for 512 units of 409-819 rows)
+      float zero = 0.f;
+      asm volatile("" : "+f"(zero));
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        mrow[r] = -INFINITY;
+        lrow[r] = zero;
+      }
+#pragma unroll
+      for (int n8 = 0; n8 < NT; ++n8)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[n8][e] = zero;
+    };
+    // a state's output, times f, into the warp's rows of the scratch
+    auto put_output = [&](float fa, float fb) {
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const int g = g0 + r * 8;
+        if (g >= G) continue;
+        const float f = r == 0 ? fa : fb;
+#pragma unroll
+        for (int n8 = 0; n8 < NT; ++n8)
+          *reinterpret_cast<float2*>(wo + (warp * U::kRows + g) * U::kFoldLd + n8 * 8 + c2) =
+              make_float2(o[n8][r * 2] * f, o[n8][r * 2 + 1] * f);
+      }
+    };
+    // (max, sum) of the warp's run-th state
+    auto put_stats = [&](int run) {
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        lrow[r] += __shfl_xor_sync(0xffffffffu, lrow[r], 1);
+        lrow[r] += __shfl_xor_sync(0xffffffffu, lrow[r], 2);
+        const int g = g0 + r * 8;
+        if ((lane & 3) != 0 || g >= G) continue;
+        wm[(run * kConsumers + warp) * 16 + g] = mrow[r];
+        wl[(run * kConsumers + warp) * 16 + g] = lrow[r];
+      }
+    };
+    clear_state();
     float bnext[2][2];
     if (nt > 0) fetch_bias(0, bnext);
-    for (int t = 0; t < nt; ++t, ++tg) {
+    for (int i = 0; i < nt; ++i, ++tg) {
+      const int t = U::tile_at(i, nt);
+      if (kRuns > 1 && t == 1) {
+        put_stats(0);
+        put_output(1.f, 1.f);
+        clear_state();
+      }
       float bv[2][2];
 #pragma unroll
       for (int n2 = 0; n2 < 2; ++n2)
 #pragma unroll
         for (int e = 0; e < 2; ++e) bv[n2][e] = bnext[n2][e];
-      if (t + 1 < nt) fetch_bias(t + 1, bnext);
+      if (i + 1 < nt) fetch_bias(U::tile_at(i + 1, nt), bnext);
       const int st = tg % kStages;
       if (!__all_sync(0xffffffffu, *s_abort == 0)) break;
       if (!__all_sync(0xffffffffu, mbar_wait(&full[st], (tg / kStages) & 1))) {
@@ -1050,10 +1109,10 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[st]);
     }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      lrow[r] += __shfl_xor_sync(0xffffffffu, lrow[r], 1);
-      lrow[r] += __shfl_xor_sync(0xffffffffu, lrow[r], 2);
+    put_stats(two ? 1 : 0);
+    if (kRuns > 1 && !two && lane < G) {  // no tile for the second
+      wm[(kConsumers + warp) * 16 + lane] = -INFINITY;
+      wl[(kConsumers + warp) * 16 + lane] = 0.f;
     }
     // Fold the warp states (and the appended row, bias 0) into the unit's output, among the
     // consumer warps only: the producer is already loading the next unit.
@@ -1066,34 +1125,30 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
         if (lane == 0) apm[g] = part;
       }
     }
-    if ((lane & 3) == 0) {
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const int g = g0 + r * 8;
-        if (g >= G) continue;
-        wm[warp * 16 + g] = mrow[r];
-        wl[warp * 16 + g] = lrow[r];
-      }
-    }
     named_bar_sync(kBar, kCons);
     const bool aborted = *s_abort != 0;
+    float f[2] = {0.f, 0.f};  // 2^(max of this lane's state - max of all)
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const int g = g0 + r * 8;
       if (g >= G) continue;
       float M = app ? apm[g] : -INFINITY;
 #pragma unroll
-      for (int w = 0; w < kConsumers; ++w) M = fmaxf(M, wm[w * 16 + g]);
-      const float f = M == -INFINITY ? 0.f : exp2f(mrow[r] - M);
+      for (int w = 0; w < kStates; ++w) M = fmaxf(M, wm[w * 16 + g]);
+      f[r] = M == -INFINITY ? 0.f : exp2f(mrow[r] - M);
+      if (two) {  // (each lane its own words)
+        const float f1 = M == -INFINITY ? 0.f : exp2f(wm[warp * 16 + g] - M);
 #pragma unroll
-      for (int n8 = 0; n8 < NT; ++n8)
-        *reinterpret_cast<float2*>(wo + (warp * U::kRows + g) * U::kFoldLd + n8 * 8 + c2) =
-            make_float2(o[n8][r * 2] * f, o[n8][r * 2 + 1] * f);
+        for (int n8 = 0; n8 < NT; ++n8) {
+          float2* x = reinterpret_cast<float2*>(wo + (warp * U::kRows + g) * U::kFoldLd + n8 * 8 + c2);
+          *x = make_float2(x->x * f1, x->y * f1);
+        }
+      }
       if (warp == 0 && (lane & 3) == 0) {
         float Ls = 0.f;
         if (M != -INFINITY) {
 #pragma unroll
-          for (int w = 0; w < kConsumers; ++w) Ls = fmaf(wl[w * 16 + g], exp2f(wm[w * 16 + g] - M), Ls);
+          for (int w = 0; w < kStates; ++w) Ls = fmaf(wl[w * 16 + g], exp2f(wm[w * 16 + g] - M), Ls);
         }
         const float wa = app ? exp2f(apm[g] - M) : 0.f;  // M >= apm[g] > -inf when app
         Ls += wa;
@@ -1102,22 +1157,44 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
         s_inv[g] = inv;
       }
     }
+    if (!two) put_output(f[0], f[1]);
     named_bar_sync(kBar, kCons);
     {
-      constexpr int D4 = D / 4;
-      for (int i = tid; i < G * D4; i += kCons) {
-        const int g = i / D4, d4 = i % D4;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      // the states are added in their order: the scratch holds one of each warp at a time
+      constexpr int D4 = D / 4, kItems = (U::kRows * D4 + kCons - 1) / kCons;
+      float4 acc[kItems];
 #pragma unroll
-        for (int w = 0; w < kConsumers; ++w) {
-          const float4 v = *reinterpret_cast<const float4*>(wo + (w * U::kRows + g) * U::kFoldLd + d4 * 4);
-          acc.x += v.x;
-          acc.y += v.y;
-          acc.z += v.z;
-          acc.w += v.w;
+      for (int k4 = 0; k4 < kItems; ++k4) acc[k4] = make_float4(0.f, 0.f, 0.f, 0.f);
+      auto add_states = [&]() {
+#pragma unroll
+        for (int k4 = 0; k4 < kItems; ++k4) {
+          const int i = k4 * kCons + tid;
+          if (i >= G * D4) break;
+          const int g = i / D4, d4 = i % D4;
+#pragma unroll
+          for (int w = 0; w < kConsumers; ++w) {
+            const float4 v = *reinterpret_cast<const float4*>(wo + (w * U::kRows + g) * U::kFoldLd + d4 * 4);
+            acc[k4].x += v.x;
+            acc[k4].y += v.y;
+            acc[k4].z += v.z;
+            acc[k4].w += v.w;
+          }
         }
+      };
+      add_states();
+      if (two) {
+        named_bar_sync(kBar, kCons);  // the first states are added
+        put_output(f[0], f[1]);
+        named_bar_sync(kBar, kCons);
+        add_states();
+      }
+#pragma unroll
+      for (int k4 = 0; k4 < kItems; ++k4) {
+        const int i = k4 * kCons + tid;
+        if (i >= G * D4) break;
+        const int g = i / D4, d4 = i % D4;
         const float inv = s_inv[g];
-        float r[4] = {acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv};
+        float r[4] = {acc[k4].x * inv, acc[k4].y * inv, acc[k4].z * inv, acc[k4].w * inv};
         if (app) {
           const float wa = apw[g];
           const __nv_bfloat16* vn = snew + D + d4 * 4;
@@ -1177,10 +1254,10 @@ cudaError_t launch_tc_t(const DecodeArgs& a, cudaStream_t st) {
     // one split per (b, kv), more units than SMs, short units: persistent CTAs walk the units
     // (with longer units the static walk balances worse than the hardware's CTA scheduling)
     // 64-row tiles let two CTAs share an SM, so that one streams while the other folds a unit and fetches
-    // the next one's queries (512 units of 409-819 rows: 45.7 -> 39.4 us, 2048 of 200-400: 102 -> 80).
-    // With at most one unit for each of those CTAs a fold is paid once, and one CTA per SM balances
-    // better unless the units are short (256 units of 750-1500 rows: 37.1 us, 39.9 with two; 264 of
-    // 350-700: 25.0 and 23.1).
+    // the next one's queries (512 units of 409-819 rows: 48.0 -> 41.2 us, 2048 of 200-400: 106 -> 85).
+    // With at most one unit for each of those CTAs a fold is paid once, and one CTA per SM is as fast or
+    // faster unless the units are short (256 units of 750-1500 rows: 40.1 us, 41.0 with two; 264 of
+    // 350-700: 26.0 and 23.8).
     const bool one = a.B * a.Hkv <= 2 * kPlanSMs && a.m_cap > 1024;
     return one ? launch_units_t<D, R16, 128>(cfg, tk, tv, a) : launch_units_t<D, R16, 64>(cfg, tk, tv, a);
   }

@@ -61,3 +61,24 @@ def test_tokens(B, hq, hkv, d, cap, lens):
         n = rows.int()
         assert torch.equal(lengths[:B], n)
         assert ws.errors() == (0 if bool(app.all()) else S.SELKV_DEVERR_CAPACITY)
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(32, 8, 128), (128, 8, 128), (16, 8, 64)])
+def test_the_output_does_not_depend_on_the_tile(hq, hkv, d):
+    """Up to 304 units of more than 1024 rows are walked in 128-row tiles, more of them in 64-row
+    tiles: the same sequences, once alone and once among copies of themselves, give the same bits."""
+    B, cap = 20, 1088
+    g = torch.Generator(device="cuda").manual_seed(hq + d)
+    K, V = (torch.randn((B, hkv, cap, d), generator=g, device="cuda").bfloat16() for _ in range(2))
+    bias = torch.rand((B, hkv, cap), generator=g, device="cuda")
+    n = torch.randint(1, cap - 1, (B,), generator=g, device="cuda").int()
+    n[:7] = torch.tensor([1, 16, 64, 65, 128, 129, cap - 1])
+    q = torch.randn((B, hq, d), generator=g, device="cuda").bfloat16()
+    kn, vn = (torch.randn((B, hkv, d), generator=g, device="cuda").bfloat16() for _ in range(2))
+    outs = []
+    for copies in (1, 2):
+        both = [x.repeat(copies, *[1] * (x.dim() - 1)) for x in (K, V, bias, n, q, kn, vn)]
+        shape = api.make_shape("bf16", B * copies, hq, hkv, d, 32, cap, cap)
+        cache = api.CompressedCache(shape, *both[:4])
+        outs.append(api.decode(cache, *both[4:]))
+    assert torch.equal(outs[1][:B], outs[0]) and torch.equal(outs[1][B:], outs[0])

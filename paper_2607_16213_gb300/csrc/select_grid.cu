@@ -46,6 +46,14 @@ __device__ __forceinline__ void cluster_sync(int cs) {
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
 }
+// The two halves of a first barrier of the cluster: shared memory of another CTA may be touched only
+// once that CTA runs.  The work between the halves hides the wait.
+__device__ __forceinline__ void cluster_started_arrive(int cs) {
+  if (cs > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_started_wait(int cs) {
+  if (cs > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ uint32_t peer_addr(const void* p, int rank) {
   uint32_t a;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
@@ -340,6 +348,7 @@ __device__ __forceinline__ void compact(const CompressArgs& a, Shared<NT>& sh, c
 template <int POOL, int NT>
 __global__ __launch_bounds__(NT) void topk_kernel(CompressArgs a, SelectWs w, int near_keys) {
   chain_begin();
+  cluster_started_arrive(gridDim.x);
   __shared__ Shared<NT> sh;
   extern __shared__ uint32_t dyn_keys[];
   const int u = blockIdx.y, b = u / a.Hkv, lane = threadIdx.x & 31;
@@ -384,6 +393,7 @@ __global__ __launch_bounds__(NT) void topk_kernel(CompressArgs a, SelectWs w, in
       if (near_keys) s.keys[i] = __float_as_uint(v);
     }
   }
+  cluster_started_wait(s.cs);
   uint32_t T = 0u;  // select every candidate ...
   int jcut = INT_MAX;
   if (k <= 0) {
@@ -410,6 +420,7 @@ __global__ __launch_bounds__(NT) void topk_kernel(CompressArgs a, SelectWs w, in
 template <int NT>
 __global__ __launch_bounds__(NT) void trim_kernel(CompressArgs a, SelectWs w, int near_keys) {
   chain_begin();
+  cluster_started_arrive(gridDim.x);
   __shared__ Shared<NT> sh;
   __shared__ RadixCut cut[32];
   extern __shared__ uint32_t dyn_keys[];
@@ -476,6 +487,7 @@ __global__ __launch_bounds__(NT) void trim_kernel(CompressArgs a, SelectWs w, in
             j < ncand && (x > cut[kv].T || (x == cut[kv].T && j <= cut[kv].jcut));
       }
     }
+  cluster_started_wait(s.cs);
   scan_cluster(sh, s, 0, cnt, members);
   uint32_t T = 0u;
   int jcut = INT_MAX;

@@ -73,3 +73,26 @@ def test_selection_matches_a_plain_top_k(hkv, lens, pool, per_head, tied):
         union = heads.any(axis=0)
         chosen = top(total, union, ms) if union.sum() > ms else union
         np.testing.assert_array_equal(kept_idx[b, :m], np.append(np.flatnonzero(chosen), np.arange(ncand, nb)))
+
+
+@pytest.mark.parametrize("per_head", [False, True])
+@pytest.mark.parametrize("rho,recent", [(1.0, 16), (1.0, 0), (0.25, 1025)])
+@pytest.mark.parametrize("hkv,n", [(8, 4101), (1, 4101)])
+def test_every_candidate_or_none(hkv, n, rho, recent, per_head):
+    """No threshold is searched for, so the compaction's counts are the first that the CTAs of a
+    cluster tell each other (rho 1: all kept; m = recent: the recent window alone)."""
+    d, W = 64, 32
+    g = torch.Generator(device="cuda").manual_seed(n + hkv)
+    K, V = (torch.randn((2, hkv, n, d), generator=g, device="cuda").bfloat16() for _ in range(2))
+    Q = torch.randn((2, hkv, W, d), generator=g, device="cuda").bfloat16()
+    shape = api.make_shape("bf16", 2, hkv, hkv, d, W, n, api.capacity(n, rho))
+    params = S.selkv_params.defaults(recent=recent,
+                                     select_mode=S.SELKV_SELECT_PER_HEAD if per_head else S.SELKV_SELECT_SHARED)
+    ws = api.Workspace(S.selkv_compress_workspace_size(shape))
+    c = api.compress(shape, [n, n], rho, K, V, Q, params, debug=True, workspace=ws)
+    torch.cuda.synchronize()
+    assert ws.errors() == 0
+    m = int(rho * n)
+    kept = c.debug["kept_idx"].cpu().numpy()[..., :m].reshape(-1, m)
+    np.testing.assert_array_equal(kept, np.broadcast_to(np.arange(n - m, n), kept.shape))
+    assert bool(c.debug["topk"][:, :, :n - recent].all()) == (rho == 1.0)

@@ -93,7 +93,7 @@ CompressPlan plan_compress(const selkv_shape& s) {
 }
 
 struct ScorePlan {
-  size_t seq_n, seq_m, seq_t1, rowpart, rowstat, total;
+  size_t seq_n, seq_m, seq_t1, walk, rowpart, rowstat, total;
   int nchunks, R;
 };
 
@@ -111,6 +111,7 @@ ScorePlan plan_score(const selkv_shape& s) {
   p.seq_n = take(B * 4);
   p.seq_m = take(B * 4);
   p.seq_t1 = take(B * 4);
+  p.walk = take(sizeof(ScoreWalk));
   p.rowpart = take(score_partials(s, p.R) * p.R * sizeof(float2));
   p.rowstat = take(B * Hkv * (size_t)p.R * sizeof(float2));
   p.total = off;
@@ -407,14 +408,15 @@ selkv_status selkv_score(const selkv_shape* shape, const int32_t* n_len, const v
   a.seq_n = at<int32_t>(workspace, plan.seq_n);
   a.seq_m = at<int32_t>(workspace, plan.seq_m);
   a.seq_t1 = at<int32_t>(workspace, plan.seq_t1);
+  a.p2_walk = at<ScoreWalk>(workspace, plan.walk);
   a.rowpart = at<float2>(workspace, plan.rowpart);
   a.rowstat = at<float2>(workspace, plan.rowstat);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   a.chain = may_chain(st);
   cudaError_t e = cudaSuccess;
   int kernels = 0;
-  if (passes & SELKV_SCORE_ROWSTATS) {  // the column-sum pass reuses the table of its row-statistics call
-    e = launch_seq_setup(a, tab, st);
+  if (passes & SELKV_SCORE_ROWSTATS) {  // a column-sum call reuses the table and shares of its row-statistics call
+    e = launch_seq_setup(a, tab, score_uses_tc(a.dtype, a.D, a.R) ? plan_colsums(a, tab) : ScoreWalk{}, st);
     kernels += score_uses_tc(a.dtype, a.D, a.R) ? 2 : 3;
   }
   if (passes & SELKV_SCORE_COLSUMS) kernels += 1;

@@ -39,6 +39,7 @@ constexpr uint32_t kTmemCols = 512;  // two accumulators of up to 256 fp32 colum
 #ifndef SELKV_P1_CPW
 #define SELKV_P1_CPW 2     // pass 1: 32-column accumulator chunks per epilogue warp and tile
 #endif
+constexpr int kP2Keys = 128;  // pass 2: keys per tile
 // Epilogue warps: pass 1 splits a tile's keys over the warps of each TMEM lane quarter (32
 // columns x SELKV_P1_CPW per warp), pass 2 splits the rows over four warps per lane quarter.
 // A TMA producer warp and an MMA warp follow them.
@@ -190,7 +191,7 @@ __device__ __forceinline__ float colsum64(uint32_t taddr, uint32_t rn, float sc)
 // for the 512 staged rows.
 template <int D, int PASS, int HALVES = 1>
 struct SCfg {
-  static constexpr int kKeys = PASS == 1 ? SELKV_P1_KEYS : 128;        // keys per tile
+  static constexpr int kKeys = PASS == 1 ? SELKV_P1_KEYS : kP2Keys;    // keys per tile
   static constexpr int kStages = PASS == 1 ? 2 : (HALVES == 2 ? 2 : 4);  // K tiles in flight
   static constexpr int kRows = (PASS == 1 ? 128 : 256) * HALVES;        // Q rows staged per CTA
   static constexpr int kBoxes = D / 64;                  // 128-byte-wide boxes per row
@@ -243,9 +244,9 @@ __host__ __device__ __forceinline__ Partials partials_of(int split, int per, int
   }
   return {c0 + u, c1 - c0 + 1};
 }
-__device__ __forceinline__ Partials partials_of(const CompressArgs& a, const Walk& w) {
+__device__ __forceinline__ Partials partials_of(const CompressArgs& a, const ScoreWalk& s, const Walk& w) {
   const int T1 = (w.n + SELKV_P1_KEYS - 1) / SELKV_P1_KEYS;
-  return partials_of(a.p1_split, a.p1_per, w.u, a.p1_split > 0 ? 0 : a.seq_t1[w.b] * a.Hkv + w.kv * T1, T1);
+  return partials_of(s.p1_split, s.p1_per, w.u, s.p1_split > 0 ? 0 : a.seq_t1[w.b] * a.Hkv + w.kv * T1, T1);
 }
 
 // Fold of the partials of row r: -(M + log2(G Z)), the row's whole normaliser as one exponent offset
@@ -291,11 +292,13 @@ __device__ __forceinline__ float rowsum32(const float (&v)[32], float sc, float 
   return (s0 + s1) + (s2 + s3);
 }
 
-template <int D, int PASS, int HALVES>
+// TABLE (pass 2 in a call of its own): the shares are those that the call with pass 1 left in the
+// workspace, which go with its lengths there; otherwise they come with the launch.
+template <int D, int PASS, int HALVES, bool TABLE = false>
 __global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
                                                                         const __grid_constant__ CUtensorMap tmK,
                                                                         CompressArgs a,
-                                                                        const __grid_constant__ ScoreWalk walk) {
+                                                                        const __grid_constant__ ScoreWalk shares) {
   using C = SCfg<D, PASS, HALVES>;
   constexpr int kEpiWarps = epi_warps(PASS);
   constexpr int kProducerWarp = kEpiWarps, kMmaWarp = kEpiWarps + 1;
@@ -338,6 +341,7 @@ __global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_k
   const int group = PASS == 1 ? (int)blockIdx.x / MT : (int)blockIdx.x;  // CTAs with the same tiles
   const int nph = PASS == 1 ? min(HALVES, (R - h * kP1Rows + 127) / 128) : HALVES;  // row halves in use
   const int Rq = PASS == 1 ? kP1Rows : (HALVES == 2 ? 512 : (R > 128 ? 256 : 128));  // Q rows staged (whole boxes)
+  const ScoreWalk& walk = TABLE ? *a.p2_walk : shares;
   Walk w0{walk.u0[group], walk.t0[group], walk.cnt[group], 0, 0, 0, 0, 0};
   w0.open(a, kKeys, walk.n[group]);
 
@@ -609,7 +613,7 @@ __global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_k
           // (Q of the piece and its first tiles are on their way meanwhile)
           const int r = threadIdx.x;
           // the first unit's partials from the table: its chain of loads is not hidden by earlier tiles
-          const Partials ps = w.left == w0.left ? Partials{walk.part0[group], walk.parts[group]} : partials_of(a, w);
+          const Partials ps = w.left == w0.left ? Partials{walk.part0[group], walk.parts[group]} : partials_of(a, walk, w);
           const float x = r < R ? fold_row_tc(a, ps, r) : -INFINITY;
           if (w.left < w0.left) named_bar_sync(1, kEpiWarps * 32);  // the last piece's rows are done with
           if (r < 256 * HALVES) {
@@ -713,13 +717,20 @@ __global__ __launch_bounds__(cta_threads(PASS, HALVES, true), 1) void score_tc_k
   }
 }
 
+// How pass 1 cuts the tiles: row halves per CTA, splits per unit (or 0) and tiles per CTA group.
+struct P1Cut {
+  int halves, split, per;
+};
+
 // Shares of a pass's key tiles: `groups` CTAs (of `row_parts` each in pass 1) with the same number of
 // consecutive tiles of all units, which crosses from one unit to the next; or, where it is no more tiles
 // for the longest unit, every unit cut into the same number of splits, with no crossing.  A fixed grid of
 // splits per unit left SMs idle where the units did not divide them (32 heads: 128 of 152 CTAs) or had
 // unequal lengths (8 ragged prompts of 32k: passes 131 + 146 us, now 91 + 96; 64 of 8k: 233 + 284, now
 // 195 + 221).  A crossing costs a reload of Q while the epilogue works on the two tiles in flight.
-int plan_walk(const CompressArgs& a, const SeqTable& tab, int row_parts, int keys, ScoreWalk& w, int& split, int& per) {
+// `p1`: for pass 2, pass 1's plan.
+int plan_walk(const CompressArgs& a, const SeqTable& tab, int row_parts, int keys, ScoreWalk& w, int& split, int& per,
+              const P1Cut* p1 = nullptr) {
   const int groups = kPlanSMs / row_parts;
   const int units = a.B * a.Hkv;
   auto tiles = [&](int b) { return (tab.n[b] + keys - 1) / keys; };
@@ -757,18 +768,44 @@ int plan_walk(const CompressArgs& a, const SeqTable& tab, int row_parts, int key
   for (int c = 0; c < used; ++c) {
     const int b = w.u0[c] / a.Hkv;
     w.n[c] = tab.n[b];
-    // (pass 2, after pass 1 has been planned)
+    if (p1 == nullptr) continue;
     const int T1 = score_tc_tiles1(tab.n[b]);
-    const Partials ps = a.p1_per > 0 ? partials_of(a.p1_split, a.p1_per, w.u0[c], tab.t1[b] * a.Hkv + w.u0[c] % a.Hkv * T1, T1)
-                                     : Partials{0, 0};
+    const Partials ps = partials_of(p1->split, p1->per, w.u0[c], tab.t1[b] * a.Hkv + w.u0[c] % a.Hkv * T1, T1);
     w.part0[c] = ps.first;
     w.parts[c] = ps.count;
   }
   return used;
 }
 
+// Row halves of a CTA in pass 1.  Two 128-row halves read a tile's keys once for both, where two CTAs with
+// a half each read them twice (from L2, or HBM where they drift apart: 8 x 32k 100 -> 90 us, 64 x 8k
+// 215 -> 197); but a CTA's share is then twice as coarse.  From 8 tiles (16 accumulators) a CTA on, unless
+// rounding to whole tiles makes it longer (16k: 8 accumulators against 7, 18.9 against 16.4 us).
+int p1_halves(const CompressArgs& a, const SeqTable& tab) {
+  long long total = 0;
+  for (int b = 0; b < a.B; ++b) total += (long long)score_tc_tiles1(tab.n[b]) * a.Hkv;
+  auto accs = [&](int halves) {  // accumulators of the longest share
+    const int groups = kPlanSMs / ((a.R + 128 * halves - 1) / (128 * halves));
+    return (total + groups - 1) / groups * halves;
+  };
+  return a.R > 128 && accs(2) >= 16 && accs(2) <= accs(1) ? 2 : 1;
+}
+int p1_row_parts(int R, int halves) { return (R + 128 * halves - 1) / (128 * halves); }
+
+// Both passes' shares: the CTA groups of pass 1 and the CTAs of pass 2.
+void plan_passes(const CompressArgs& a, const SeqTable& tab, ScoreWalk& w1, ScoreWalk& w2, P1Cut& cut, int& groups1,
+                 int& groups2) {
+  cut.halves = p1_halves(a, tab);
+  groups1 = plan_walk(a, tab, p1_row_parts(a.R, cut.halves), SELKV_P1_KEYS, w1, cut.split, cut.per);
+  int split2, per2;
+  groups2 = plan_walk(a, tab, 1, kP2Keys, w2, split2, per2, &cut);
+  w2.p1_split = cut.split;
+  w2.p1_per = cut.per;
+}
+
 template <int D, int H1, int H2>
-cudaError_t launch_tc_t(CompressArgs a, const SeqTable& tab, cudaStream_t st, int passes) {
+cudaError_t launch_tc_t(const CompressArgs& a, const ScoreWalk& w1, const ScoreWalk& w2, int groups1, int groups2,
+                        cudaStream_t st, int passes) {
   using C1 = SCfg<D, 1, H1>;
   using C2 = SCfg<D, 2, H2>;
   CUtensorMap tq, tk1, tk2;
@@ -776,27 +813,26 @@ cudaError_t launch_tc_t(CompressArgs a, const SeqTable& tab, cudaStream_t st, in
       !encode_rows_bf16(&tk1, a.K, (uint64_t)a.B * a.Hkv * a.n_cap, D, C1::kKeys) ||
       !encode_rows_bf16(&tk2, a.K, (uint64_t)a.B * a.Hkv * a.n_cap, D, C2::kKeys))
     return cudaErrorInvalidValue;
-  const int MT = (a.R + 128 * H1 - 1) / (128 * H1);
-  ScoreWalk w1{}, w2{};
-  int split2, per2;
-  int split1, per1;
-  const int groups1 = plan_walk(a, tab, MT, C1::kKeys, w1, split1, per1);
-  a.p1_split = split1;
-  a.p1_per = per1;
-  const int groups2 = plan_walk(a, tab, 1, C2::kKeys, w2, split2, per2);
-  auto k1 = score_tc_kernel<D, 1, H1>;
-  auto k2 = score_tc_kernel<D, 2, H2>;
-  cudaError_t e = set_smem_once<score_tc_kernel<D, 1, H1>>(C1::kSmem);
-  if (e == cudaSuccess) e = set_smem_once<score_tc_kernel<D, 2, H2>>(C2::kSmem);
-  if (e != cudaSuccess) return e;
   if (passes & kScoreRowstats) {
-    launch_chained(a.chain, k1, groups1 * MT, cta_threads(1, H1, a.V != nullptr), C1::kSmem, st, tq, tk1, a, w1);
+    cudaError_t e = set_smem_once<score_tc_kernel<D, 1, H1>>(C1::kSmem);
+    if (e != cudaSuccess) return e;
+    launch_chained(a.chain, score_tc_kernel<D, 1, H1>, groups1 * p1_row_parts(a.R, H1), cta_threads(1, H1, a.V != nullptr),
+                   C1::kSmem, st, tq, tk1, a, w1);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  // (alone, pass 2 follows a kernel of the caller's and starts only after it)
-  const bool chain2 = a.chain && (passes & kScoreRowstats);
-  if (passes & kScoreColsums) launch_chained(chain2, k2, groups2, cta_threads(2, H2, a.V != nullptr), C2::kSmem, st, tq, tk2, a, w2);
+  if (!(passes & kScoreColsums)) return cudaSuccess;
+  if (passes & kScoreRowstats) {
+    const cudaError_t e = set_smem_once<score_tc_kernel<D, 2, H2>>(C2::kSmem);
+    if (e != cudaSuccess) return e;
+    launch_chained(a.chain, score_tc_kernel<D, 2, H2>, groups2, cta_threads(2, H2, a.V != nullptr), C2::kSmem, st, tq, tk2,
+                   a, w2);
+  } else {  // (alone, it follows a kernel of the caller's and starts only after it)
+    const cudaError_t e = set_smem_once<score_tc_kernel<D, 2, H2, true>>(C2::kSmem);
+    if (e != cudaSuccess) return e;
+    launch_chained(false, score_tc_kernel<D, 2, H2, true>, kPlanSMs, cta_threads(2, H2, a.V != nullptr), C2::kSmem, st, tq,
+                   tk2, a, w2);
+  }
   return cudaGetLastError();
 }
 
@@ -812,21 +848,23 @@ size_t score_tc_partials(int B, int Hkv) { return (size_t)B * Hkv + kPlanSMs; }
 
 int score_tc_tiles1(int n) { return (n + SELKV_P1_KEYS - 1) / SELKV_P1_KEYS; }
 
+ScoreWalk plan_colsums(const CompressArgs& a, const SeqTable& tab) {
+  ScoreWalk w1{}, w2{};
+  P1Cut cut;
+  int groups1, groups2;
+  plan_passes(a, tab, w1, w2, cut, groups1, groups2);
+  return w2;
+}
+
 cudaError_t launch_score_tc(const CompressArgs& a, const SeqTable& tab, cudaStream_t st, int passes) {
-  // Pass 1 with two 128-row halves per CTA reads a tile's keys once for both, where two CTAs with a half
-  // each read them twice (from L2, or HBM where they drift apart: 8 x 32k 100 -> 90 us, 64 x 8k 215 ->
-  // 197); but a CTA's share is then twice as coarse.  From 8 tiles (16 accumulators) a CTA on, unless
-  // rounding to whole tiles makes it longer (16k: 8 accumulators against 7, 18.9 against 16.4 us).
-  long long total = 0;
-  for (int b = 0; b < a.B; ++b) total += (long long)score_tc_tiles1(tab.n[b]) * a.Hkv;
-  auto accs = [&](int halves) {  // accumulators of the longest share
-    const int groups = kPlanSMs / ((a.R + 128 * halves - 1) / (128 * halves));
-    return (total + groups - 1) / groups * halves;
-  };
-  const bool both = a.R > 128 && accs(2) >= 16 && accs(2) <= accs(1);
+  ScoreWalk w1{}, w2{};
+  P1Cut cut;
+  int groups1, groups2;
+  plan_passes(a, tab, w1, w2, cut, groups1, groups2);
   auto go = [&](auto d, auto h2) {
     constexpr int D = decltype(d)::value, H2 = decltype(h2)::value;
-    return both ? launch_tc_t<D, 2, H2>(a, tab, st, passes) : launch_tc_t<D, 1, H2>(a, tab, st, passes);
+    return cut.halves == 2 ? launch_tc_t<D, 2, H2>(a, w1, w2, groups1, groups2, st, passes)
+                           : launch_tc_t<D, 1, H2>(a, w1, w2, groups1, groups2, st, passes);
   };
   using std::integral_constant;
   if (a.R > 256) return a.D == 128 ? go(integral_constant<int, 128>{}, integral_constant<int, 2>{}) : go(integral_constant<int, 64>{}, integral_constant<int, 2>{});

@@ -136,12 +136,12 @@ struct SeqTable {
   int32_t t1[SELKV_MAX_BATCH];  // tensor-core scoring, pass 1: key tiles of the sequences before b (one KV head)
 };
 
+struct ScoreWalk;
 struct CompressArgs {
   bool chain;     // launch with launch_chained's early start
   int dtype, B, Hq, Hkv, G, D, W, n_cap, m_cap;
   int R;          // observation rows per KV head: G * W
   int nchunks;    // column chunks of the row-statistics pass
-  int p1_split, p1_per;  // tensor-core scoring: how pass 1 cut the tiles (splits per unit, or 0 and tiles per CTA)
   int row_chunk;  // columns of a chunk (CUDA-core scoring)
   float alpha;
   int pool_kernel, bucket, recent, gate_mode, empty_bucket;
@@ -171,6 +171,7 @@ struct CompressArgs {
   int32_t* seq_n;
   int32_t* seq_m;
   int32_t* seq_t1;   // [B] SeqTable::t1
+  ScoreWalk* p2_walk;  // scoring entry point, tensor cores: pass 2's shares for a call with that pass alone
   float2* rowpart;   // (max, sum) of 2^(s' - max): [B][Hkv][nchunks][R] per column chunk; tensor cores: [pieces][R]
   float2* rowstat;   // [B][Hkv][R] (M, 1 / (G * Z))
   float* attn;       // [B][Hkv][n_cap]
@@ -214,6 +215,7 @@ struct ScoreWalk {
   int32_t u0[kPlanSMs], t0[kPlanSMs], cnt[kPlanSMs];
   int32_t n[kPlanSMs];                      // length of the first unit's sequence
   int32_t part0[kPlanSMs], parts[kPlanSMs];  // pass 2: the first unit's partials of pass 1
+  int32_t p1_split, p1_per;  // pass 2: how pass 1 cut the tiles (splits per unit, or 0 and tiles per CTA)
 };
 
 // Selection unit of (b, kv): the sequence in the shared mode, the KV head in the per-head mode.
@@ -255,7 +257,8 @@ int score_tc_tiles1(int n);                // pass-1 key tiles of n keys
 constexpr int kScoreRowstats = 1, kScoreColsums = 2, kScoreAll = 3;
 cudaError_t launch_score_tc(const CompressArgs& a, const SeqTable& tab, cudaStream_t s, int passes = kScoreAll);
 cudaError_t launch_score_simt(const CompressArgs& a, cudaStream_t s, int passes = kScoreAll);
-cudaError_t launch_seq_setup(const CompressArgs& a, const SeqTable& tab, cudaStream_t s);
+ScoreWalk plan_colsums(const CompressArgs& a, const SeqTable& tab);  // tensor cores: pass 2's shares
+cudaError_t launch_seq_setup(const CompressArgs& a, const SeqTable& tab, const ScoreWalk& w, cudaStream_t s);
 cudaError_t launch_rowstat_reduce(const CompressArgs& a, cudaStream_t s);
 // Routing, merge and kept-row copy in one kernel (merge_mma.cu): bf16, buckets of 32, bucket routing.
 bool merge_uses_mma(int dtype, int D, int bucket, int routing);

@@ -49,3 +49,25 @@ def test_scores(d, lens, hq, hkv, W):
         torch.testing.assert_close(c.debug["attn"][b, :, :nb].double(), want, rtol=5e-5, atol=1e-12)
         want = c.debug["attn"][b, :, :nb].double() * V[b, :, :nb].double().norm(dim=2)
         torch.testing.assert_close(c.debug["score"][b, :, :nb].double(), want, rtol=9 * 2.0 ** -24, atol=0)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("lens,hq,hkv,W", [((9000, 257, 4100), 8, 4, 64), ((700, 5000) * 20, 16, 8, 40), ((2500, 8000, 64), 16, 2, 64)])
+def test_column_sums_alone_keep_the_lengths_of_the_row_statistics(lens, hq, hkv, W, dtype):
+    """A call with the second pass alone works on the lengths of the call before, whatever valid
+    lengths it is given itself."""
+    B, n, d = len(lens), max(lens), 64
+    g = torch.Generator(device="cuda").manual_seed(n)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    K = torch.randn((B, hkv, n, d), generator=g, device="cuda").to(dt)
+    Q = torch.randn((B, hq, W, d), generator=g, device="cuda").to(dt)
+    shape = api.make_shape(dtype, B, hq, hkv, d, W, n, 64)
+    ws = api.Workspace(S.selkv_score_workspace_size(shape))
+    want = torch.full((B, hkv, n), -1.0, device="cuda")
+    S.check(S.selkv_score(shape, lens, K, Q, want, S.SELKV_SCORE_ALL, ws.buf, ws.nbytes), "all")
+    for other in (lens, [W] * B, [n] * B, list(reversed(lens))):
+        got = torch.full_like(want, -1.0)
+        S.check(S.selkv_score(shape, lens, K, Q, None, S.SELKV_SCORE_ROWSTATS, ws.buf, ws.nbytes), "rowstats")
+        S.check(S.selkv_score(shape, other, K, Q, got, S.SELKV_SCORE_COLSUMS, ws.buf, ws.nbytes), "colsums")
+        assert torch.equal(got, want)
+    assert ws.errors() == 0

@@ -713,16 +713,20 @@ struct UCfg {
 };
 
 // Sequences by descending length, by one warp: a stable counting sort of the lengths in 64-row steps.
-// Every CTA finds the same order: the lengths advance only when all CTAs have come to their end.
+// Every CTA finds the same order: the lengths advance only when all CTAs have come to their end.  Both
+// roles of a CTA take a unit's length from here: the producer warp has no part in the arrivals, and for
+// units without rows the consumers do not wait for it, so it may still be at them when the lengths in
+// global memory advance.
 // (`ordered` false: before griddepcontrol.wait, from lengths that may still change.)
 constexpr int kLenKeys = 64;
-static_assert(SELKV_DEC_UNITS_MAX_ROWS <= 64 * (kLenKeys - 1), "a key per length step");
+static_assert(SELKV_DEC_UNITS_MAX_ROWS <= 64 * (kLenKeys - 1) && SELKV_DEC_UNITS_MAX_ROWS < 32767, "a key per length step");
 struct LenOrder {
   uint16_t seq[SELKV_MAX_BATCH];
+  int16_t len[SELKV_MAX_BATCH];  // by sequence; -1 and m_cap + 1 stand for lengths out of range
   uint8_t key[SELKV_MAX_BATCH];
   uint32_t start[kLenKeys];
 };
-__device__ __forceinline__ void order_by_length(const int* lengths, int B, bool ordered, LenOrder& o) {
+__device__ __forceinline__ void order_by_length(const int* lengths, int B, int m_cap, bool ordered, LenOrder& o) {
   const int lane = threadIdx.x & 31;
   const uint32_t below = (1u << lane) - 1u;
   o.start[lane] = o.start[lane + 32] = 0u;
@@ -731,7 +735,8 @@ __device__ __forceinline__ void order_by_length(const int* lengths, int B, bool 
     const int b = b0 + lane;
     int key = kLenKeys + lane;  // past the end: alone
     if (b < B) {
-      const int L = max(ordered ? lengths[b] : ld_relaxed_gpu(lengths + b), 0);
+      const int raw = ordered ? lengths[b] : ld_relaxed_gpu(lengths + b), L = max(raw, 0);
+      o.len[b] = (int16_t)min(max(raw, -1), m_cap + 1);
       key = kLenKeys - 1 - min(L / 64 + (L % 64 != 0), kLenKeys - 1);
       o.key[b] = (uint8_t)key;
     }
@@ -801,7 +806,7 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
     return i < units ? (int)s_ord.seq[i / a.Hkv] * a.Hkv + i % a.Hkv : units;
   };
 
-  if (warp == kConsumers) order_by_length(a.lengths, a.B, false, s_ord);
+  if (warp == kConsumers) order_by_length(a.lengths, a.B, a.m_cap, false, s_ord);
   if (warp == kConsumers && lane == 0) {
     for (int i = 0; i < kStages; ++i) {
       mbar_init(&full[i], 1);
@@ -845,7 +850,7 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
   pdl_launch_dependents();
   if (warp == kConsumers) {
     __syncwarp();
-    order_by_length(a.lengths, a.B, true, s_ord);
+    order_by_length(a.lengths, a.B, a.m_cap, true, s_ord);
   }
   __syncthreads();
   const bool has_new = a.k_new != nullptr;
@@ -858,7 +863,7 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
       int issued = 0;  // tiles handed to the consumers so far, over all of this CTA's units
       bool stop = false;
       for (int k = 0, u = unit_at(0); u < units && !stop; u = unit_at(++k)) {
-        const int L = min(max(a.lengths[u / a.Hkv], 0), a.m_cap);
+        const int L = min(max((int)s_ord.len[u / a.Hkv], 0), a.m_cap);
         const int nt = (L + kTile - 1) / kTile;
         const int row0 = (int)((size_t)u * a.m_cap);
         for (int i = 0; i < nt; ++i) {
@@ -916,7 +921,7 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
   for (int k = 0, u = unit_at(0); u < units; u = unit_at(++k)) {
     const int b = u / a.Hkv;
     const size_t bk = (size_t)u;
-    int L = a.lengths[b];
+    int L = s_ord.len[b];
     if (L < 0 || L > a.m_cap) {
       if (tid == 0 && u % a.Hkv == 0) raise_flag(a.flags, SELKV_DEVERR_LENGTH);
       L = L < 0 ? 0 : a.m_cap;
@@ -1209,14 +1214,15 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
     // after every consumer has passed this barrier
     named_bar_sync(kBar, kCons);
   }
-  // The last CTA to come to its end advances the lengths: every CTA has read them all by now.
+  // The last CTA to come to its end advances the lengths: every CTA has read them before its barrier
+  // above, none after it.
   if (has_new && warp == 0) {
     uint32_t old = 0u;
     if (lane == 0) old = atom_add_acq_rel_gpu(&a.cnt_seq[0], 1u);
     old = __shfl_sync(0xffffffffu, old, 0);
     if (old == (uint32_t)P - 1u) {
       for (int b = lane; b < a.B; b += 32) {
-        const int L = min(max(a.lengths[b], 0), a.m_cap);
+        const int L = min(max((int)s_ord.len[b], 0), a.m_cap);
         if (L + 1 <= a.m_cap) a.lengths[b] = L + 1;
       }
       if (lane == 0) a.cnt_seq[0] = 0u;

@@ -82,3 +82,30 @@ def test_the_output_does_not_depend_on_the_tile(hq, hkv, d):
         cache = api.CompressedCache(shape, *both[:4])
         outs.append(api.decode(cache, *both[4:]))
     assert torch.equal(outs[1][:B], outs[0]) and torch.equal(outs[1][B:], outs[0])
+
+
+@pytest.mark.parametrize("B,hkv,full", [(1000, 1, 0), (1000, 1, 3), (90, 8, 40), (20, 8, 0)])
+def test_many_empty_caches(B, hkv, full):
+    """All but `full` caches are empty, several for each CTA: no consumer waits for a tile of theirs.
+    Three tokens in a row, with nothing between them that waits for the device."""
+    d, cap = 64, 192
+    g = torch.Generator(device="cuda").manual_seed(B + full)
+    K, V = (torch.randn((B, hkv, cap, d), generator=g, device="cuda").bfloat16() for _ in range(2))
+    bias = torch.rand((B, hkv, cap), generator=g, device="cuda")
+    lengths = torch.zeros(((B + 3) // 4 * 4,), dtype=torch.int32, device="cuda")
+    lengths[:full] = cap - 3
+    shape = api.make_shape("bf16", B, 2 * hkv, hkv, d, 32, cap, cap)
+    cache = api.CompressedCache(shape, K, V, bias, lengths)
+    ws = api.Workspace(S.selkv_decode_workspace_size(shape))
+    q = torch.randn((3, B, 2 * hkv, d), generator=g, device="cuda").bfloat16()
+    kn, vn = (torch.randn((3, B, hkv, d), generator=g, device="cuda").bfloat16() for _ in range(2))
+    outs = [api.decode(cache, q[t], kn[t], vn[t], workspace=ws) for t in range(3)]
+    assert ws.errors() == 0
+    assert torch.equal(lengths[:B], (torch.arange(B, device="cuda") < full).int() * (cap - 3) + 3)
+    assert torch.equal(K[full:, :, :3], kn[:, full:].permute(1, 2, 0, 3)) and torch.equal(V[full:, :, :3], vn[:, full:].permute(1, 2, 0, 3))
+    # one row: its value; then a softmax over the rows so far, all with bias 0
+    assert torch.equal(outs[0][full:], vn[0, full:].repeat_interleave(2, 1))
+    for t in range(1, 3):
+        s = torch.einsum("bkgd,tbkd->bkgt", q[t, full:].view(-1, hkv, 2, d).double(), kn[:t + 1, full:].double()) / math.sqrt(d)
+        want = torch.einsum("bkgt,tbkd->bkgd", torch.softmax(s, 3), vn[:t + 1, full:].double()).reshape(-1, 2 * hkv, d)
+        assert float((outs[t][full:].double() - want).abs().max()) <= DEC_BF16_MAX

@@ -132,8 +132,9 @@ __global__ __launch_bounds__(warps_of(GM) * 32) void decode_simt_kernel(DecodeAr
 #pragma unroll
       for (int d = kLow; d < 32; d <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
       const float mn = fmaxf(m[g], mx);
-      const float corr = exp2f(m[g] - mn);
-      const float p = exp2f(x - mn);
+      const float mref = mn == -INFINITY ? 0.f : mn;  // (so far every key has weight 0)
+      const float corr = exp2f(m[g] - mref);
+      const float p = exp2f(x - mref);
       float ps = p;
 #pragma unroll
       for (int d = kLow; d < 32; d <<= 1) ps += __shfl_xor_sync(0xffffffffu, ps, d);

@@ -66,3 +66,27 @@ def test_decode(lens, d, hq, hkv, append):
         assert float((out[b].double() - want).abs().max()) <= 1e-5 * max(1.0, float(want.abs().max()))
         assert int(lengths[b]) == nb + append
     np.testing.assert_equal(lengths[B:].cpu().numpy(), 0)
+
+
+@pytest.mark.parametrize("append", [False, True])
+@pytest.mark.parametrize("d,hq,hkv", [(64, 4, 2), (128, 4, 2), (128, 16, 1)])
+@pytest.mark.parametrize("masked", [(0, 1), (0, 8), (0, 16), (0, 32), (0, 64), (0, 255), (64, 128), (3, 300)])
+def test_decode_of_rows_masked_by_the_bias(masked, d, hq, hkv, append):
+    """A bias of -inf takes a row out, also where it does so for all rows of a warp's step (8 at d 128, 16
+    at d 64), of a warp or of a split."""
+    cap, n, G = 384, 320, hq // hkv
+    g = torch.Generator(device="cuda").manual_seed(sum(masked) + d)
+    K, V = (torch.randn((1, hkv, cap, d), generator=g, device="cuda") for _ in range(2))
+    bias = torch.rand((1, hkv, cap), generator=g, device="cuda")
+    bias[:, :, masked[0]:masked[1]] = -math.inf
+    q = torch.randn((1, hq, d), generator=g, device="cuda")
+    kn, vn = (torch.randn((1, hkv, d), generator=g, device="cuda") for _ in range(2))
+    lengths = torch.tensor([n, 0, 0, 0], dtype=torch.int32, device="cuda")
+    cache = api.CompressedCache(api.make_shape("fp32", 1, hq, hkv, d, 32, cap, cap), K, V, bias, lengths)
+    out = api.decode(cache, q, kn if append else None, vn if append else None)
+    rows = n + append  # (an appended row is in the cache now, with bias 0)
+    s = torch.einsum("kgd,knd->kgn", q[0].view(hkv, G, d).double(), K[0, :, :rows].double()) / math.sqrt(d)
+    s = s + bias[0, :, None, :rows].double()
+    want = torch.einsum("kgn,knd->kgd", torch.softmax(s, 2), V[0, :, :rows].double()).reshape(hq, d)
+    # fp32 sums of a few hundred terms of order 1, as above
+    assert float((out[0].double() - want).abs().max()) <= 1e-5 * max(1.0, float(want.abs().max()))

@@ -445,7 +445,7 @@ __global__ __launch_bounds__(kThreads, SELKV_DEC_MINBLOCKS) void decode_tc_kerne
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           const int key = lo + t * kTile + warp * 16 + nt * 8 + c2 + e;
-          dst[nt][e] = (brow != nullptr && key < hi) ? __ldg(brow + key) * kLog2e : 0.f;
+          dst[nt][e] = (brow != nullptr && key < hi) ? brow[key] * kLog2e : 0.f;
         }
     };
     float bnext[2][2];
@@ -960,7 +960,7 @@ __global__ __launch_bounds__(UCfg<D, ROWS16, TILE>::kThreads, UCfg<D, ROWS16, TI
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           const int key = t * kTile + warp * 16 + n2 * 8 + c2 + e;
-          dst[n2][e] = (brow != nullptr && key < L) ? __ldg(brow + key) * kLog2e : 0.f;
+          dst[n2][e] = (brow != nullptr && key < L) ? brow[key] * kLog2e : 0.f;
         }
     };
     const bool two = kRuns > 1 && nt > 1;  // the warp goes through two states

@@ -215,7 +215,9 @@ __device__ __forceinline__ void pdl_launch_dependents() {
 // (which lets no kernel of the caller's start early): wait for the kernels before, then let the next
 // one be launched while this one runs.  Every thread of every CTA comes through here, so a kernel that
 // has got past it knows that all kernels but its predecessor have completed, and that the
-// predecessor has too.
+// predecessor has too.  What follows reads with ordinary loads: the read-only path (__ldg) is for data
+// that nothing writes while the kernel is resident, and a kernel is resident while its predecessor
+// still writes.
 __device__ __forceinline__ void chain_begin() {
   pdl_wait();
   pdl_launch_dependents();

@@ -236,11 +236,11 @@ __global__ __launch_bounds__(kThreads, 1) void cos_tc_kernel(const __grid_consta
     // 1 / ||v|| of this warp's 64 columns of a tile, fetched a tile ahead (cos_mpad is whole tiles)
     const float2* invn = reinterpret_cast<const float2*>(a.cos_invn + bk * a.cos_mpad + part * 64) + lane;
     float2* wown = reinterpret_cast<float2*>(winv + warp * 64);
-    if (nt > 0) wown[lane] = __ldg(invn);
+    if (nt > 0) wown[lane] = *invn;
     __syncwarp();
     for (int t = 0; t < nt; ++t) {
       float2 wnext = make_float2(0.f, 0.f);
-      if (t + 1 < nt) wnext = __ldg(invn + (size_t)(t + 1) * (kCols / 2));
+      if (t + 1 < nt) wnext = invn[(size_t)(t + 1) * (kCols / 2)];
 #pragma unroll
       for (int ph = 0; ph < 2; ++ph) {
         if (ph >= nph) break;

@@ -370,24 +370,30 @@ __global__ __launch_bounds__(NT) void topk_kernel(CompressArgs a, SelectWs w, in
 #pragma unroll
     for (int p = 0; p < kAhead; ++p) {
       const int j = s.base + g0 + p * 32 + lane;
-      own_a[p] = j < ncand ? __ldg(at + j) : 0.f;
-      own_v[p] = j < ncand ? __ldg(vn + j) : 0.f;
+      own_a[p] = j < ncand ? at[j] : 0.f;
+      own_v[p] = j < ncand ? vn[j] : 0.f;
     }
+    float pooled[kAhead];  // (all of them before the first store, which a later load might depend on)
 #pragma unroll
     for (int p = 0; p < kAhead; ++p) {
-      const int i0 = g0 + p * 32, i = i0 + lane, j = s.base + i;
-      if (i0 >= end) break;  // the rest belongs to the next warp
+      const int i0 = g0 + p * 32, j = s.base + i0 + lane;
       float v = 0.f;
       if (POOL && s.base + i0 >= half && s.base + i0 + 31 + half < ncand) {  // every tap of the warp's positions
         const float *pa = at + j, *pv = vn + j;
 #pragma unroll
         for (int t = -(POOL / 2); t <= POOL / 2; ++t)
-          v = t == 0 ? fmaf(own_a[p], own_v[p], v) : fmaf(__ldg(pa + t), __ldg(pv + t), v);
+          v = t == 0 ? fmaf(own_a[p], own_v[p], v) : fmaf(pa[t], pv[t], v);
       } else if (j < ncand) {
         for (int jj = max(0, j - half); jj <= min(ncand - 1, j + half); ++jj)
-          v = fmaf(__ldg(at + jj), __ldg(vn + jj), v);
+          v = fmaf(at[jj], vn[jj], v);
       }
-      v = v / (float)pool;
+      pooled[p] = v / (float)pool;
+    }
+#pragma unroll
+    for (int p = 0; p < kAhead; ++p) {
+      const int i0 = g0 + p * 32, i = i0 + lane, j = s.base + i;
+      if (i0 >= end) break;  // the rest belongs to the next warp
+      const float v = pooled[p];
       if (narrow && j < ncand) count_key(sh.hist, __float_as_uint(v));
       if (j < n) sc[j] = v;
       if (near_keys) s.keys[i] = __float_as_uint(v);
@@ -455,7 +461,7 @@ __global__ __launch_bounds__(NT) void trim_kernel(CompressArgs a, SelectWs w, in
       for (int p = 0; p < kAhead; ++p)
 #pragma unroll
         for (int h = 0; h < kHeads; ++h)
-          v[p][h] = h < nh && j0 + p * 32 < n ? __ldg(row + h * stride + p * 32) : 0.f;
+          v[p][h] = h < nh && j0 + p * 32 < n ? row[h * stride + p * 32] : 0.f;
 #pragma unroll
       for (int h = 0; h < kHeads; ++h) {
         if (h >= nh) break;

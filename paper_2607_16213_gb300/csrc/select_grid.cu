@@ -19,9 +19,11 @@
 // kernels and a memset, 75 us for one layer of 8 x 100k and 61 us at 8 x 16k; now 38 and 23 us.
 // What bounds it is latency: a CTA walks its positions with a few loads in flight a warp, then
 // three passes of barriers and remote reads.  Nothing waits outside the cluster.
+#include <algorithm>
 #include <climits>
 #include <type_traits>
 
+#include "cluster_fit.h"
 #include "ptx.cuh"
 #include "selkv_internal.cuh"
 
@@ -520,13 +522,44 @@ bool wide_ctas(int units, int n_cap) {
   return units * cs <= 100 && n_cap > 512 * cs;
 }
 
+// The largest cluster of the kernel's CTAs, with the most shared memory they take, that the device can
+// place, looked up once per kernel and device.  Sixteen CTAs need as many free SMs in one GPC, which a
+// partition of the GPU may not have; the selection is the same for every cluster size.
 template <auto Kern, int NT>
-cudaError_t launch_clusters(const CompressArgs& a, const SelectWs& w, int units, int cs, cudaStream_t s) {
-  const int span = ((a.n_cap + cs - 1) / cs + NT - 1) / NT * NT;
-  const int near_keys = span <= kMaxSpan ? 1 : 0;
+int largest_cluster() {
+  static std::atomic<int> found[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+  int cs = found[dev].load(std::memory_order_acquire);
+  if (cs > 0) return cs;
+  cs = fit_cluster(kMaxCluster, [](int size) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(size);
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = kMaxSpan * 4;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = size;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, Kern, &cfg) == cudaSuccess) return clusters > 0;
+    cudaGetLastError();  // (a refusal is an answer, not an error of the call)
+    return false;
+  });
+  found[dev].store(cs, std::memory_order_release);
+  return cs;
+}
+
+template <auto Kern, int NT>
+cudaError_t launch_clusters(const CompressArgs& a, const SelectWs& w, int units, int want, cudaStream_t s) {
   cudaError_t e = set_smem_once<Kern>(kMaxSpan * 4);
   if (e == cudaSuccess) e = allow_any_cluster_once<Kern>();
   if (e != cudaSuccess) return e;
+  const int cs = std::min(want, largest_cluster<Kern, NT>());
+  const int span = ((a.n_cap + cs - 1) / cs + NT - 1) / NT * NT;
+  const int near_keys = span <= kMaxSpan ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cs, units);
   cfg.blockDim = dim3(NT);

@@ -426,6 +426,7 @@ __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_
       uint32_t bad = __ballot_sync(kFull, !in || !(Ne < INFINITY));
       const uint32_t cons = __ballot_sync(kFull, con);
       const bool cleared = bad != 0u;
+      if (cleared) __syncwarp();  // other lanes' reads of these rows (the copy of the kept ones, the cosines) come first
       for (; bad; bad &= bad - 1u) {
         const int row = __ffs(bad) - 1;
         if ((cons >> row) & 1u) {

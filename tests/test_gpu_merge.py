@@ -1,6 +1,8 @@
 """The one-kernel merge of bf16 caches with 32-token buckets, against the oracle: lengths around the
 edges of a bucket and of a warp's walk, buckets without a kept token (tight budgets), both head
 sizes, and rows that are not finite."""
+import functools
+
 import numpy as np
 import pytest
 import torch
@@ -72,3 +74,10 @@ def test_a_kept_row_that_is_not_finite_stays_where_it_is(bad):
     others = np.arange(m) != slot
     np.testing.assert_array_equal(got[:, others], host["V_c"][0, :, :m][:, others])
     np.testing.assert_array_equal(got[:, slot], V2[0, :, pos].float().cpu().numpy())
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_the_same_with_the_gate_open(bad, monkeypatch):
+    """Without the cosines nothing comes between the copy of the row and its clearing in the tile."""
+    monkeypatch.setattr(O, "Params", functools.partial(O.Params, gate_mode=O.GATE_OPEN))
+    test_a_kept_row_that_is_not_finite_stays_where_it_is(bad)

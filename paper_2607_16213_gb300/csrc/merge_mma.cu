@@ -36,6 +36,11 @@ constexpr int kKeySlots = 64;    // key rows a copying warp moves
 #define SELKV_MERGE_SEG 8  // most buckets a warp walks
 #endif
 constexpr uint32_t kFull = 0xffffffffu;
+// The weights go to the product times 2^40, so that the lower pieces of the smallest ones are not lost
+// among bf16's subnormals (a weight of 2^-125 kept 9 of its 24 bits).  A power of two changes no other
+// result.  The weights of a target add up to at most W, and the elements of a row with a finite norm are
+// below 2^64, so nothing overflows for W up to 2^24.
+constexpr float kWeightUp = 0x1p40f, kWeightDown = 0x1p-40f;
 
 template <int D>
 struct MCfg {
@@ -412,8 +417,9 @@ __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_
         if (a.dbg_decision) a.dbg_decision[o] = g > 0.f ? 1 : 0;
       }
       // the weight in three bf16 pieces
-      const bf16 w0 = __float2bfloat16_rn(w);
-      const float r1 = w - __bfloat162float(w0);
+      const float ws = w * kWeightUp;
+      const bf16 w0 = __float2bfloat16_rn(ws);
+      const float r1 = ws - __bfloat162float(w0);
       const bf16 w1 = __float2bfloat16_rn(r1);
       const bf16 w2 = __float2bfloat16_rn(r1 - __bfloat162float(w1));
       bf16* wrow = reinterpret_cast<bf16*>(smem + C::kW) + lane;
@@ -468,8 +474,8 @@ __global__ __launch_bounds__(32, kCtasPerSm) void merge_mma_kernel(const __grid_
       s0 += __shfl_xor_sync(kFull, s0, 1);
       s1 += __shfl_xor_sync(kFull, s1, 1);
       if (c4 == 0) {
-        nums[m * 16 + g8] = s0;
-        nums[m * 16 + 8 + g8] = s1;
+        nums[m * 16 + g8] = s0 * kWeightDown;
+        nums[m * 16 + 8 + g8] = s1 * kWeightDown;
       }
     }
     den = warp_sum(den);

@@ -81,3 +81,43 @@ def test_the_same_with_the_gate_open(bad, monkeypatch):
     """Without the cosines nothing comes between the copy of the row and its clearing in the tile."""
     monkeypatch.setattr(O, "Params", functools.partial(O.Params, gate_mode=O.GATE_OPEN))
     test_a_kept_row_that_is_not_finite_stays_where_it_is(bad)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_the_smallest_weights_keep_their_bits(d):
+    """All tokens but one have an attention of 2^-120 to 2^-125, close to the smallest normal number: the
+    merged values are still the exact ones rounded to bf16."""
+    n, W, m_r = 2000, 1, 16
+    g = torch.Generator(device="cuda").manual_seed(d)
+    V = torch.randn((1, 1, n, d), generator=g, device="cuda").bfloat16()
+    V[..., 0] = 4.0  # cosines well above 0
+    K = torch.zeros((1, 1, n, d), device="cuda")
+    Q = torch.zeros((1, 1, W, d), device="cuda")
+    Q[..., 0] = 8.0
+    # one key takes all of the attention
+    K[..., 0] = -(120.0 + 4.5 * torch.rand((1, 1, n), generator=g, device="cuda")) * float(np.log(2.0)) * d ** 0.5 / 8.0
+    K[0, 0, n // 2, 0] = 0.0
+    K, Q = K.bfloat16(), Q.bfloat16()
+    shape = api.make_shape("bf16", 1, 1, 1, d, W, n, 576)
+    c = api.compress(shape, [n], 0.25, K, V, Q, S.selkv_params.defaults(recent=m_r), debug=True)
+    m = int(c.lengths[0])
+    a = c.debug["attn"][0, 0, :n].double().cpu().numpy()
+    small = a[:n - W]
+    assert np.median(small) < 2.0 ** -121 and (small > 0).mean() > 0.9
+    kept, target = (c.debug[k][0, 0].cpu().numpy() if c.debug[k].dim() == 3 else c.debug[k][0].cpu().numpy()
+                    for k in ("kept_idx", "target"))
+    kept, gate = kept[:m], c.debug["gate"][0, 0].double().cpu().numpy()
+    v = V[0, 0].double().cpu().numpy()
+    num, den = a[kept, None] * v[kept], a[kept].copy()
+    slot = {int(p): i for i, p in enumerate(kept)}
+    for j in range(n):
+        if target[j] >= 0:
+            num[slot[target[j]]] += gate[j] * a[j] * v[j]
+            den[slot[target[j]]] += gate[j] * a[j]
+    ok = den > 0
+    want = num[ok] / den[ok, None]
+    got = c.V_c[0, 0, :m].double().cpu().numpy()[ok]
+    # half a unit in the last place of bf16, and fp32 sums of tens of terms up to 4 (g a below 2^-126
+    # loses up to 2^-23 of itself as a subnormal number)
+    half_ulp = 2.0 ** (np.floor(np.log2(np.maximum(np.abs(want), 2.0 ** -100))) - 8)
+    assert (np.abs(got - want) - half_ulp).max() <= 1e-5

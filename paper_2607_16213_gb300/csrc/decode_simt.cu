@@ -207,7 +207,8 @@ cudaError_t launch_t(const DecodeArgs& a, cudaStream_t st) {
 // fill-and-fold cost worth kFillRows rows.  S minimises waves * (rows per CTA + kFillRows) over
 // the capacity m_cap, fewest splits on ties.  With `unit_walk` (the tensor-core decode), one
 // split over more units than slots with at most SELKV_DEC_UNITS_MAX_ROWS rows runs as
-// persistent CTAs that pay the fixed cost once: waves * rows + kFillRows.  There too, one split
+// persistent CTAs that pay the fixed cost once: waves * rows + kFillRows (the walk priced as the one CTA
+// per SM on 128-row tiles that it was; with 64-row tiles and two it is faster than that).  There too, one split
 // over at least BACKFILL_WAVES waves of units of at most BACKFILL_MAX_ROWS rows counts its waves as
 // units / slots: the block scheduler starts each unit as a slot frees, so ragged units pack
 // (batch 64 x 8k at 50%: 151.0 -> 144.0 us per launch, 64 x 32k at 10%: 129.6 -> 120.7; with

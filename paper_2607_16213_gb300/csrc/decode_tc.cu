@@ -676,7 +676,8 @@ __global__ __launch_bounds__(kThreads, SELKV_DEC_MINBLOCKS) void decode_tc_kerne
 // lengths (in 64-row steps), and CTA p takes unit p of that order, then 2P - 1 - p, 2P + p, ..., back
 // and forth, so that a long first unit is followed by a short one and the last, partial round has the
 // shortest.  In sequence order the longest share of a ragged batch carried the launch (64 sequences
-// of 409-819 rows, 8 KV heads: 50.3 us a launch against 45.8).  The producer streams the next unit's tiles while the consumer warps fold the
+// of 409-819 rows, 8 KV heads, 128-row tiles: 50.3 us a launch against 45.8).  The producer streams the
+// next unit's tiles while the consumer warps fold the
 // previous one (the ring runs on across units), so the start and drain of a CTA are paid once
 // per CTA instead of once per unit.  Each unit is held whole by one CTA: its fold is its output.
 // The group's queries (and the appended row) are staged in shared memory per unit, so the

@@ -16,7 +16,8 @@
 // finds the digit for itself from the others' counts, read through distributed shared memory
 // (first the sums of 16 slices of the bins, then the bins of one slice).  A grid-wide pass cost a
 // launch, a histogram in L2, an arrival and a last CTA working alone: the selection was eight such
-// kernels and a memset, 75 us for one layer of 8 x 100k and 61 us at 8 x 16k; now 38 and 23 us.
+// kernels and a memset, 75 us for one layer of 8 x 100k and 61 us at 8 x 16k; now 43 and 26 us (each
+// kernel alone, from a cold start).
 // What bounds it is latency: a CTA walks its positions with a few loads in flight a warp, then
 // three passes of barriers and remote reads.  Nothing waits outside the cluster.
 #include <algorithm>
